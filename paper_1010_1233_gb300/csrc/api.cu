@@ -35,11 +35,10 @@ int fft_rows_smem(int precision, int nx);
 int fft_cols_smem(int precision, int F, int ny, int ncol);
 cudaError_t set_fft_smem_limits();
 void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int grid, int block, int smem, cudaStream_t st, int slot,
-                     int paths, int sms);
+                     int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms);
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
-                     const TimeCorr& tc, int paths, int nslots, int max_fields);
+                     int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
+                     int nslots, int max_fields, int max_len, int max_pairs, int sms);
 void launch_time_corr(const ReplicaDesc* descs, int n_reps, int max_fields, const TimeCorr& tc, cudaStream_t st);
 void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                        int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
@@ -128,11 +127,12 @@ struct Layout {
   int64_t total = 0;
   int64_t n_vb_step = 0, n_vb_rows = 0, n_vb_cols = 0, n_vb_cols_a = 0;
   std::vector<int64_t> vb_step, vb_rows, vb_cols, vb_cols_a;
-  int vec = 1, q = 9, ncol = 0, rows_block = 32, rows_smem = 0, cols_smem = 0;
+  int vec = 1, q = 9, ncol = 0, rows_smem = 0, cols_smem = 0;
   int cols_a_paths = 0, cols_paths = 0;   // column-pass kernels the replicas need (cols16_b)
   int rows_paths = 0;                     // row-pass kernels (launch_fft_rows)
   int fold = 1;               // 2: two spectrum slots, two samples per accumulation pass
   int max_fields = 0;         // the most sampled fields of a replica with pair sums
+  int max_len = 1;            // the longest column transform
   int staged = 0;             // 1: the step kernel of lb_step_bulk.cu (tiles of 256 vec sites)
   bool any_fields = false;
 };
@@ -412,6 +412,7 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   }
   // column tile width of the sampling passes (it fixes the blocked layout of the pair sums)
   L.max_fields = maxF;
+  L.max_len = maxlen;
   if (maxF) {
     L.ncol = kColsMax;
     while (L.ncol > 1 && fft_cols_smem(precision, maxF, maxlen, L.ncol) > kColsSmemBudget) L.ncol >>= 1;
@@ -463,13 +464,9 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   L.vb_step.resize(n); L.vb_rows.resize(n); L.vb_cols.resize(n); L.vb_cols_a.resize(n);
   if (maxF) {
     // the shared-memory row kernel's launch (replicas the Stockham kernel does not take)
-    int gnx = 2;
     for (const ReplicaDesc& d : L.desc)
-      if (d.n_pairs && !rows16(precision, d.nx)) gnx = std::max(gnx, d.nx);
-    L.rows_smem = fft_rows_smem(precision, gnx);
-    L.rows_block = std::max(32, std::min(kRowsBlockMax, gnx / 2));
+      if (d.n_pairs && !rows16(precision, d.nx)) L.rows_smem = std::max(L.rows_smem, fft_rows_smem(precision, d.nx));
     L.cols_smem = fft_cols_smem(precision, maxF, maxlen, L.ncol);
-    if (L.fold == 2) L.cols_smem = std::max(L.cols_smem, fft_cols16_smem(maxF, maxlen, L.ncol, 2));
   }
   plan_step(lat, L.vec, 0, L);
   for (int r = 0; r < n; ++r) {
@@ -940,10 +937,9 @@ static void launch_step_any(flb_ctx* c, int vec, int staged, const StepLaunch& S
 static void flush_samples(flb_ctx* c, const StepLaunch& S, cudaStream_t st) {
   const Layout& L = c->L;
   if (!c->pending) return;
-  const int cols_grid = (int)std::min<int64_t>(L.n_vb_cols, (int64_t)c->sms * 8);
   launch_fft_cols(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_cols), c->n,
-                  L.n_vb_cols, c->ws, L.ncol, cols_grid, kColsBlock, L.cols_smem, st, c->tc, L.cols_paths,
-                  c->pending, L.max_fields);
+                  L.n_vb_cols, c->ws, L.ncol, st, c->tc, L.cols_paths, c->pending, L.max_fields, L.max_len,
+                  L.max_fields * (L.max_fields + 1) / 2, c->sms);
   count_kernels(c, path_launches(c->precision, L.cols_paths));
   c->pending = 0;
   if (c->tc.base) {
@@ -977,7 +973,7 @@ static void issue_step(flb_ctx* c, StepLaunch& S, bool sample, cudaStream_t st) 
     const int rows_grid = (int)std::min<int64_t>(L.n_vb_rows, (int64_t)c->sms * 8);
     const int cols_a_grid = (int)std::min<int64_t>(L.n_vb_cols_a, (int64_t)c->sms * 8);
     launch_fft_rows(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_rows), c->n,
-                    L.n_vb_rows, c->ws, rows_grid, L.rows_block, L.rows_smem, st, slot, L.rows_paths, c->sms);
+                    L.n_vb_rows, c->ws, rows_grid, L.rows_smem, st, slot, L.rows_paths, c->sms);
     if (L.n_vb_cols_a)
       launch_fft_cols_a(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_cols_a), c->n,
                         L.n_vb_cols_a, c->ws, L.ncol, cols_a_grid, kColsBlock, L.cols_smem, st,

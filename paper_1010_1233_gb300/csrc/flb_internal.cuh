@@ -200,8 +200,10 @@ template <int FL> struct Flavor { static constexpr bool kOne = FL != 2, kGen = F
 // length ny when F columns of 4 fit the budget, else ny = N1 * N2 with
 // N1 = 2^floor(log2(ny)/2) (four-step).
 constexpr int kColsSmemBudget = 200 * 1024;
-constexpr int kRowsBlockMax = 1024;      // threads of a row-FFT block (at most nx / 2)
+constexpr int kRowsBlock = 256;          // threads of a row-FFT block (shared-memory kernel)
 constexpr int kColsBlock = 256;
+// most threads of a block of the accumulation pass: 64 registers each in FP32, 128 in FP64
+__host__ __device__ constexpr int cols_block_max(int real_size) { return real_size == 4 ? 1024 : 512; }
 #ifndef FLB_COLS_MAX
 #define FLB_COLS_MAX 16
 #endif
@@ -221,8 +223,43 @@ __host__ __device__ __forceinline__ bool rows16_nx(int nx) {
   return nx >= 4096 && nx <= 32768 && (nx & (nx - 1)) == 0;
 }
 inline bool rows16(int precision, int nx) { return precision != FLB_FP64 && rows16_nx(nx); }
+// (the shared-memory pass: pairs of rows, 2048 points and at most 8 pairs per block, sequences
+// with 32 pad slots an odd number of elements apart)
+__host__ __device__ __forceinline__ int rows_per_block(int nx) { return nx >= 2048 ? 1 : (nx <= 256 ? 8 : 2048 / nx); }
+__host__ __device__ __forceinline__ int rows_seq_stride(int nx) { return nx + 33; }
 inline int64_t rows_blocks(int precision, int nx, int n_fields, int ny) {
-  return rows16(precision, nx) ? (int64_t)n_fields * ny : ((int64_t)n_fields * ny + 1) / 2;
+  if (rows16(precision, nx)) return (int64_t)n_fields * ny;
+  const int64_t pairs = ((int64_t)n_fields * ny + 1) / 2, p = rows_per_block(nx);
+  return (pairs + p - 1) / p;
+}
+// How a launch of the accumulation pass (pass 2b) cuts the layout's tiles of ncol columns:
+// blocks of w columns (w divides ncol) and ps groups of the field pairs.
+struct ColsSplit { int w, ps; };
+// A tile is a block's shared memory, so wide tiles mean few warps on an SM, and on lattices of
+// a few hundred columns few blocks at all.  Halve the tiles until there are 8 blocks per SM,
+// not below the columns that keep the sums' accesses in whole 32-byte sectors (4 FP64 sums; one
+// column in FP64, whose transforms bound the pass).  With fewer blocks than SMs even then, the
+// FP32 kernels also cut the pairs (each group transforms the tile again, which is cheap next
+// to its FP64 additions).  256^2, 9 fields, FP32: 17 blocks 173 us, 136 blocks 28 us;
+// FP64: 33 blocks 231 us, 129 blocks 69 us.
+inline ColsSplit cols_split(int precision, int64_t n_tiles, int ncol, int max_pairs, int sms) {
+  ColsSplit sp{ncol, 1};
+  const int wmin = precision == FLB_FP64 ? 1 : 4;
+  int64_t nb = n_tiles;
+  while (sp.w > wmin && nb < 8 * (int64_t)sms) { sp.w >>= 1; nb *= 2; }
+  if (precision != FLB_FP64 && nb < sms) {
+    const int most = (max_pairs + 2) / 3;                // at least three pairs in a group
+    sp.ps = (int)(sms / nb < most ? sms / nb : most);
+  }
+  return sp;
+}
+// threads of a block of the accumulation pass: about 1024 per SM, no more than the tile's points
+inline int cols_threads(int64_t nb, int sms, int points, int smem) {
+  const int64_t fit = 227 * 1024 / (smem + 1024), per_sm = (nb + sms - 1) / sms;
+  const int64_t bps = per_sm < fit ? per_sm : (fit < 1 ? 1 : fit);
+  int t = bps >= 4 ? 256 : (bps >= 2 ? 512 : 1024);
+  while (t > 256 && t > points) t >>= 1;
+  return t;
 }
 // The register-resident pass-2a kernel takes tiles of kColsA16 columns of one field
 // (pass 2a needs no field pairs); the shared-memory kernel tiles of the layout's ncol

@@ -18,92 +18,101 @@
 
 namespace flb {
 
-// Pass 1: one block per (replica, packed pair of row units).
+// Pass 1: one block per (replica, group of rows_per_block(nx) packed pairs of row units).
+//
+// Each pass of the transform is a few dozen instructions between two barriers, so what
+// bounds it is how many rows an SM works on at a time.  With one pair per block of nx / 2
+// threads only nx / 8 threads had work in the radix-8 and radix-16 passes, and a batched
+// launch sized its blocks for the longest row.  256 threads and up to 2048 points per block
+// keep every thread busy and 4 blocks on an SM (64 registers): 64 replicas of 64^2 .. 512^2
+// (3 fields) 153 -> 70 us, 3 x 1024 x 2048 42 -> 24 us.
 template <typename R>
-__global__ void __launch_bounds__(kRowsBlockMax)
+__global__ void __launch_bounds__(kRowsBlock, sizeof(R) == 4 ? 4 : 2)
 k_fft_rows(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin,
                            int n_reps, int64_t n_vblocks, char* __restrict__ ws, int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C<R>* z = reinterpret_cast<C<R>*>(smem_raw);
+  const int tid = (int)threadIdx.x, nt = (int)blockDim.x;
   for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
     const int r = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[r];
     if (sizeof(R) == 4 && rows16_nx(d.nx)) continue;   // k_fft_rows16's row
-    // block vb packs the row units u = 2 local and u + 1 (unit u: field u / ny, row u % ny;
-    // ny is a power of two), so an odd field count leaves at most one half-empty transform
-    const int64_t ua = 2 * (vb - vb_begin[r]), ub = ua + 1;
-    const bool has_b = ub < (int64_t)d.n_fields << d.log2ny;
-    const int fa = (int)(ua >> d.log2ny), ya = (int)(ua & (d.ny - 1));
-    const int fb = (int)(ub >> d.log2ny), yb = (int)(ub & (d.ny - 1));
-    const int nx = d.nx, logn = d.log2nx;
-    const int64_t plane = (int64_t)nx * d.ny;
-    const R* fields = reinterpret_cast<const R*>(ws + d.off_fields);
-    const R* xa = fields + fa * plane + (int64_t)ya * nx;
-    const R* xb = fields + fb * plane + (int64_t)yb * nx;
+    // pair p packs the row units u = 2 p and u + 1 (unit u: field u / ny, row u % ny; ny is a
+    // power of two), so an odd field count leaves at most one half-empty transform
+    const int nx = d.nx, logn = d.log2nx, hn = nx >> 1;
+    const int64_t units = (int64_t)d.n_fields << d.log2ny, pairs = (units + 1) >> 1;
+    const int P = rows_per_block(nx);
+    const int64_t p0 = (vb - vb_begin[r]) * P;
+    const int np = (int)min((int64_t)P, pairs - p0);           // this block's pairs, sequences of z
+    const int ss = rows_seq_stride(nx);
+    const R* fields = reinterpret_cast<const R*>(ws + d.off_fields) + 2 * p0 * nx;   // unit u starts at u nx
+    const int n_units = (int)min((int64_t)2 * np, units - 2 * p0);
     const int ps = logn > 5 ? logn - 5 : 31;        // 32 pad slots per row
     const C<R>* tw = reinterpret_cast<const C<R>*>(ws + d.off_tw_x);
-    // the rows of this block's next pair into L2 while this pair is transformed
-    if (threadIdx.x == 0 && vb + gridDim.x < n_vblocks) {
+    // the rows of this block's next group into L2 while this one is transformed
+    if (tid == 0 && vb + gridDim.x < n_vblocks) {
       const int64_t vbn = vb + gridDim.x;
       const int rn = find_rep(vb_begin, n_reps, vbn);
       const ReplicaDesc& dn = descs[rn];
-      const int64_t un = 2 * (vbn - vb_begin[rn]);
-      const R* fn = reinterpret_cast<const R*>(ws + dn.off_fields);
-      const uint32_t bytes = (uint32_t)(dn.nx * sizeof(R));
-      if (bytes % 16 == 0) {         // unit u starts at u nx (the fields are contiguous rows)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(fn + un * dn.nx), "r"(bytes) : "memory");
-        if (un + 1 < (int64_t)dn.n_fields << dn.log2ny)
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(fn + (un + 1) * dn.nx), "r"(bytes)
-                       : "memory");
-      }
+      const int64_t un = 2 * (vbn - vb_begin[rn]) * rows_per_block(dn.nx);
+      const int64_t left = ((int64_t)dn.n_fields << dn.log2ny) - un;
+      const R* fn = reinterpret_cast<const R*>(ws + dn.off_fields) + un * dn.nx;
+      const int64_t bytes = min((int64_t)2 * rows_per_block(dn.nx), left) * dn.nx * (int64_t)sizeof(R);
+      if (left > 0 && bytes % 16 == 0 && (reinterpret_cast<uintptr_t>(fn) & 15) == 0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(fn), "r"((uint32_t)bytes) : "memory");
     }
     if (logn >= 3) {
-      // thread x0 < nx/8 loads x0 + j nx/8 (j < 8, coalesced): after bit reversal these are
-      // elements t = brev3(j) of the group m = brev(x0) of the first three stages, which
-      // run in registers before the group is stored
+      // item (pair, x0), x0 < nx/8, loads x0 + j nx/8 (j < 8, coalesced): after bit reversal
+      // these are elements t = brev3(j) of the group m = brev(x0) of the first three stages,
+      // which run in registers before the group is stored
       const int n8 = nx >> 3;
-      for (int x0 = threadIdx.x; x0 < n8; x0 += blockDim.x) {
+      for (int it = tid; it < np * n8; it += nt) {
+        const int k = it >> (logn - 3), x0 = it & (n8 - 1);
+        const R* xa = fields + (int64_t)(2 * k) * nx;
+        const bool has_b = 2 * k + 1 < n_units;
         C<R> v[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
           const int x = x0 + (((t & 1) << 2) | (t & 2) | ((t >> 2) & 1)) * n8;
-          const bool in = FLB_INB(x >= 0 && x < nx, 131);
+          const bool in = FLB_INB(x >= 0 && x < nx && 2 * k < n_units, 131);
           v[t].x = in ? xa[x] : (R)0;
-          v[t].y = has_b && in ? xb[x] : (R)0;
+          v[t].y = has_b && in ? xa[nx + x] : (R)0;
         }
         dit_group<R, 3>(v, logn, 0, 0, tw, 1);
         const int i0 = brev(x0, logn - 3) << 3;
 #pragma unroll
         for (int t = 0; t < 8; ++t)
-          if (FLB_INB(i0 + t < nx, 132)) z[i0 + t + ((i0 + t) >> ps)] = v[t];
+          if (FLB_INB(i0 + t < nx, 132)) z[k * ss + i0 + t + ((i0 + t) >> ps)] = v[t];
       }
       __syncthreads();
-      dit_fft<R, sizeof(R) == 4 ? 4 : 3>(z, logn, 1, 0, tw, 1, ps, 3);   // FP32: four stages per pass
+      dit_fft<R, sizeof(R) == 4 ? 4 : 3>(z, logn, np, ss, tw, 1, ps, 3);   // FP32: four stages per pass
     } else {
-      for (int x = threadIdx.x; x < nx; x += blockDim.x) {
-        C<R> v; v.x = xa[x]; v.y = has_b ? xb[x] : (R)0;
+      for (int it = tid; it < np << logn; it += nt) {
+        const int k = it >> logn, x = it & (nx - 1);
+        const R* xa = fields + (int64_t)(2 * k) * nx;
+        C<R> v; v.x = xa[x]; v.y = 2 * k + 1 < n_units ? xa[nx + x] : (R)0;
         const int i = brev(x, logn);
-        if (FLB_INB(i < nx, 132)) z[i + (i >> ps)] = v;
+        if (FLB_INB(i < nx && 2 * k < n_units, 132)) z[k * ss + i + (i >> ps)] = v;
       }
       __syncthreads();
-      dit_fft<R>(z, logn, 1, 0, tw, 1, ps);
+      dit_fft<R>(z, logn, np, ss, tw, 1, ps);
     }
-    C<R>* spec = reinterpret_cast<C<R>*>(ws + d.off_spec + slot * d.spec_slot);
-    const int64_t fplane = (int64_t)d.ny * d.wpitch;
-    C<R>* ra = spec + fa * fplane + (int64_t)ya * d.wpitch;
-    C<R>* rb = spec + fb * fplane + (int64_t)yb * d.wpitch;
-    const int hn = nx >> 1;
-    const bool rows_ok = FLB_INB(fa < (int)d.n_fields && ya < d.ny && (!has_b || (fb < (int)d.n_fields && yb < d.ny)) &&
-                                 hn < d.wpitch, 133);
-    for (int k = threadIdx.x; k <= hn && rows_ok; k += blockDim.x) {
+    // row u's half spectrum starts at u wpitch (the rows of all fields are contiguous)
+    C<R>* spec = reinterpret_cast<C<R>*>(ws + d.off_spec + slot * d.spec_slot) + 2 * p0 * d.wpitch;
+    const bool rows_ok = FLB_INB(2 * p0 + n_units <= units && hn < d.wpitch, 133);
+    // items (pair, k < nx/2), then k = nx/2 of every pair
+    const int body = np << (logn - 1);
+    for (int it = tid; it < body + np && rows_ok; it += nt) {
+      const int q = it < body ? it >> (logn - 1) : it - body, k = it < body ? it & (hn - 1) : hn;
       const int km = (nx - k) & (nx - 1);
-      const C<R> Z = z[k + (k >> ps)];
-      const C<R> Zm = z[km + (km >> ps)];
+      const C<R> Z = z[q * ss + k + (k >> ps)];
+      const C<R> Zm = z[q * ss + km + (km >> ps)];
+      C<R>* ra = spec + (int64_t)(2 * q) * d.wpitch + k;
       C<R> A; A.x = (R)0.5 * (Z.x + Zm.x); A.y = (R)0.5 * (Z.y - Zm.y);
-      ra[k] = A;
-      if (has_b) {            // (Z - conj(Zm)) / (2i)
+      *ra = A;
+      if (2 * q + 1 < n_units) {            // (Z - conj(Zm)) / (2i)
         C<R> B; B.x = (R)0.5 * (Z.y + Zm.y); B.y = (R)0.5 * (Zm.x - Z.x);
-        rb[k] = B;
+        ra[d.wpitch] = B;
       }
     }
     __syncthreads();
@@ -190,45 +199,45 @@ k_fft_cols_a(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ 
   }
 }
 
-// Pass 2b: one block per (replica, k1, tile of ncol columns); all fields of the tile.
-// One-pass columns are the case N1 = 1.
+// Pass 2b: one block per (replica, k1, tile of w columns, group of pairs); all fields of the
+// tile.  One-pass columns are the case N1 = 1.  vb_begin counts the layout's tiles of ncol
+// columns, each cut as sp says (ColsSplit).
 template <typename R>
-__global__ void __launch_bounds__(kColsBlock, sizeof(R) == 4 ? 4 : 2)     // FP32: four blocks per SM
+__global__ void __launch_bounds__(cols_block_max(sizeof(R)), 1)
 k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin,
-                               int n_reps, int64_t n_vblocks, char* __restrict__ ws, int ncol, TimeCorr tc) {
+                               int n_reps, int64_t n_vblocks, char* __restrict__ ws, int ncol, ColsSplit sp,
+                               TimeCorr tc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C<R>* s = reinterpret_cast<C<R>*>(smem_raw);
-  for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
+  const int w = sp.w, lc = 31 - __clz(w), lsub = 31 - __clz(ncol) - lc;      // powers of two
+  const int n_sub = sp.ps << lsub;
+  for (int64_t v = blockIdx.x; v < n_vblocks * n_sub; v += gridDim.x) {
+    const int64_t vb = v / n_sub;
+    const int sub = (int)(v - vb * n_sub), pg = sub >> lsub;
     const int r = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[r];
     if (sizeof(R) == 4 && cols16_b(d.ny >> d.log2n1)) continue;     // a register-resident kernel's block
-    const int lc = 31 - __clz(ncol);                    // ncol is a power of two
-    const int tiles = (d.half_nx + ncol - 1) >> lc;
+    const int tiles = (d.half_nx + ncol - 1) >> (lc + lsub);
     const int64_t local = vb - vb_begin[r];
     const int k1 = (int)(local / tiles);
-    const int kx0 = (int)(local - (int64_t)k1 * tiles) << lc;
+    const int kx0 = ((int)(local - (int64_t)k1 * tiles) << (lc + lsub)) + ((sub & ((1 << lsub) - 1)) << lc);
+    if (kx0 >= d.half_nx) continue;                     // past the last column
     const int logn1 = d.log2n1, n1 = 1 << logn1, logn2 = d.log2ny - logn1, n2 = d.ny >> logn1;
     const int F = (int)d.n_fields;
-    const int ncl = min(ncol, d.half_nx - kx0);
+    const int ncl = min(w, d.half_nx - kx0);
     const C<R>* spec = reinterpret_cast<const C<R>*>(ws + d.off_spec);
     const int64_t fplane = (int64_t)d.ny * d.wpitch;
-    // blocked pair sums: this block's sums of every pair are one contiguous range, pulled
+    // blocked pair sums: the layout tile's sums of every pair are one contiguous range, pulled
     // into L2 by bulk prefetches while the columns are loaded and transformed
-    if (d.acc_ncol && threadIdx.x < d.n_pairs) {
-      const int pr = threadIdx.x;
-      const int64_t el = d.pair_a[pr] == d.pair_b[pr] ? 8 : 16;
-      const int64_t first = (int64_t)(k1 * tiles + (kx0 >> lc)) * n2 * ncol;
-      const char* base = ws + d.pair_off[pr] + first * el;
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(base), "r"((uint32_t)(n2 * ncol * el)) : "memory");
-    }
+    if (d.acc_ncol && sub == 0) prefetch_sums(d, ws, k1, kx0, ncol, tiles, n2);
     // smem layout: [field][column][n2]
-    const int total = F * n2 * ncol;
+    const int total = F * n2 * w;
     for (int i0 = threadIdx.x; i0 < total; i0 += 4 * blockDim.x) {   // four loads in flight
       C<R> v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int i = i0 + u * blockDim.x;
-        const int c = i & (ncol - 1), y2 = (i >> lc) & (n2 - 1), f = i >> (lc + logn2);
+        const int c = i & (w - 1), y2 = (i >> lc) & (n2 - 1), f = i >> (lc + logn2);
         v[u].x = (R)0; v[u].y = (R)0;
         if (i < total && c < ncl && FLB_INB(f < F && n2 * k1 + y2 < d.ny && kx0 + c < d.half_nx, 161))
           v[u] = spec[f * fplane + (int64_t)(n2 * k1 + y2) * d.wpitch + kx0 + c];
@@ -236,14 +245,15 @@ k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int i = i0 + u * blockDim.x;
-        const int c = i & (ncol - 1), y2 = (i >> lc) & (n2 - 1), f = i >> (lc + logn2);
-        if (i < total && FLB_INB(f < F && c < ncol && brev(y2, logn2) < n2, 162))
-          s[(f * ncol + c) * (n2 + 1) + brev(y2, logn2)] = v[u];
+        const int c = i & (w - 1), y2 = (i >> lc) & (n2 - 1), f = i >> (lc + logn2);
+        if (i < total && FLB_INB(f < F && c < w && brev(y2, logn2) < n2, 162))
+          s[(f * w + c) * (n2 + 1) + brev(y2, logn2)] = v[u];
       }
     }
     __syncthreads();
-    dit_fft<R>(s, logn2, F * ncol, n2 + 1, reinterpret_cast<const C<R>*>(ws + d.off_tw_y), n1);
-    accumulate_tile<R, 0>(d, ws, s, n2 + 1, r, k1, kx0, ncl, ncol, tiles, tc);
+    dit_fft<R>(s, logn2, F * w, n2 + 1, reinterpret_cast<const C<R>*>(ws + d.off_tw_y), n1);
+    accumulate_tile<R, 0>(d, ws, s, n2 + 1, k1, kx0, ncl, w, ncol, tiles, pg, sp.ps);
+    if (pg == 0) tile_tail<R, 0>(d, ws, s, n2 + 1, r, k1, kx0, ncl, w, tc, 1, 0);
     __syncthreads();
   }
 }
@@ -295,8 +305,8 @@ __global__ void k_twiddles(C<R>* tw, int n) {
 void launch_fft_cols_a16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
                          char* ws, int grid, cudaStream_t st, int slot);
 void launch_fft_cols_acc16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
-                           char* ws, int ncol, int grid, int max_fields, cudaStream_t st, const TimeCorr& tc,
-                           int nslots);
+                           char* ws, int ncol, const ColsSplit& sp, int sms, int max_fields, cudaStream_t st,
+                           const TimeCorr& tc, int nslots);
 cudaError_t set_fft16_smem_limits();
 void launch_fft_rows16(const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks, char* ws,
                        int grid, int nx, cudaStream_t st, int slot);
@@ -312,10 +322,10 @@ void launch_twiddles(int precision, void* tw, int n, cudaStream_t st) {
 }
 
 // shared memory of the row pass for rows of nx: k_fft_rows16 holds nx / 2 complex values
-// (one pad slot per 16), k_fft_rows nx plus 32 pad slots
+// (one pad slot per 16), k_fft_rows its group of rows
 int fft_rows_smem(int precision, int nx) {
   if (rows16(precision, nx)) return (nx / 2 + nx / 32) * 8;
-  return (nx + 32) * (precision == FLB_FP64 ? 16 : 8);
+  return rows_per_block(nx) * rows_seq_stride(nx) * (precision == FLB_FP64 ? 16 : 8);
 }
 // the columns of every field of a tile, plus a table of up to 256 roots of unity
 // (the register-resident passes of spectra_cols.cu)
@@ -344,8 +354,8 @@ cudaError_t set_fft_smem_limits() {
 // grid: blocks of the shared-memory kernel; the Stockham kernel takes at most two blocks
 // per SM of the sms SMs (its blocks loop over their rows)
 void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int grid, int block, int smem, cudaStream_t st, int slot,
-                     int paths, int sms) {
+                     int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms) {
+  const int block = kRowsBlock;
   if (precision == FLB_FP64) {
     k_fft_rows<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
     return;
@@ -374,17 +384,25 @@ void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* v
                       (int)std::min<int64_t>((int64_t)grid, 4 * (int64_t)sms), st, slot);
 }
 
+// max_fields, max_len: the most fields and the longest column transform of a replica (the
+// shared-memory kernel's launch holds them)
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
-                     const TimeCorr& tc, int paths, int nslots, int max_fields) {
-  if (precision == FLB_FP64) {
-    k_fft_cols_acc<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, tc);
-    return;
+                     int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
+                     int nslots, int max_fields, int max_len, int max_pairs, int sms) {
+  const ColsSplit sp = cols_split(precision, n_vblocks, ncol, max_pairs, sms);
+  if (precision == FLB_FP64 || (paths & kColsGeneric)) {    // one slot (the host folds samples only without it)
+    const int smem = fft_cols_smem(precision, max_fields, max_len, sp.w);
+    const int64_t nb = n_vblocks * (ncol / sp.w) * sp.ps;
+    const int grid = (int)std::min<int64_t>(nb, 8 * (int64_t)sms);
+    const int block = std::min(cols_threads(nb, sms, sp.w * max_len, smem), cols_block_max(precision == FLB_FP64 ? 8 : 4));
+    if (precision == FLB_FP64)
+      k_fft_cols_acc<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc);
+    else
+      k_fft_cols_acc<float><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc);
   }
-  if (paths & kColsGeneric)         // one slot (the host folds samples only without this kernel)
-    k_fft_cols_acc<float><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, tc);
-  launch_fft_cols_acc16(paths & (kColsGeneric - 1), descs, vb_begin, n_reps, n_vblocks, ws, ncol, grid, max_fields, st,
-                        tc, nslots);
+  if (precision != FLB_FP64)
+    launch_fft_cols_acc16(paths & (kColsGeneric - 1), descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, sms,
+                          max_fields, st, tc, nslots);
 }
 
 void launch_time_corr(const ReplicaDesc* descs, int n_reps, int max_fields, const TimeCorr& tc, cudaStream_t st) {

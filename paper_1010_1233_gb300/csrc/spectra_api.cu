@@ -15,11 +15,10 @@ int fft_rows_smem(int precision, int nx);
 int fft_cols_smem(int precision, int F, int ny, int ncol);
 cudaError_t set_fft_smem_limits();
 void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int grid, int block, int smem, cudaStream_t st, int slot,
-                     int paths, int sms);
+                     int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms);
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
-                     const TimeCorr& tc, int paths, int nslots, int max_fields);
+                     int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
+                     int nslots, int max_fields, int max_len, int max_pairs, int sms);
 void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                        int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
                        int paths, int slot, int sms);
@@ -57,7 +56,6 @@ int spectra_plan(int precision, int nx, int ny, int F, SpectraPlan& P) {
   P.ncol = kColsMax;
   while (P.ncol > 1 && fft_cols_smem(precision, F, len, P.ncol) > kColsSmemBudget) P.ncol >>= 1;
   P.rows_smem = fft_rows_smem(precision, nx);
-  P.rows_block = std::max(32, std::min(kRowsBlockMax, nx / 2));
   P.cols_smem = fft_cols_smem(precision, F, len, P.ncol);
   const int64_t tiles = (d.half_nx + P.ncol - 1) / P.ncol;
   P.n_vb_rows = rows_blocks(precision, nx, F, ny);
@@ -112,16 +110,16 @@ int spectra_launch(int precision, SpectraPlan& P, char* scratch, const void* fie
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int gr = (int)std::min<int64_t>(P.n_vb_rows, (int64_t)sms * 8);
-  launch_fft_rows(precision, ddesc, vb, 1, P.n_vb_rows, scratch, gr, P.rows_block, P.rows_smem, st, 0,
+  launch_fft_rows(precision, ddesc, vb, 1, P.n_vb_rows, scratch, gr, P.rows_smem, st, 0,
                   rows16(precision, d.nx) ? 1 << (d.log2nx - 12) : kColsGeneric, sms);
   if (P.n_vb_cols_a) {
     const int ga = (int)std::min<int64_t>(P.n_vb_cols_a, (int64_t)sms * 8);
     launch_fft_cols_a(precision, ddesc, vb + 1, 1, P.n_vb_cols_a, scratch, P.ncol, ga, kColsBlock, P.cols_smem, st,
                       cols16_b(1 << d.log2n1) ? cols16_b(1 << d.log2n1) : kColsGeneric, 0, sms);
   }
-  const int gc = (int)std::min<int64_t>(P.n_vb_cols, (int64_t)sms * 8);
-  launch_fft_cols(precision, ddesc, vb + 2, 1, P.n_vb_cols, scratch, P.ncol, gc, kColsBlock, P.cols_smem, st,
-                  TimeCorr{}, cols16_b(d.ny >> d.log2n1) ? cols16_b(d.ny >> d.log2n1) : kColsGeneric, 1, (int)d.n_fields);
+  launch_fft_cols(precision, ddesc, vb + 2, 1, P.n_vb_cols, scratch, P.ncol, st, TimeCorr{},
+                  cols16_b(d.ny >> d.log2n1) ? cols16_b(d.ny >> d.log2n1) : kColsGeneric, 1, (int)d.n_fields,
+                  std::max(1 << d.log2n1, d.ny >> d.log2n1), d.n_pairs, sms);
   e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(FLB_ECUDA, "spectra launch: %s", cudaGetErrorString(e));
   return FLB_OK;

@@ -26,8 +26,6 @@
 
 namespace flb {
 
-constexpr int kCols16Block = 256;
-
 template <int B> constexpr int log2_ct() { return B == 1 ? 0 : 1 + log2_ct<B / 2>(); }
 
 // W_L^m for m < L from the length-ny table tw (exp(-2 pi i m' / ny), m' < ny / 2):
@@ -124,13 +122,13 @@ __device__ __forceinline__ void a16_issue(const ReplicaDesc& d, const A16Unit& u
 // to the FP64 sums.  All threads call it; it ends with a barrier.
 template <int B>
 __device__ __forceinline__ void cols_acc16_tile(const ReplicaDesc& d, char* __restrict__ ws, float2* s, int rep,
-                                                int k1, int kx0, int ncl, int ncol, int tiles, const TimeCorr& tc,
-                                                int nslots) {
+                                                int k1, int kx0, int ncl, int w, int ncol, int tiles, int pg, int ps,
+                                                const TimeCorr& tc, int nslots) {
   constexpr int L = 16 * B, SS = L + 1, QN = 16 / B, LB = log2_ct<B>();
-  const int lc = 31 - __clz(ncol);
+  const int lc = 31 - __clz(w);
   const int n2 = d.ny >> d.log2n1, F = (int)d.n_fields;
   const int rs = spec_row_stride(d);
-  const int slot_elems = F * ncol * SS;                 // shared-memory rows of one sample
+  const int slot_elems = F * w * SS;                 // shared-memory rows of one sample
   float2* wl = s + nslots * slot_elems;
   fill_wl(wl, L, reinterpret_cast<const float2*>(ws + d.off_tw_y), d.ny);
   __syncthreads();
@@ -139,20 +137,20 @@ __device__ __forceinline__ void cols_acc16_tile(const ReplicaDesc& d, char* __re
   // stage 1: rows y = N2 k1 + r + B j
   for (int it = threadIdx.x; it < items; it += blockDim.x) {
     const int k = it >= per_slot, i = it - k * per_slot;
-    const int c = i & (ncol - 1), r = (i >> lc) & (B - 1), f = i >> (lc + LB);
+    const int c = i & (w - 1), r = (i >> lc) & (B - 1), f = i >> (lc + LB);
     const float2* spec = reinterpret_cast<const float2*>(ws + d.off_spec + k * d.spec_slot);
     const bool in = c < ncl && FLB_INB(f < F && n2 * k1 + r + B * 15 < d.ny && kx0 + c < d.half_nx, 211);
-    if (!FLB_INB((f * ncol + c + 1) * SS <= slot_elems, 212)) continue;
+    if (!FLB_INB((f * w + c + 1) * SS <= slot_elems, 212)) continue;
     stage1<B>(spec + spec_index(d, f, n2 * k1 + r, kx0) + c, (int64_t)B * rs, in,
-              s + k * slot_elems + (f * ncol + c) * SS + r, wl, r);
+              s + k * slot_elems + (f * w + c) * SS + r, wl, r);
   }
   __syncthreads();
   // stage 2 in place
   for (int it = threadIdx.x; it < items; it += blockDim.x) {
     const int k = it >= per_slot, i = it - k * per_slot;
-    const int c = i & (ncol - 1), t = (i >> lc) & (B - 1), f = i >> (lc + LB);
-    if (!FLB_INB((f * ncol + c + 1) * SS <= slot_elems, 212)) continue;
-    float2* e = s + k * slot_elems + (f * ncol + c) * SS;
+    const int c = i & (w - 1), t = (i >> lc) & (B - 1), f = i >> (lc + LB);
+    if (!FLB_INB((f * w + c + 1) * SS <= slot_elems, 212)) continue;
+    float2* e = s + k * slot_elems + (f * w + c) * SS;
 #pragma unroll
     for (int qi = 0; qi < QN; ++qi) {
       const int q = t * QN + qi;
@@ -165,8 +163,8 @@ __device__ __forceinline__ void cols_acc16_tile(const ReplicaDesc& d, char* __re
     }
   }
   __syncthreads();
-  accumulate_points<B>(d, ws, s, SS, k1, kx0, ncl, ncol, tiles, nslots, slot_elems);
-  tile_tail<float, B>(d, ws, s, SS, rep, k1, kx0, ncl, ncol, tc, nslots, slot_elems);
+  accumulate_points<B>(d, ws, s, SS, k1, kx0, ncl, w, ncol, tiles, pg, ps, nslots, slot_elems);
+  if (pg == 0) tile_tail<float, B>(d, ws, s, SS, rep, k1, kx0, ncl, w, tc, nslots, slot_elems);
   __syncthreads();
 }
 
@@ -275,20 +273,22 @@ k_fft_cols_a16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// Pass 2b (N2 = L): one block per (replica, k1, tile of ncol columns), all fields and
-// the nslots samples of the tile; four blocks per SM (measured against three, with 80
-// registers and no spills: 10.08 against 10.50 ms per 16384^2 sample).
-#ifndef FLB_ACC16_MIN_BLOCKS
-#define FLB_ACC16_MIN_BLOCKS 4
-#endif
+// Pass 2b (N2 = L): one block per (replica, k1, tile of w columns, group of pairs), all
+// fields and the nslots samples of the tile; 64 registers a thread, four blocks of 256 threads
+// per SM on large lattices (measured against three, with 80 registers and no spills: 10.08
+// against 10.50 ms per 16384^2 sample), fewer and larger ones where there are few tiles.
+// vb_begin counts the layout's tiles of ncol columns, each cut as sp says (ColsSplit).
 template <int B>
-__global__ void __launch_bounds__(kCols16Block, FLB_ACC16_MIN_BLOCKS)
+__global__ void __launch_bounds__(cols_block_max(4), 1)
 k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
-                 int64_t n_vblocks, char* __restrict__ ws, int ncol, TimeCorr tc, int nslots) {
+                 int64_t n_vblocks, char* __restrict__ ws, int ncol, ColsSplit sp, TimeCorr tc, int nslots) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* s = reinterpret_cast<float2*>(smem_raw);
-  const int lc = 31 - __clz(ncol);
-  for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
+  const int lw = 31 - __clz(sp.w), lc = 31 - __clz(ncol), lsub = lc - lw;
+  const int n_sub = sp.ps << lsub;
+  for (int64_t v = blockIdx.x; v < n_vblocks * n_sub; v += gridDim.x) {
+    const int64_t vb = v / n_sub;
+    const int sub = (int)(v - vb * n_sub);
     const int rp = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[rp];
     const int n2 = d.ny >> d.log2n1;
@@ -296,17 +296,13 @@ k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restric
     const int tiles = (d.half_nx + ncol - 1) >> lc;
     const int64_t local = vb - vb_begin[rp];
     const int k1 = (int)(local / tiles);
-    const int kx0 = (int)(local - (int64_t)k1 * tiles) << lc;
-    // blocked pair sums: this block's sums of every pair are one contiguous range, pulled
+    const int kx0 = ((int)(local - (int64_t)k1 * tiles) << lc) + ((sub & ((1 << lsub) - 1)) << lw);
+    if (kx0 >= d.half_nx) continue;                     // past the last column
+    // blocked pair sums: the layout tile's sums of every pair are one contiguous range, pulled
     // into L2 by bulk prefetches while the columns are loaded and transformed
-    if (d.acc_ncol && threadIdx.x < d.n_pairs) {
-      const int pr = threadIdx.x;
-      const int64_t el = d.pair_a[pr] == d.pair_b[pr] ? 8 : 16;
-      const int64_t first = (int64_t)(k1 * tiles + (kx0 >> lc)) * n2 * ncol;
-      const char* base = ws + d.pair_off[pr] + first * el;
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(base), "r"((uint32_t)(n2 * ncol * el)) : "memory");
-    }
-    cols_acc16_tile<B>(d, ws, s, rp, k1, kx0, min(ncol, d.half_nx - kx0), ncol, tiles, tc, nslots);
+    if (d.acc_ncol && sub == 0) prefetch_sums(d, ws, k1, kx0, ncol, tiles, n2);
+    cols_acc16_tile<B>(d, ws, s, rp, k1, kx0, min(sp.w, d.half_nx - kx0), sp.w, ncol, tiles, sub >> lsub, sp.ps, tc,
+                       nslots);
   }
 }
 
@@ -345,12 +341,16 @@ void launch_fft_cols_a16(int mask, const ReplicaDesc* descs, const int64_t* vb_b
 // nslots = 2: the tiles of the samples in spectrum slots 0 and 1 in one pass; each launch
 // with the shared memory of its column length (max_fields: the most fields of a replica)
 void launch_fft_cols_acc16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
-                           char* ws, int ncol, int grid, int max_fields, cudaStream_t st, const TimeCorr& tc,
-                           int nslots) {
+                           char* ws, int ncol, const ColsSplit& sp, int sms, int max_fields, cudaStream_t st,
+                           const TimeCorr& tc, int nslots) {
+  const int64_t nb = n_vblocks * (ncol / sp.w) * sp.ps;
+  const int grid = (int)std::min<int64_t>(nb, 8 * (int64_t)sms);
 #define FLB_L(B)                                                                                            \
-  if (mask & B)                                                                                             \
-    k_fft_cols_acc16<B><<<grid, kCols16Block, fft_cols16_smem(max_fields, 16 * B, ncol, nslots), st>>>(     \
-        descs, vb_begin, n_reps, n_vblocks, ws, ncol, tc, nslots);
+  if (mask & B) {                                                                                           \
+    const int smem = fft_cols16_smem(max_fields, 16 * B, sp.w, nslots);                                     \
+    k_fft_cols_acc16<B><<<grid, cols_threads(nb, sms, sp.w * 16 * B, smem), smem, st>>>(                    \
+        descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc, nslots);                                      \
+  }
   FLB_L(1) FLB_L(2) FLB_L(4) FLB_L(8) FLB_L(16)
 #undef FLB_L
 }
