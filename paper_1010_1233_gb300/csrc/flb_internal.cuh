@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 
 #include "../../include/flb.h"
+#include "normals64.cuh"
 
 namespace flb {
 
@@ -128,14 +129,9 @@ __device__ __forceinline__ float sin_approx(float x) { float y; asm("sin.approx.
 __device__ __forceinline__ float cos_approx(float x) { float y; asm("cos.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
 // Box-Muller on a word pair: N0 = r cos(2 pi ub), N1 = r sin(2 pi ub), r = sqrt(-2 ln ua).
-// FP64: u = (w + 1/2) 2^-32 (exact).
+// FP64: u = (w + 1/2) 2^-32 (exact), evaluated in fixed point (normals64.cuh).
 __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, double& n0, double& n1) {
-  const double ua = ((double)wa + 0.5) * 0x1p-32;
-  const double ub = ((double)wb + 0.5) * 0x1p-32;
-  const double r = sqrt(-2.0 * log(ua));
-  double s, c;
-  sincospi(2.0 * ub, &s, &c);
-  n0 = r * c; n1 = r * s;
+  fx_box_muller(wa, wb, n0, n1);
 }
 
 // FP32: ua = RN(wa) 2^-32 + 2^-33 (relative error <= 2^-24 for every ua, small ua

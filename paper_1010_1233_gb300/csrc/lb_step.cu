@@ -55,10 +55,9 @@ k_step_d2q9(const ReplicaDesc* __restrict__ descs, const __grid_constant__ Repli
       R sum, ux, uy;
       macro_d2q9<R, DEV>(g, rho0, sum, ux, uy);
       R n[6] = {(R)0, (R)0, (R)0, (R)0, (R)0, (R)0};
-      const R one[6] = {(R)1, (R)1, (R)1, (R)1, (R)1, (R)1};
       if (noisy) normals_d2q9<R>(d, (uint32_t)u.y * (uint32_t)d.nx + (uint32_t)(u.x0 + s), step, n);
       R fl[kMaxFields];
-      collide_d2q9<R, DEV, SAMPLE, Flavor<FL>::kGen>(d, g, sum, ux, uy, noisy, n, one, fl);
+      collide_d2q9<R, DEV, SAMPLE, Flavor<FL>::kGen>(d, g, sum, ux, uy, noisy, n, fl);
 #pragma unroll
       for (int i = 0; i < 9; ++i) f[i][s] = g[i];
       if constexpr (SAMPLE) {

@@ -243,7 +243,9 @@ k_step_d2q9_bulk(const ReplicaDesc* __restrict__ descs, const __grid_constant__ 
 #pragma unroll
       for (int i = 0; i < 9; ++i) g[i] = f[i][v];
       R fl[kMaxFields];
-      collide_d2q9<R, true, SAMPLE, Flavor<FL>::kGen>(d, g, sum[v], ux[v], uy[v], noisy, nrm[v], sc[v], fl);
+      R D[6];
+      collide_relax<R, true, SAMPLE>(d, g, sum[v], ux[v], uy[v], D, fl);
+      collide_apply<R, true, Flavor<FL>::kGen>(d, g, sum[v], noisy, nrm[v], sc[v], D);
 #pragma unroll
       for (int i = 0; i < 9; ++i) out[i * G::HALF + 128 * v + tw] = g[i];
       if constexpr (SAMPLE) {

@@ -360,8 +360,10 @@ __device__ __forceinline__ void relax_site(const ReplicaDesc& d, const T (&g)[9]
 }
 
 // GEN: the replica may use noise modes 1 and 2 (branch on d.noise_mode); without it only
-// mode 0 is compiled (the common case keeps its registers and instruction count).
-template <typename T, bool DEV, bool GEN>
+// mode 0 is compiled (the common case keeps its registers and instruction count).  SCALED:
+// without the network s = 1 and sc is not read (the same values: 1 x = x exactly; it saves the
+// FP64 kernels six multiplications a site).
+template <typename T, bool DEV, bool GEN, bool SCALED = true>
 __device__ __forceinline__ void apply_site(const ReplicaDesc& d, T (&g)[9], T sum, bool noisy, const T (&n)[6],
                                            const T (&sc)[6], const T (&Drel)[6]) {
   using A = Lane<T>;
@@ -374,7 +376,7 @@ __device__ __forceinline__ void apply_site(const ReplicaDesc& d, T (&g)[9], T su
       T z = A::mul(A::splat(coef<S>(d, kCoNoiseR + 6 * c)), n[0]);
 #pragma unroll
       for (int e = 1; e < 6; ++e) z = A::fma(A::splat(coef<S>(d, kCoNoiseR + 6 * c + e)), n[e], z);
-      D[c] = A::fma(sc[c], z, D[c]);
+      D[c] = A::fma(SCALED ? sc[c] : A::splat((S)1), z, D[c]);
     }
   } else if (noisy) {                            // Eq. 8, scaled per moment by s
     T fac = A::splat((S)1);
@@ -384,7 +386,8 @@ __device__ __forceinline__ void apply_site(const ReplicaDesc& d, T (&g)[9], T su
     }
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      T s = A::mul(sc[c], A::splat(coef<S>(d, kCoAmp + 3 + c)));
+      T s = A::splat(coef<S>(d, kCoAmp + 3 + c));
+      if constexpr (SCALED) s = A::mul(sc[c], s);
       if (GEN && d.noise_mode == 2) s = A::mul(s, fac);
       D[c] = A::fma(s, n[c], D[c]);
     }
@@ -414,18 +417,20 @@ __device__ __forceinline__ void collide_relax(const ReplicaDesc& d, const R (&g)
   relax_site<R, DEV, SAMPLE>(d, g, sum, ux, uy, D, fld);
 }
 
-template <typename R, bool DEV, bool GEN>
+template <typename R, bool DEV, bool GEN, bool SCALED = true>
 __device__ __forceinline__ void collide_apply(const ReplicaDesc& d, R (&g)[9], R sum, bool noisy, const R (&n)[6],
                                               const R (&sc)[6], const R (&Drel)[6]) {
-  apply_site<R, DEV, GEN>(d, g, sum, noisy, n, sc, Drel);
+  apply_site<R, DEV, GEN, SCALED>(d, g, sum, noisy, n, sc, Drel);
 }
 
+// without the network
 template <typename R, bool DEV, bool SAMPLE, bool GEN>
 __device__ __forceinline__ void collide_d2q9(const ReplicaDesc& d, R (&g)[9], R sum, R ux, R uy, bool noisy,
-                                             const R (&n)[6], const R (&sc)[6], R (&fld)[kMaxFields]) {
+                                             const R (&n)[6], R (&fld)[kMaxFields]) {
   R D[6];
   collide_relax<R, DEV, SAMPLE>(d, g, sum, ux, uy, D, fld);
-  collide_apply<R, DEV, GEN>(d, g, sum, noisy, n, sc, D);
+  const R one[6] = {(R)1, (R)1, (R)1, (R)1, (R)1, (R)1};
+  collide_apply<R, DEV, GEN, sizeof(R) == 4>(d, g, sum, noisy, n, one, D);
 }
 
 // Store the post-collision populations (and the sampled fields) of a thread's sites.
