@@ -230,7 +230,8 @@ int flb_get_time_correlator(flb_ctx* ctx, int replica, int field_a, int field_b,
 
 /* Launch configuration of the step kernel.  staged = 0: direct kernels, vec
  * consecutive sites per thread (1, 2 or 4; > 1 only on the FP32 D2Q9 path,
- * every nx a multiple of vec), grid_blocks persistent blocks (0 = 16 per SM).
+ * every nx a multiple of vec), grid_blocks persistent blocks (0 = 16 per SM, or one
+ * per SM with the network on the warp engine).
  * staged = 1 (FP32 D2Q9 path, every nx a multiple of 4): row tiles of 256 vec
  * sites staged through shared memory by TMA bulk copies, one persistent block
  * per resident slot (grid_blocks caps it).  Results agree to rounding across
@@ -267,7 +268,7 @@ int flb_stability(const flb_replica* rep, int max_k, double* radius_out, int32_t
 
 /* Autotuner: times `trials` launches of the step kernel (current network
  * setting, no sampling) for every valid configuration: direct kernels with
- * every vec and grid size in {2,4,8,16} x SMs and all-blocks (with the network
+ * every vec and grid size in {2,4,8,16} x SMs ({1,2,4,8} for the warp engine) and all-blocks (with the network
  * on: with each network engine), and the staged kernel with every vec; keeps
  * the fastest, engine included, and reports it (ms_out: time per launch).  The timing launches recompute the next step from the current state
  * without advancing it, so the simulation is unchanged.  Synchronises. */

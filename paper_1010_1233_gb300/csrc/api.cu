@@ -119,6 +119,7 @@ static inline int first_nonconserved(int lat) { return is3d(lat) ? 4 : (lat == F
 static constexpr int kMaxPointItems = 2048;    // 3D direct transforms: fields x wave vectors
 
 static constexpr int kStepBlock = 256;
+static constexpr int64_t kVec4Sites = 1 << 20;
 
 struct Layout {
   std::vector<ReplicaDesc> desc;
@@ -391,8 +392,12 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   L.vec = 1;
   if (precision == FLB_FP32_DEV && lat == FLB_D2Q9) {
     bool all4 = true;
-    for (int r = 0; r < n; ++r) all4 = all4 && reps[r].nx % 4 == 0;
-    L.vec = all4 ? 4 : 2;
+    int64_t sites = 0;
+    for (int r = 0; r < n; ++r) { all4 = all4 && reps[r].nx % 4 == 0; sites += (int64_t)reps[r].nx * reps[r].ny; }
+    // four sites per thread where the lattice fills the GPU; below, two, for twice the threads
+    // and half of each thread's chain (us per step, vec 2 / 4: 64^2 2.1 / 2.8, 256^2 2.6 / 3.2,
+    // 512^2 4.8 / 5.2, 2048^2 51.1 / 49.2; with the network 256^2 4.3 / 5.8)
+    L.vec = all4 && sites >= kVec4Sites ? 4 : 2;
   } else if (precision == FLB_FP32_DEV && is3d(lat)) {
     bool all4 = lat == FLB_D3Q15;                // nx is even; D3Q19 at vec 4 spills registers
     for (int r = 0; r < n; ++r) all4 = all4 && reps[r].nx % 4 == 0;
@@ -985,6 +990,16 @@ static void issue_step(flb_ctx* c, StepLaunch& S, bool sample, cudaStream_t st) 
   }
 }
 
+// Blocks of the step launch: the caller's or the autotuner's choice, by default 16 per SM.  The
+// warp-engine network kernel keeps its weights in registers and is resident once per SM (two
+// half blocks at vec 1 and 2), so it defaults to one persistent block per SM (4096^2: 295 us
+// per step against 346 with 16; 512^2 at vec 2: 8.1 against 12.4).
+static int step_grid_blocks(const flb_ctx* c) {
+  const bool net = c->mlp_on && !c->L.staged && c->net_engine == FLB_NET_WARP;
+  const int64_t g = c->step_grid > 0 ? (int64_t)c->step_grid : (int64_t)c->sms * (net ? 1 : 16);
+  return (int)std::min<int64_t>(c->L.n_vb_step, g);
+}
+
 static StepLaunch step_launch(flb_ctx* c) {
   const Layout& L = c->L;
   StepLaunch S;
@@ -995,7 +1010,7 @@ static StepLaunch step_launch(flb_ctx* c) {
   S.ws = c->ws;
   S.mlp = c->ws + L.off_mlp;
   S.block = kStepBlock;
-  S.grid = (int)std::min<int64_t>(L.n_vb_step, c->step_grid > 0 ? (int64_t)c->step_grid : (int64_t)c->sms * 16);
+  S.grid = step_grid_blocks(c);
   S.parity = 0;
   S.step = 0;
   S.status = status_dev(c);
@@ -1489,7 +1504,7 @@ int flb_get_step_config(flb_ctx* c, int* vec, int* grid_blocks, int* staged) {
   if (!c || !vec || !grid_blocks || !staged) return set_error(FLB_EINVAL, "NULL argument");
   *vec = c->L.vec;
   *staged = c->L.staged;
-  *grid_blocks = (int)std::min<int64_t>(c->L.n_vb_step, c->step_grid > 0 ? (int64_t)c->step_grid : (int64_t)c->sms * 16);
+  *grid_blocks = step_grid_blocks(c);
   return FLB_OK;
 }
 
@@ -1558,8 +1573,10 @@ int flb_autotune(flb_ctx* c, int trials, int* vec_out, int* grid_out, int* stage
       ok = ok && c->L.desc[r].nx % vec == 0 && (vec > 1 || volume(c->L.desc[r]) < (int64_t(1) << 31));
     if (!ok) continue;
     // the staged kernel is persistent (its launcher caps the grid at the resident blocks)
-    const int mults[5] = {2, 4, 8, 16, 0};
-    for (int mi = staged ? 4 : 0; mi < 5 && !rc; ++mi) {
+    const int mults[6] = {1, 2, 4, 8, 16, 0};
+    const bool wn = two_engines && engine == FLB_NET_WARP;      // resident once per SM: 1 x SMs in place of 16 x
+    for (int mi = staged ? 5 : (wn ? 0 : 1); mi < 6 && !rc; ++mi) {
+      if (wn && mults[mi] == 16) continue;
       const int grid = mults[mi] ? mults[mi] * c->sms : 0;
       rc = flb_set_step_config(c, vec, grid ? grid : INT32_MAX, staged);
       if (rc) break;

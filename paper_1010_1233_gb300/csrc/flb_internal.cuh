@@ -30,20 +30,37 @@ constexpr int kNumCoef = kCoNoiseR + 36;
 
 // Per-replica description, resident in device memory (one array per context).
 // Offsets are byte offsets from the workspace base.
-struct ReplicaDesc {
-  int32_t nx, ny, log2nx, log2ny;
-  int32_t nz;                   // 3D depth (1 otherwise); a row is (y, z), row = z ny + y
-  int32_t q;
+struct alignas(16) ReplicaDesc {
+  // -- what the D2Q9 step kernels read, first and contiguous (kStepHeadBytes): the batched
+  // launches keep a copy of it in shared memory.  The arrays' alignment decides which constant-
+  // bank loads the compiler can merge, and the network kernel, whose registers are full, takes
+  // 4.42 ms per 16384^2 step with both at 4 mod 16 bytes, 4.45 - 4.75 with the seven others tried.
+  int32_t nx, ny;
   int32_t units_per_row;        // nx / VEC of the step launch
   uint32_t upr_magic;           // row of a unit u < 2^31: (u * upr_magic) >> upr_shift
   int32_t upr_shift;            //   (Granlund & Montgomery, PLDI'94, round-up multiplier)
-  int64_t n_units;              // units_per_row * ny * nz
-  int64_t block_begin;          // first virtual block of this replica in the step launch
-  uint32_t seed_lo, seed_hi, stream, noise_mask;
-  uint32_t rkey[20];            // Philox round keys (k0 + r W0, k1 + r W1), r = 0..9, of the key (seed_lo, seed_hi)
+  uint32_t stream, noise_mask;
   int32_t noise_mode;           // 0: independent noise (Eq. 8); 1: correlated (root in kCoNoiseR)
+  int64_t n_units;              // units_per_row * ny * nz
+  int64_t off_pop[2];           // population buffers (ping-pong)
+  int64_t off_fields;           // [n_fields][nz][ny][nx] Real
+  int32_t align0_;
+  uint32_t rkey[20];            // Philox round keys (k0 + r W0, k1 + r W1), r = 0..9, of the key (seed_lo, seed_hi)
   uint32_t field_mask, n_fields;
-  int32_t field_id[kMaxFields];     // slot -> field id
+  // the per-replica coefficients in the arithmetic type of the path (host-filled),
+  // so the FP32 kernels never convert from FP64: [kCoRho0], [kCoU0x .. kCoU0z],
+  // [kCoInvTau + a], [kCoAmp + a], [kCoMref + field], [kCoNoiseR + 6 c + c'] (c, c' index
+  // the non-conserved moments 3..8)
+  int32_t align1_[2];
+  float fco[kNumCoef];
+  // -- the rest
+  alignas(16) int32_t log2nx;
+  int32_t log2ny;
+  int32_t nz;                   // 3D depth (1 otherwise); a row is (y, z), row = z ny + y
+  int32_t q;
+  int64_t block_begin;          // first virtual block of this replica in the step launch
+  uint32_t seed_lo, seed_hi;
+  int32_t field_id[kMaxFields];     // slot -> field id, ascending
   int32_t n_pairs;
   int32_t pair_a[kMaxPairs], pair_b[kMaxPairs];   // slot indices, a <= b
   int64_t pair_off[kMaxPairs];      // byte offset of the pair's accumulator plane
@@ -51,8 +68,6 @@ struct ReplicaDesc {
   double inv_tau[kMaxQ];
   double amp[kMaxQ];                // (1/tau) sqrt(mu rho0 (2 tau - 1)), 0 when masked
   double mref[kMaxQ];               // reference value subtracted from each field id
-  int64_t off_pop[2];               // population buffers (ping-pong)
-  int64_t off_fields;               // [n_fields][nz][ny][nx] Real
   int64_t off_spec;                 // [n_fields][ny][wpitch] complex Real (row-transformed)
   int64_t spec_slot;                // bytes from spectrum slot 0 to slot 1 (two samples folded
                                     // into one accumulation pass; 0: one slot)
@@ -69,13 +84,11 @@ struct ReplicaDesc {
   int32_t acc_ncol;                 // pair-sum layout: 0 = [ky][kx]; c > 0 = blocked in the order
                                     // the column pass produces the points: [k1][kx / c][k2][kx % c]
                                     // (ky = k1 + N1 k2; kx padded to a multiple of c)
-  // the per-replica coefficients in the arithmetic type of the path (host-filled),
-  // so the FP32 kernels never convert from FP64: [kCoRho0], [kCoU0x .. kCoU0z],
-  // [kCoInvTau + a], [kCoAmp + a], [kCoMref + field], [kCoNoiseR + 6 c + c'] (c, c' index
-  // the non-conserved moments 3..8)
-  float fco[kNumCoef];
-  double dco[kNumCoef];
+  double dco[kNumCoef];             // fco in FP64
 };
+constexpr int kStepHeadBytes = offsetof(ReplicaDesc, log2nx);
+static_assert(offsetof(ReplicaDesc, rkey) % 16 == 4 && offsetof(ReplicaDesc, fco) % 16 == 4, "see the head's comment");
+static_assert(kStepHeadBytes % 16 == 0 && kStepHeadBytes <= 640 && sizeof(ReplicaDesc) % 16 == 0, "copied by 16 bytes");
 
 template <typename R> __device__ __forceinline__ R coef(const ReplicaDesc& d, int i);
 template <> __device__ __forceinline__ float coef<float>(const ReplicaDesc& d, int i) { return d.fco[i]; }
@@ -132,6 +145,18 @@ __device__ __forceinline__ float cos_approx(float x) { float y; asm("cos.approx.
 // FP64: u = (w + 1/2) 2^-32 (exact), evaluated in fixed point (normals64.cuh).
 __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, double& n0, double& n1) {
   fx_box_muller(wa, wb, n0, n1);
+}
+
+// The same with CUDA's FP64 functions, for the thermal starts: one pass per run, and an FP32 run
+// of a given seed stays the same bit for bit (a last-bit change of a normal rarely moves an FP32
+// population, but on a large lattice somewhere, and every later rounding with it).
+__device__ __forceinline__ void box_muller_start(uint32_t wa, uint32_t wb, double& n0, double& n1) {
+  const double ua = ((double)wa + 0.5) * 0x1p-32;
+  const double ub = ((double)wb + 0.5) * 0x1p-32;
+  const double r = sqrt(-2.0 * log(ua));
+  double s, c;
+  sincospi(2.0 * ub, &s, &c);
+  n0 = r * c; n1 = r * s;
 }
 
 // FP32: ua = RN(wa) 2^-32 + 2^-33 (relative error <= 2^-24 for every ua, small ua

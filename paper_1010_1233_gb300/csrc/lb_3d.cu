@@ -392,8 +392,8 @@ __device__ __forceinline__ void thermal_normals3(const ReplicaDesc& d, uint32_t 
 #pragma unroll
   for (int c = 0; c < Lat3<Q>::kThermalCalls; ++c) {
     const uint4 w = philox4x32_10(site, 0u, (uint32_t)c | (1u << 8), d.stream, d.seed_lo, d.seed_hi);
-    box_muller(w.x, w.y, N[4 * c + 0], N[4 * c + 1]);
-    box_muller(w.z, w.w, N[4 * c + 2], N[4 * c + 3]);
+    box_muller_start(w.x, w.y, N[4 * c + 0], N[4 * c + 1]);
+    box_muller_start(w.z, w.w, N[4 * c + 2], N[4 * c + 3]);
   }
 }
 

@@ -9,8 +9,9 @@
 // f*_i = f_i + sum_{a non-conserved} n_i^a (Delta M^a + xi^a), n_i^a = w_i m_i^a.
 // Density and momentum are untouched, so they are conserved up to rounding.
 // The variant with the noise-scale network is in lb_step_tc.cu.
+#include <algorithm>
 #include <cstdio>
-#include "step_common.cuh"
+#include "step_pair.cuh"
 #include "d1q3_common.cuh"
 
 #ifndef FLB_STEP_MINB_PLAIN
@@ -70,6 +71,92 @@ k_step_d2q9(const ReplicaDesc* __restrict__ descs, const __grid_constant__ Repli
 }
 
 // ---------------------------------------------------------------------------
+// The same step on the FP32 path for VEC = 2 or 4 sites per thread, two sites at a time on the
+// packed FP32 instructions (step_pair.cuh; bit for bit the scalar update) and with three
+// Philox calls per pair instead of two per site.  The scalar form is bound by instruction
+// issue: 370 instructions per site in the 64-replica sweep, 58 % of the issue slots.  us per
+// step, scalar and pairs: sweep 93 -> 81, 4096^2 202 -> 188 (95 % of the copy rate), 2048^2
+// 55 -> 49, 1510 x 1001 (vec 2, correlated noise) 24.6 -> 20.1.  24 (vec 4) and 32 (vec 2) warps
+// per SM are worth their few spilled registers: with 16 and 24, 198 us at 4096^2.
+//
+// Batched launches read a replica's description from shared memory (copied when a block's
+// replica changes): from global memory every use is a load through L1.  One-replica launches
+// have it in the constant bank.  Blocks may be smaller than the kStepThreads units of a virtual
+// block (blockDim = kStepThreads >> split), so that a small lattice reaches more SMs.
+// Fields are stored pair by pair where sampled (their slots follow from the field mask).
+template <int VEC, bool SAMPLE, int FL>
+__global__ void __launch_bounds__(kStepThreads, VEC == 4 ? 3 : 4)
+k_step_d2q9_pair(const ReplicaDesc* __restrict__ descs, const __grid_constant__ ReplicaDesc one,
+                 const int64_t* __restrict__ vb_begin, int n_reps, int64_t n_vblocks, char* __restrict__ ws,
+                 int parity, uint32_t step, const uint64_t* __restrict__ step_dev, int split) {
+  constexpr bool ONE = Flavor<FL>::kOne;
+  __shared__ uint4 head[ONE ? 1 : kStepHeadBytes / 16];
+  if (step_dev) {                  // graph replay: step = device base + offset
+    const uint64_t t = *step_dev + step;
+    step = (uint32_t)t;
+    parity = (int)(t & 1);
+  }
+  int cur = -1;
+  int64_t vb0 = 0;
+  for (int64_t h = blockIdx.x; h < n_vblocks << split; h += gridDim.x) {
+    const int64_t vb = h >> split;
+    const int tid = (int)(h & ((1 << split) - 1)) * (int)blockDim.x + (int)threadIdx.x;
+    if constexpr (!ONE) {
+      const int r = find_replica(vb_begin, n_reps, vb);
+      if (r != cur) {              // uniform over the block
+        __syncthreads();
+        const uint4* src = reinterpret_cast<const uint4*>(descs + r);
+        for (int i = threadIdx.x; i < kStepHeadBytes / 16; i += blockDim.x) head[i] = src[i];
+        __syncthreads();
+        cur = r;
+        vb0 = vb_begin[r];
+      }
+    }
+    const ReplicaDesc& d = ONE ? one : *reinterpret_cast<const ReplicaDesc*>(head);   // (its head)
+    const UnitPos u = unit_position(d, vb, vb0, tid, kStepThreads, VEC);
+    const int64_t plane = (int64_t)d.nx * d.ny;
+    const float* __restrict__ src = reinterpret_cast<const float*>(ws + d.off_pop[parity]);
+    float* __restrict__ dst = reinterpret_cast<float*>(ws + d.off_pop[parity ^ 1]);
+    float f[9][VEC];
+    pull_d2q9<float, VEC>(src, plane, d.nx, d.ny, u, f);
+    const float rho0 = coef<float>(d, kCoRho0);
+    const bool noisy = d.noise_mask != 0;
+    const bool in = u.active && FLB_INB(u.y >= 0 && u.y < d.ny && u.x0 >= 0 && u.x0 + VEC <= d.nx, 103);
+    const int64_t off = (int64_t)u.y * d.nx + u.x0;
+#pragma unroll
+    for (int p = 0; p < VEC / 2; ++p) {
+      float2 g[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) g[i] = make_float2(f[i][2 * p], f[i][2 * p + 1]);
+      float2 sum, ux, uy, D[6], fl[kMaxFields];
+      macro_pair(g, rho0, sum, ux, uy);
+      relax_pair<SAMPLE>(d, g, sum, ux, uy, D, fl);
+      if constexpr (SAMPLE) {
+        if (in) {
+          float* fields = reinterpret_cast<float*>(ws + d.off_fields) + off + 2 * p;
+          const uint32_t mask = d.field_mask;
+#pragma unroll
+          for (int a = 0; a < kMaxFields; ++a)
+            if ((mask >> a) & 1) *reinterpret_cast<float2*>(fields + __popc(mask & ((1u << a) - 1)) * plane) = fl[a];
+        }
+      }
+      float2 n[6] = {};
+      if (noisy) {
+        uint4 w0a, w1a, w0b, w1b;
+        philox_words_pair(d, (uint32_t)u.y * (uint32_t)d.nx + (uint32_t)(u.x0 + 2 * p), step, w0a, w1a, w0b, w1b);
+        normals_pair(w0a, w1a, w0b, w1b, n);
+      }
+      apply_pair<Flavor<FL>::kGen, false>(d, g, sum, noisy, n, n, D);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) { f[i][2 * p] = g[i].x; f[i][2 * p + 1] = g[i].y; }
+    }
+    if (!in) continue;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) VecIO<float, VEC>::st(dst + i * plane + off, f[i]);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // D1Q3, one step (d1q3_common.cuh) per launch.
 template <typename R, bool DEV, bool SAMPLE>
 __global__ void __launch_bounds__(256)
@@ -103,8 +190,8 @@ __device__ __forceinline__ void thermal_normals(const ReplicaDesc& d, uint32_t s
   const int calls = (q + 3) / 4;
   for (int c = 0; c < calls; ++c) {
     const uint4 w = philox4x32_10(site, 0u, (uint32_t)c | (1u << 8), d.stream, d.seed_lo, d.seed_hi);
-    box_muller(w.x, w.y, N[4 * c + 0], N[4 * c + 1]);
-    box_muller(w.z, w.w, N[4 * c + 2], N[4 * c + 3]);
+    box_muller_start(w.x, w.y, N[4 * c + 0], N[4 * c + 1]);
+    box_muller_start(w.z, w.w, N[4 * c + 2], N[4 * c + 3]);
   }
 }
 
@@ -244,6 +331,19 @@ static void launch_d2q9_vec(const StepLaunch& L, bool sample, bool mlp, cudaStre
       return;
     }
   }
+  if constexpr (VEC >= 2) {
+    // a lattice too small for a block of kStepThreads per SM: blocks of a quarter of that
+    const int split = L.n_vblocks < L.sms ? 2 : 0;
+    const int grid = (int)std::min<int64_t>(L.n_vblocks << split, (int64_t)L.grid << split);
+#define FLB_L(S, F) k_step_d2q9_pair<VEC, S, F><<<grid, kStepThreads >> split, 0, st>>>( \
+      L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
+#define FLB_LF(F) { if (sample) FLB_L(true, F); else FLB_L(false, F); }
+    const int fl = L.flavor();
+    if (fl == 0) FLB_LF(0) else if (fl == 1) FLB_LF(1) else FLB_LF(2)
+    return;
+#undef FLB_LF
+#undef FLB_L
+  } else {
 #define FLB_L(S, F) k_step_d2q9<R, DEV, VEC, S, F><<<L.grid, kStepThreads, 0, st>>>( \
       L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev)
 #define FLB_LF(F) { if (sample) FLB_L(true, F); else FLB_L(false, F); }
@@ -251,6 +351,7 @@ static void launch_d2q9_vec(const StepLaunch& L, bool sample, bool mlp, cudaStre
   if (fl == 0) FLB_LF(0) else if (fl == 1) FLB_LF(1) else FLB_LF(2)
 #undef FLB_LF
 #undef FLB_L
+  }
 }
 
 void launch_step(int lattice, int precision, int vec, const StepLaunch& L, bool sample, bool mlp,

@@ -78,22 +78,25 @@ __device__ __forceinline__ int64_t sum_limit(const ReplicaDesc& d, int ncol, int
 // point's shared-memory slot and its pair-sum index are computed once, each pair's sum is read
 // once for the nslots samples, three pairs' reads in flight.  The block's pairs are those
 // of group pg of ps (pairs 3 i .. 3 i + 2 with i % ps == pg); with more threads than points
-// they are dealt out again among the threads of a point.
-template <int PB>
+// they are dealt out again among the threads of a point.  SPLIT = false is the case of whole
+// tiles with no more threads than points (the index arithmetic of the split costs 6 % at 16384^2).
+template <int PB, bool SPLIT>
 __device__ __forceinline__ void accumulate_points(const ReplicaDesc& d, char* __restrict__ ws, const float2* s, int ss,
                                                   int k1, int kx0, int ncl, int w, int ncol, int tiles, int pg, int ps,
                                                   int nslots, int slot_elems) {
   const int lc = 31 - __clz(w);
   const int logn1 = d.log2n1, n1 = 1 << logn1, n2 = d.ny >> logn1;
   const int npts = n2 << lc, fstride = w * ss, np = d.n_pairs;
-  const int T = max((int)blockDim.x / npts, 1);          // threads per point (npts is a power of two)
+  const int T = SPLIT ? max((int)blockDim.x / npts, 1) : 1;      // threads per point (npts is a power of two)
   for (int it = threadIdx.x; it < npts * T; it += blockDim.x) {
-    const int i = it & (npts - 1), c = i & (w - 1), k2 = i >> lc;
+    const int i = SPLIT ? it & (npts - 1) : it, c = i & (w - 1), k2 = i >> lc;
     if (c >= ncl) continue;
-    const int64_t pt = sum_index(d, k1, n1, n2, kx0, c, k2, ncol, tiles);
+    int64_t pt;
+    if constexpr (SPLIT) pt = sum_index(d, k1, n1, n2, kx0, c, k2, ncol, tiles);
+    else pt = d.acc_ncol ? (int64_t)(k1 * tiles + (kx0 >> lc)) * npts + i : (int64_t)(k1 + n1 * k2) * d.half_nx + kx0 + c;
     if (!FLB_INB(pt < sum_limit(d, ncol, tiles) && c * ss + out_slot<PB>(k2) < fstride, 165)) continue;
     const float2* sp = s + c * ss + out_slot<PB>(k2);
-    for (int p0 = 3 * (pg + ps * (T > 1 ? it / npts : 0)); p0 < np; p0 += 3 * ps * T) {
+    for (int p0 = SPLIT ? 3 * (pg + ps * (it / npts)) : 0; p0 < np; p0 += SPLIT ? 3 * ps * T : 3) {
       double2 acc[3];
 #pragma unroll
       for (int u = 0; u < 3; ++u) {

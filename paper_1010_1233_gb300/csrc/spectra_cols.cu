@@ -120,7 +120,7 @@ __device__ __forceinline__ void a16_issue(const ReplicaDesc& d, const A16Unit& u
 // Pass 2b tile (N2 = L; one-pass columns are N1 = 1): the rows N2 k1 + y2 of the tile
 // transformed over y2, X(k2) left at slot out_slot<B>(k2), then the pair products added
 // to the FP64 sums.  All threads call it; it ends with a barrier.
-template <int B>
+template <int B, bool SPLIT>
 __device__ __forceinline__ void cols_acc16_tile(const ReplicaDesc& d, char* __restrict__ ws, float2* s, int rep,
                                                 int k1, int kx0, int ncl, int w, int ncol, int tiles, int pg, int ps,
                                                 const TimeCorr& tc, int nslots) {
@@ -163,7 +163,7 @@ __device__ __forceinline__ void cols_acc16_tile(const ReplicaDesc& d, char* __re
     }
   }
   __syncthreads();
-  accumulate_points<B>(d, ws, s, SS, k1, kx0, ncl, w, ncol, tiles, pg, ps, nslots, slot_elems);
+  accumulate_points<B, SPLIT>(d, ws, s, SS, k1, kx0, ncl, w, ncol, tiles, pg, ps, nslots, slot_elems);
   if (pg == 0) tile_tail<float, B>(d, ws, s, SS, rep, k1, kx0, ncl, w, tc, nslots, slot_elems);
   __syncthreads();
 }
@@ -273,21 +273,26 @@ k_fft_cols_a16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+#ifndef FLB_ACC16_MIN_BLOCKS
+#define FLB_ACC16_MIN_BLOCKS 4
+#endif
 // Pass 2b (N2 = L): one block per (replica, k1, tile of w columns, group of pairs), all
 // fields and the nslots samples of the tile; 64 registers a thread, four blocks of 256 threads
 // per SM on large lattices (measured against three, with 80 registers and no spills: 10.08
 // against 10.50 ms per 16384^2 sample), fewer and larger ones where there are few tiles.
-// vb_begin counts the layout's tiles of ncol columns, each cut as sp says (ColsSplit).
-template <int B>
-__global__ void __launch_bounds__(cols_block_max(4), 1)
+// vb_begin counts the layout's tiles of ncol columns, each cut as sp says (ColsSplit); SPLIT =
+// false: not at all, with blocks of 256 threads.
+template <int B, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? cols_block_max(4) : kColsBlock, SPLIT ? 1 : FLB_ACC16_MIN_BLOCKS)
 k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
                  int64_t n_vblocks, char* __restrict__ ws, int ncol, ColsSplit sp, TimeCorr tc, int nslots) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* s = reinterpret_cast<float2*>(smem_raw);
-  const int lw = 31 - __clz(sp.w), lc = 31 - __clz(ncol), lsub = lc - lw;
-  const int n_sub = sp.ps << lsub;
+  const int w = SPLIT ? sp.w : ncol, ps = SPLIT ? sp.ps : 1;
+  const int lw = 31 - __clz(w), lc = 31 - __clz(ncol), lsub = lc - lw;
+  const int n_sub = ps << lsub;
   for (int64_t v = blockIdx.x; v < n_vblocks * n_sub; v += gridDim.x) {
-    const int64_t vb = v / n_sub;
+    const int64_t vb = SPLIT ? v / n_sub : v;
     const int sub = (int)(v - vb * n_sub);
     const int rp = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[rp];
@@ -301,8 +306,8 @@ k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restric
     // blocked pair sums: the layout tile's sums of every pair are one contiguous range, pulled
     // into L2 by bulk prefetches while the columns are loaded and transformed
     if (d.acc_ncol && sub == 0) prefetch_sums(d, ws, k1, kx0, ncol, tiles, n2);
-    cols_acc16_tile<B>(d, ws, s, rp, k1, kx0, min(sp.w, d.half_nx - kx0), sp.w, ncol, tiles, sub >> lsub, sp.ps, tc,
-                       nslots);
+    cols_acc16_tile<B, SPLIT>(d, ws, s, rp, k1, kx0, min(w, d.half_nx - kx0), w, ncol, tiles, sub >> lsub, ps, tc,
+                              nslots);
   }
 }
 
@@ -314,8 +319,9 @@ cudaError_t set_fft16_smem_limits() {
   if (!e) e = cudaFuncSetAttribute(K, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
   FLB_ATTR(k_fft_cols_a16<1>) FLB_ATTR(k_fft_cols_a16<2>) FLB_ATTR(k_fft_cols_a16<4>)
   FLB_ATTR(k_fft_cols_a16<8>) FLB_ATTR(k_fft_cols_a16<16>)
-  FLB_ATTR(k_fft_cols_acc16<1>) FLB_ATTR(k_fft_cols_acc16<2>) FLB_ATTR(k_fft_cols_acc16<4>)
-  FLB_ATTR(k_fft_cols_acc16<8>) FLB_ATTR(k_fft_cols_acc16<16>)
+#define FLB_ACC(B) FLB_ATTR((k_fft_cols_acc16<B, false>)) FLB_ATTR((k_fft_cols_acc16<B, true>))
+  FLB_ACC(1) FLB_ACC(2) FLB_ACC(4) FLB_ACC(8) FLB_ACC(16)
+#undef FLB_ACC
 #undef FLB_ATTR
   return e;
 }
@@ -348,8 +354,13 @@ void launch_fft_cols_acc16(int mask, const ReplicaDesc* descs, const int64_t* vb
 #define FLB_L(B)                                                                                            \
   if (mask & B) {                                                                                           \
     const int smem = fft_cols16_smem(max_fields, 16 * B, sp.w, nslots);                                     \
-    k_fft_cols_acc16<B><<<grid, cols_threads(nb, sms, sp.w * 16 * B, smem), smem, st>>>(                    \
-        descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc, nslots);                                      \
+    const int block = cols_threads(nb, sms, sp.w * 16 * B, smem);                                           \
+    if (sp.w == ncol && sp.ps == 1 && block == kColsBlock && sp.w * 16 * B >= kColsBlock)                   \
+      k_fft_cols_acc16<B, false><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol,   \
+                                                            sp, tc, nslots);                                \
+    else                                                                                                    \
+      k_fft_cols_acc16<B, true><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol,    \
+                                                           sp, tc, nslots);                                 \
   }
   FLB_L(1) FLB_L(2) FLB_L(4) FLB_L(8) FLB_L(16)
 #undef FLB_L

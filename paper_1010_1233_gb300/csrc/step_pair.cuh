@@ -19,10 +19,10 @@ __device__ __forceinline__ void relax_pair(const ReplicaDesc& d, const float2 (&
   relax_site<float2, true, SAMPLE>(d, g, sum, ux, uy, D, fld);
 }
 
-template <bool GEN>
+template <bool GEN, bool SCALED = true>
 __device__ __forceinline__ void apply_pair(const ReplicaDesc& d, float2 (&g)[9], float2 sum, bool noisy,
                                            const float2 (&n)[6], const float2 (&sc)[6], const float2 (&Drel)[6]) {
-  apply_site<float2, true, GEN>(d, g, sum, noisy, n, sc, Drel);
+  apply_site<float2, true, GEN, SCALED>(d, g, sum, noisy, n, sc, Drel);
 }
 
 __device__ __forceinline__ void macro_pair(const float2 (&g)[9], float rho0, float2& sum, float2& ux, float2& uy) {
