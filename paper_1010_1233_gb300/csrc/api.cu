@@ -46,8 +46,14 @@ void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* v
 void launch_wait_probe(DevStatus* status, long long limit, cudaStream_t st);   // lb_step_tc.cu
 // D1Q3 runs of steps with their sampling in one launch (lb_d1q3_fused.cu)
 size_t d1q3_fused_smem(int precision, int nx, int F);
-cudaError_t launch_d1q3_fused(int precision, const ReplicaDesc* descs, int n_reps, char* ws, uint64_t t0,
+cudaError_t launch_d1q3_fused(const ReplicaDesc* descs, int n_reps, char* ws, uint64_t t0,
                               uint32_t n_steps, uint32_t every, size_t smem, cudaStream_t st);
+// FP64 D1Q3 runs (lb_d1q3_runs.cu)
+size_t d1q3_steps_smem(int nx);
+size_t d1q3_sample_smem(int nx, int F);
+cudaError_t set_d1q3_runs_smem();
+int launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0, uint32_t n_steps,
+                      int sms, cudaStream_t st);
 // D3Q15 / D3Q19 (lb_3d.cu), q = 15 or 19
 void launch_step3(int q, int precision, int vec, const StepLaunch& L, bool sample, cudaStream_t st);
 void launch_init3(int q, int precision, const ReplicaDesc* descs, int r, char* ws, int mode, const double* feq0,
@@ -120,6 +126,9 @@ static constexpr int kMaxPointItems = 2048;    // 3D direct transforms: fields x
 
 static constexpr int kStepBlock = 256;
 static constexpr int64_t kVec4Sites = 1 << 20;
+static constexpr size_t kFusedSmemMax = 200 * 1024;           // D1Q3 runs: shared memory of a block
+static constexpr int64_t kD1ScratchBytes = 64 << 20;
+static constexpr int kD1SampleBlocks = 152;
 
 struct Layout {
   std::vector<ReplicaDesc> desc;
@@ -134,6 +143,7 @@ struct Layout {
   int fold = 1;               // 2: two spectrum slots, two samples per accumulation pass
   int max_fields = 0;         // the most sampled fields of a replica with pair sums
   int max_len = 1;            // the longest column transform
+  D1Run d1;                   // FP64 D1Q3: chunked runs (chunk = 0: not used)
   int staged = 0;             // 1: the step kernel of lb_step_bulk.cu (tiles of 256 vec sites)
   bool any_fields = false;
 };
@@ -465,6 +475,30 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
       d.off_tw_y = off; off = align256(off + (int64_t)(d.ny / 2) * 2 * rs + 16);
     }
   }
+  if (lat == FLB_D1Q3 && precision == FLB_FP64) {
+    D1Run& run = L.d1;
+    size_t steps_smem = 0;
+    int64_t sites = 0;
+    for (const ReplicaDesc& d : L.desc) {
+      sites += d.nx;
+      run.max_nx = std::max(run.max_nx, (int)d.nx);
+      run.max_items = std::max(run.max_items, (int)d1q3_items(d));
+      if (d.n_fields) run.sample_smem = std::max(run.sample_smem, d1q3_sample_smem(d.nx, (int)d.n_fields));
+      steps_smem = std::max(steps_smem, d1q3_steps_smem(d.nx));
+    }
+    if (steps_smem <= kFusedSmemMax && run.sample_smem <= kFusedSmemMax) {
+      // a chunk's noise and pulled populations in at most kD1ScratchBytes, 1024 steps at most; the
+      // sampling kernel's blocks over the GPU
+      run.chunk = (uint32_t)std::max<int64_t>(16, std::min<int64_t>(1024, kD1ScratchBytes / (32 * sites)));
+      run.blocks = std::max(1, kD1SampleBlocks / n);
+      for (ReplicaDesc& d : L.desc) {
+        d.off_d1_noise = off; off = align256(off + 8 * (int64_t)run.chunk * d.nx);
+        if (!d.n_fields) continue;
+        d.off_d1_raw = off; off = align256(off + 24 * (int64_t)run.chunk * d.nx);
+        d.off_d1_part = off; off = align256(off + 16 * (int64_t)run.blocks * d1q3_items(d));
+      }
+    }
+  }
   // virtual-block prefixes of the three launches
   L.vb_step.resize(n); L.vb_rows.resize(n); L.vb_cols.resize(n); L.vb_cols_a.resize(n);
   if (maxF) {
@@ -564,7 +598,6 @@ using namespace flb;
 static constexpr uint32_t kGraphChunk = 32;      // at least this many steps per captured chunk
 static constexpr uint32_t kMaxGraphChunk = 4096;  // longer sampling periods are issued directly
 static constexpr uint32_t kFusedChunk = 4096;     // D1Q3 steps per fused launch
-static constexpr size_t kFusedSmemMax = 200 * 1024;
 
 struct flb_ctx {
   int precision = 0, lattice = 0, n = 0;
@@ -878,7 +911,8 @@ int flb_create(int precision, const flb_replica* reps, int n_replicas, void* dev
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   if ((rc = cuda_check(set_fft_smem_limits(), "smem limits"))) { delete c; return rc; }
-  if (c->lattice == FLB_D1Q3) {      // the fused kernel holds a replica in one block's shared memory
+  if (c->L.d1.chunk && (rc = cuda_check(set_d1q3_runs_smem(), "smem limits"))) { delete c; return rc; }
+  if (c->lattice == FLB_D1Q3 && precision != FLB_FP64) {      // the fused kernel holds a replica in one block's shared memory
     size_t smem = 0;
     for (const ReplicaDesc& d : c->L.desc)
       smem = std::max(smem, d1q3_fused_smem(precision, d.nx, (int)d.n_fields));
@@ -1068,13 +1102,31 @@ int flb_run(flb_ctx* c, uint64_t n_steps, uint32_t sample_every) {
   if (!c) return set_error(FLB_EINVAL, "ctx is NULL");
   const Layout& L = c->L;
   const bool sampling = sample_every && L.any_fields;
+  if (L.d1.chunk && c->use_graphs && !c->tc.base && n_steps > 1) {
+    // FP64 D1Q3: chunks of steps, their noise before and their sampling after the serial part (one
+    // sampled step by itself: 27 us, as separate launches 17; two 28 and 29)
+    NvtxRange chunk_range("flb D1Q3 chunks");
+    D1Run run = L.d1;
+    run.every = sampling ? sample_every : 0;
+    for (uint64_t i = 0; i < n_steps;) {
+      const uint32_t n = (uint32_t)std::min<uint64_t>(n_steps - i, run.chunk);
+      count_kernels(c, launch_d1q3_chunk(descs_dev(c), c->n, c->ws, run, c->step, n, c->sms, c->stream));
+      if (run.every) {
+        const uint64_t first = (c->step + run.every - 1) / run.every * run.every;
+        if (first < c->step + n) c->n_samples += (c->step + n - 1 - first) / run.every + 1;
+      }
+      c->step += n;
+      i += n;
+    }
+    return cuda_check(cudaGetLastError(), "D1Q3 launch");
+  }
   if (c->fused_smem && c->use_graphs && !c->tc.base) {
-    // D1Q3: runs of up to kFusedChunk steps with their sampling in one launch
+    // FP32 D1Q3: runs of up to kFusedChunk steps with their sampling in one launch
     NvtxRange fused_range("flb fused D1Q3 steps");
     const uint32_t every = sampling ? sample_every : 0;
     for (uint64_t i = 0; i < n_steps;) {
       const uint32_t n = (uint32_t)std::min<uint64_t>(n_steps - i, kFusedChunk);
-      int rc = cuda_check(launch_d1q3_fused(c->precision, descs_dev(c), c->n, c->ws, c->step, n, every,
+      int rc = cuda_check(launch_d1q3_fused(descs_dev(c), c->n, c->ws, c->step, n, every,
                                             c->fused_smem, c->stream), "fused D1Q3 launch");
       if (rc) return rc;
       count_kernels(c, 1);

@@ -85,6 +85,7 @@ struct alignas(16) ReplicaDesc {
                                     // the column pass produces the points: [k1][kx / c][k2][kx % c]
                                     // (ky = k1 + N1 k2; kx padded to a multiple of c)
   double dco[kNumCoef];             // fco in FP64
+  int64_t off_d1_noise, off_d1_raw, off_d1_part;   // FP64 D1Q3 runs: scratch (lb_d1q3_runs.cu)
 };
 constexpr int kStepHeadBytes = offsetof(ReplicaDesc, log2nx);
 static_assert(offsetof(ReplicaDesc, rkey) % 16 == 4 && offsetof(ReplicaDesc, fco) % 16 == 4, "see the head's comment");
@@ -200,6 +201,18 @@ struct TimeCorr {
   uint64_t* count = nullptr;        // [n_replicas]: samples written so far
   int part_blocks = 0;              // 3D lattices: blocks of the direct transform (partials per replica)
 };
+
+// A run of FP64 D1Q3 steps (lb_d1q3_runs.cu): steps per chunk and what its launches are sized by
+// (over the replicas of the context), sampling period (0: none).
+struct D1Run {
+  uint32_t chunk = 0, every = 0;
+  int max_nx = 0, blocks = 0, max_items = 0;   // blocks of the sampling kernel per replica
+  size_t sample_smem = 0;
+};
+// partial sums of a block: every pair's half spectrum and the k = 0 value of every field
+__host__ __device__ __forceinline__ int64_t d1q3_items(const ReplicaDesc& d) {
+  return (int64_t)d.n_pairs * (d.nx / 2 + 1) + d.n_fields;
+}
 
 // Arguments of one step launch (lb_step.cu).
 struct StepLaunch {

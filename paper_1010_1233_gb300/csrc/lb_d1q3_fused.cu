@@ -1,4 +1,5 @@
-// D1Q3 steps and their correlator sampling fused into one launch.
+// FP32 D1Q3 steps and their correlator sampling fused into one launch (FP64: lb_d1q3_runs.cu,
+// whose split would change the rounding of FP32 sites here and there).
 //
 // The one-dimensional lattices are small (L = 64 in the D1Q3 workload): as separate
 // launches per step (step, row transform, pair accumulation) they are bound by launch
@@ -157,20 +158,12 @@ k_d1q3_fused(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint6
   }
 }
 
-cudaError_t launch_d1q3_fused(int precision, const ReplicaDesc* descs, int n_reps, char* ws, uint64_t t0,
+cudaError_t launch_d1q3_fused(const ReplicaDesc* descs, int n_reps, char* ws, uint64_t t0,
                               uint32_t n_steps, uint32_t every, size_t smem, cudaStream_t st) {
-  cudaError_t e;
-  if (precision == FLB_FP64) {
-    if ((e = cudaFuncSetAttribute(k_d1q3_fused<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)))
-      return e;
-    k_d1q3_fused<double, false><<<n_reps, kD1q3FusedThreads, smem, st>>>(descs, ws, t0, n_steps, every);
-  } else {
-    if ((e = cudaFuncSetAttribute(k_d1q3_fused<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)))
-      return e;
-    k_d1q3_fused<float, true><<<n_reps, kD1q3FusedThreads, smem, st>>>(descs, ws, t0, n_steps, every);
-  }
+  const cudaError_t e = cudaFuncSetAttribute(k_d1q3_fused<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+  if (e) return e;
+  k_d1q3_fused<float, true><<<n_reps, kD1q3FusedThreads, smem, st>>>(descs, ws, t0, n_steps, every);
   return cudaGetLastError();
 }
 
