@@ -38,7 +38,11 @@ void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_
                      int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms);
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
-                     int nslots, int max_fields, int max_len, int max_pairs, int sms);
+                     int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split);
+int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                      char* ws, cudaStream_t st, int paths, int slot, int max_len, int sms);
+void launch_pair_sums(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                      char* ws, int ncol, int max_fields, int nslots, cudaStream_t st, const TimeCorr& tc, int sms);
 void launch_time_corr(const ReplicaDesc* descs, int n_reps, int max_fields, const TimeCorr& tc, cudaStream_t st);
 void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                        int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
@@ -132,13 +136,16 @@ static constexpr int kD1SampleBlocks = 152;
 
 struct Layout {
   std::vector<ReplicaDesc> desc;
-  int64_t off_descs = 0, off_vb_step = 0, off_vb_rows = 0, off_vb_cols = 0, off_vb_cols_a = 0;
+  int64_t off_descs = 0, off_vb_step = 0, off_vb_rows = 0, off_vb_cols = 0, off_vb_cols_a = 0, off_vb_t = 0, off_vb_pts = 0;
   int64_t off_status = 0, off_sums = 0, off_partial = 0, off_feq0 = 0, off_mlp = 0, off_stepdev = 0;
   int64_t total = 0;
-  int64_t n_vb_step = 0, n_vb_rows = 0, n_vb_cols = 0, n_vb_cols_a = 0;
-  std::vector<int64_t> vb_step, vb_rows, vb_cols, vb_cols_a;
+  int64_t n_vb_step = 0, n_vb_rows = 0, n_vb_cols = 0, n_vb_cols_a = 0, n_vb_t = 0, n_vb_pts = 0;
+  std::vector<int64_t> vb_step, vb_rows, vb_cols, vb_cols_a, vb_t, vb_pts;
   int vec = 1, q = 9, ncol = 0, rows_smem = 0, cols_smem = 0;
   int cols_a_paths = 0, cols_paths = 0;   // column-pass kernels the replicas need (cols16_b)
+  bool split = false;         // one-pass replicas: transforms and pair sums apart (spectra.cu)
+  bool any_fused = true;      // some sampled replica's columns go through the fused pass
+  int t_paths = 0, t_len = 1; // split: lengths among the one-pass replicas, the longest of the shared-memory kernel's
   int rows_paths = 0;                     // row-pass kernels (launch_fft_rows)
   int fold = 1;               // 2: two spectrum slots, two samples per accumulation pass
   int max_fields = 0;         // the most sampled fields of a replica with pair sums
@@ -499,7 +506,30 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
       }
     }
   }
-  // virtual-block prefixes of the three launches
+  // one-pass columns apart from their pair sums, from kSplitPoints points of the launch
+  {
+    int64_t points = 0;
+    for (const ReplicaDesc& d : L.desc)
+      if (d.n_pairs && !d.log2n1 && lat != FLB_D1Q3) points += (int64_t)d.ny * d.half_nx;
+    L.split = points >= kSplitPoints;
+  }
+  if (L.split) {
+    L.any_fused = false;
+    L.cols_paths = 0;
+    for (const ReplicaDesc& d : L.desc) {
+      if (!d.n_pairs) continue;
+      const int b = precision == FLB_FP64 ? 0 : cols16_b(d.ny >> d.log2n1);
+      if (d.log2n1) {
+        L.any_fused = true;
+        L.cols_paths |= b ? b : kColsGeneric;
+      } else {
+        L.t_paths |= b ? b : kColsGeneric;
+        if (!b) L.t_len = std::max(L.t_len, (int)d.ny);
+      }
+    }
+  }
+  // virtual-block prefixes of the launches
+  L.vb_t.resize(n); L.vb_pts.resize(n);
   L.vb_step.resize(n); L.vb_rows.resize(n); L.vb_cols.resize(n); L.vb_cols_a.resize(n);
   if (maxF) {
     // the shared-memory row kernel's launch (replicas the Stockham kernel does not take)
@@ -513,6 +543,12 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
     L.vb_rows[r] = L.n_vb_rows;
     L.vb_cols[r] = L.n_vb_cols;
     L.vb_cols_a[r] = L.n_vb_cols_a;
+    L.vb_t[r] = L.n_vb_t;
+    L.vb_pts[r] = L.n_vb_pts;
+    if (d.n_pairs && L.split && !d.log2n1) {
+      L.n_vb_t += cols_t_blocks(d);
+      L.n_vb_pts += pair_blocks(d, L.ncol);
+    }
     if (d.n_pairs) {
       const int64_t tiles = (d.half_nx + L.ncol - 1) / L.ncol;
       L.n_vb_rows += rows_blocks(precision, d.nx, (int)d.n_fields, d.ny);
@@ -525,6 +561,8 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   L.off_vb_rows = off; off = align256(off + 8 * (int64_t)n);
   L.off_vb_cols = off; off = align256(off + 8 * (int64_t)n);
   L.off_vb_cols_a = off; off = align256(off + 8 * (int64_t)n);
+  L.off_vb_t = off; off = align256(off + 8 * (int64_t)n);
+  L.off_vb_pts = off; off = align256(off + 8 * (int64_t)n);
   L.off_status = off; off = align256(off + (int64_t)sizeof(DevStatus));
   L.off_sums = off; off = align256(off + 8 * 4 * (int64_t)n);
   L.off_partial = off; off = align256(off + 8 * 4 * (int64_t)kReduceBlocks);
@@ -926,6 +964,8 @@ int flb_create(int precision, const flb_replica* reps, int n_replicas, void* dev
   if (!rc) rc = cuda_check(cudaMemcpyAsync(c->ws + Lc.off_vb_rows, Lc.vb_rows.data(), 8 * n_replicas, cudaMemcpyHostToDevice, st), "copy vb");
   if (!rc) rc = cuda_check(cudaMemcpyAsync(c->ws + Lc.off_vb_cols, Lc.vb_cols.data(), 8 * n_replicas, cudaMemcpyHostToDevice, st), "copy vb");
   if (!rc) rc = cuda_check(cudaMemcpyAsync(c->ws + Lc.off_vb_cols_a, Lc.vb_cols_a.data(), 8 * n_replicas, cudaMemcpyHostToDevice, st), "copy vb");
+  if (!rc) rc = cuda_check(cudaMemcpyAsync(c->ws + Lc.off_vb_t, Lc.vb_t.data(), 8 * n_replicas, cudaMemcpyHostToDevice, st), "copy vb");
+  if (!rc) rc = cuda_check(cudaMemcpyAsync(c->ws + Lc.off_vb_pts, Lc.vb_pts.data(), 8 * n_replicas, cudaMemcpyHostToDevice, st), "copy vb");
   std::vector<double> feq(kFeqStride * (size_t)n_replicas);
   for (int r = 0; r < n_replicas; ++r) feq0_host(reps[r], &feq[kFeqStride * (size_t)r]);
   if (!rc) rc = cuda_check(cudaMemcpyAsync(c->ws + Lc.off_feq0, feq.data(), feq.size() * 8, cudaMemcpyHostToDevice, st), "copy feq0");
@@ -976,10 +1016,17 @@ static void launch_step_any(flb_ctx* c, int vec, int staged, const StepLaunch& S
 static void flush_samples(flb_ctx* c, const StepLaunch& S, cudaStream_t st) {
   const Layout& L = c->L;
   if (!c->pending) return;
-  launch_fft_cols(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_cols), c->n,
-                  L.n_vb_cols, c->ws, L.ncol, st, c->tc, L.cols_paths, c->pending, L.max_fields, L.max_len,
-                  L.max_fields * (L.max_fields + 1) / 2, c->sms);
-  count_kernels(c, path_launches(c->precision, L.cols_paths));
+  if (L.any_fused) {
+    launch_fft_cols(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_cols), c->n,
+                    L.n_vb_cols, c->ws, L.ncol, st, c->tc, L.cols_paths, c->pending, L.max_fields, L.max_len,
+                    L.max_fields * (L.max_fields + 1) / 2, c->sms, L.split);
+    count_kernels(c, path_launches(c->precision, L.cols_paths));
+  }
+  if (L.split) {
+    launch_pair_sums(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_pts), c->n, L.n_vb_pts,
+                     c->ws, L.ncol, L.max_fields, c->pending, st, c->tc, c->sms);
+    count_kernels(c, 1);
+  }
   c->pending = 0;
   if (c->tc.base) {
     int maxF = 0;
@@ -1019,6 +1066,9 @@ static void issue_step(flb_ctx* c, StepLaunch& S, bool sample, cudaStream_t st) 
                         L.cols_a_paths, slot, c->sms);
     count_kernels(c, path_launches(c->precision, L.rows_paths) +
                          (L.n_vb_cols_a ? path_launches(c->precision, L.cols_a_paths) : 0));
+    if (L.split)
+      count_kernels(c, launch_fft_cols_t(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_t),
+                                         c->n, L.n_vb_t, c->ws, st, L.t_paths, slot, L.t_len, c->sms));
     c->pending = slot + 1;
     if (!fold || c->pending == 2) flush_samples(c, S, st);
   }

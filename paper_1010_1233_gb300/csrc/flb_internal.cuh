@@ -287,6 +287,16 @@ inline ColsSplit cols_split(int precision, int64_t n_tiles, int ncol, int max_pa
   }
   return sp;
 }
+// The split accumulation of one-pass columns (spectra.cu): tiles of kColsT columns of one field for the
+// transforms, kColsBlock points of the sums per block; used from kSplitPoints half-spectrum points
+// of a launch (64^2, 3 fields, is 2112: one fused launch of 11 us against two of 5).
+constexpr int kColsT = 4;
+constexpr int64_t kSplitPoints = 8192;
+inline int64_t cols_t_blocks(const ReplicaDesc& d) { return (int64_t)d.n_fields * ((d.half_nx + kColsT - 1) / kColsT); }
+inline int64_t pair_blocks(const ReplicaDesc& d, int ncol) {
+  const int64_t pts = d.acc_ncol ? (int64_t)d.ny * ((d.half_nx + ncol - 1) / ncol) * ncol : (int64_t)d.ny * d.half_nx;
+  return (pts + kColsBlock - 1) / kColsBlock;
+}
 // threads of a block of the accumulation pass: about 1024 per SM, no more than the tile's points
 inline int cols_threads(int64_t nb, int sms, int points, int smem) {
   const int64_t fit = 227 * 1024 / (smem + 1024), per_sm = (nb + sms - 1) / sms;

@@ -201,12 +201,12 @@ k_fft_cols_a(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ 
 
 // Pass 2b: one block per (replica, k1, tile of w columns, group of pairs); all fields of the
 // tile.  One-pass columns are the case N1 = 1.  vb_begin counts the layout's tiles of ncol
-// columns, each cut as sp says (ColsSplit).
+// columns, each cut as sp says (ColsSplit); split: one-pass replicas are k_pair_sums'.
 template <typename R>
 __global__ void __launch_bounds__(cols_block_max(sizeof(R)), 1)
 k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin,
                                int n_reps, int64_t n_vblocks, char* __restrict__ ws, int ncol, ColsSplit sp,
-                               TimeCorr tc) {
+                               TimeCorr tc, bool split) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C<R>* s = reinterpret_cast<C<R>*>(smem_raw);
   const int w = sp.w, lc = 31 - __clz(w), lsub = 31 - __clz(ncol) - lc;      // powers of two
@@ -217,6 +217,7 @@ k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
     const int r = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[r];
     if (sizeof(R) == 4 && cols16_b(d.ny >> d.log2n1)) continue;     // a register-resident kernel's block
+    if (split && !d.log2n1) continue;                               // k_pair_sums' replica
     const int tiles = (d.half_nx + ncol - 1) >> (lc + lsub);
     const int64_t local = vb - vb_begin[r];
     const int k1 = (int)(local / tiles);
@@ -255,6 +256,165 @@ k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
     accumulate_tile<R, 0>(d, ws, s, n2 + 1, k1, kx0, ncl, w, ncol, tiles, pg, sp.ps);
     if (pg == 0) tile_tail<R, 0>(d, ws, s, n2 + 1, r, k1, kx0, ncl, w, tc, 1, 0);
     __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// One-pass columns (N1 = 1) of lattices with kSplitPoints or more half-spectrum points in the launch:
+// the column transforms in place (k_fft_cols_t here, k_fft_cols_t16 in spectra_cols.cu), then the pair
+// sums point by point (k_pair_sums).  The fused pass holds all fields of a tile in shared memory
+// through the FP64 additions, so few warps were left to keep the sums' reads and writes in flight;
+// apart, the transforms run one field per block and the sums stream at whole lines, for one more
+// write and read of the spectrum.  us per sample, fused and apart: FP64 256^2 with 9 fields 70 -> 57,
+// the 64-replica sweep 286 -> 231, 3 x 1024 x 2048 96 -> 73; whole runs: 256^2 with 9 fields FP32, 2000
+// steps with 200 samples, 11.5 -> 10.5 ms.
+
+// One block per (replica, field, tile of w columns): the columns transformed over y in place.
+template <typename R>
+__global__ void __launch_bounds__(kColsBlock, sizeof(R) == 4 ? 4 : 2)
+k_fft_cols_t(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
+             int64_t n_vblocks, char* __restrict__ ws, int w, int slot) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C<R>* s = reinterpret_cast<C<R>*>(smem_raw);
+  const int lw = 31 - __clz(w);
+  for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
+    const int r = find_rep(vb_begin, n_reps, vb);
+    const ReplicaDesc& d = descs[r];
+    if (d.log2n1 || (sizeof(R) == 4 && cols16_b(d.ny))) continue;      // another kernel's replica
+    const int tiles = (d.half_nx + w - 1) >> lw;
+    const int local = (int)(vb - vb_begin[r]), f = local / tiles;
+    if (f >= (int)d.n_fields) continue;                 // (the prefix counts the narrowest tiles)
+    const int kx0 = (local - f * tiles) << lw, ncl = min(w, d.half_nx - kx0);
+    const int logn = d.log2ny, n = d.ny, total = n << lw;
+    C<R>* col = reinterpret_cast<C<R>*>(ws + d.off_spec + slot * d.spec_slot) + (int64_t)f * n * d.wpitch + kx0;
+    for (int i0 = threadIdx.x; i0 < total; i0 += 4 * blockDim.x) {     // four loads in flight
+      C<R> v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * blockDim.x, c = i & (w - 1), y = i >> lw;
+        v[u].x = (R)0; v[u].y = (R)0;
+        if (i < total && c < ncl && FLB_INB(y < n && kx0 + c < d.half_nx, 151)) v[u] = col[(int64_t)y * d.wpitch + c];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * blockDim.x, c = i & (w - 1), y = i >> lw;
+        if (i < total && FLB_INB(brev(y, logn) < n, 152)) s[c * (n + 1) + brev(y, logn)] = v[u];
+      }
+    }
+    __syncthreads();
+    dit_fft<R>(s, logn, w, n + 1, reinterpret_cast<const C<R>*>(ws + d.off_tw_y), 1);
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+      const int c = i & (w - 1), y = i >> lw;
+      if (c < ncl) col[(int64_t)y * d.wpitch + c] = s[c * (n + 1) + y];
+    }
+    __syncthreads();
+  }
+}
+
+// Pair sums of transformed fields: thread = one point of the sums' layout (and one group of field rows),
+// X_f of all fields in registers, then per field a the pairs (a, b >= a), kPairBatch sums in flight.
+// gs groups: group g takes the rows a = g, 2 gs - 1 - g, 2 gs + g, .. (rows a and F - 1 - a together
+// have F + 1 pairs).  The first block of a replica also records the time-correlator ring entries and
+// adds the k = 0 values.
+// FM: the most fields of a replica the kernel is compiled for (its registers).
+constexpr int kPairBatch = 4;
+template <typename R, int FM>
+__global__ void __launch_bounds__(kColsBlock, FM <= 3 ? (sizeof(R) == 4 ? 4 : 3) : 2)
+k_pair_sums(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
+            int64_t n_vblocks, char* __restrict__ ws, int ncol, int gs, int nslots, TimeCorr tc) {
+  for (int64_t v = blockIdx.x; v < n_vblocks * gs; v += gridDim.x) {
+    const int64_t vb = v / gs;
+    const int grp = (int)(v - vb * gs);
+    const int r = find_rep(vb_begin, n_reps, vb);
+    const ReplicaDesc& d = descs[r];
+    if (d.log2n1) continue;                             // the fused pass's replica
+    const int F = (int)d.n_fields, hn = d.half_nx, ny = d.ny;
+    const int64_t pt = (vb - vb_begin[r]) * kColsBlock + threadIdx.x;
+    const C<R>* spec = reinterpret_cast<const C<R>*>(ws + d.off_spec);
+    const int64_t fplane = (int64_t)ny * d.wpitch, slot = d.spec_slot / (int64_t)sizeof(C<R>);
+    if (vb == vb_begin[r] && grp == 0) {
+      if (tc.base) {
+        const int rs = (int)(tc.count[r] % (uint64_t)tc.n_lags);
+        double2* ring = reinterpret_cast<double2*>(tc.base + d.off_tc_ring);
+        for (int i = threadIdx.x; i < tc.n_k * F; i += blockDim.x) {
+          const int j = i % tc.n_k, f = i / tc.n_k;
+          if (!FLB_INB(tc.kx[j] < hn && tc.ky[j] < ny, 164)) continue;
+          const C<R> X = spec[f * fplane + (int64_t)tc.ky[j] * d.wpitch + tc.kx[j]];
+          ring[((int64_t)rs * F + f) * tc.n_k + j] = make_double2((double)X.x, (double)X.y);
+        }
+      }
+      if (threadIdx.x < F) {
+        double* m0 = reinterpret_cast<double*>(ws + d.off_mean0) + threadIdx.x;
+        double m = *m0;
+        for (int k = 0; k < nslots; ++k) m += (double)spec[k * slot + threadIdx.x * fplane].x;
+        *m0 = m;
+      }
+    }
+    // the point's (ky, kx): blocked layout [tile][ky][c] (N1 = 1) or [ky][kx]
+    int ky, kx;
+    bool in;
+    if (d.acc_ncol) {
+      const int lc = 31 - __clz(ncol);
+      const int64_t row = pt >> lc;
+      const int tile = (int)(row >> d.log2ny);
+      ky = (int)(row & (ny - 1));
+      kx = (tile << lc) + (int)(pt & (ncol - 1));
+      in = kx < hn;
+    } else {
+      ky = (int)((uint32_t)pt / (uint32_t)hn);          // fewer than 2^31 points
+      kx = (int)(pt - (int64_t)ky * hn);
+      in = ky < ny;
+    }
+    if (!in || !FLB_INB(ky < ny && kx < d.wpitch && pt < sum_limit(d, ncol, (hn + ncol - 1) / ncol), 165)) continue;
+    const C<R>* p = spec + (int64_t)ky * d.wpitch + kx;
+    C<R> X0[FM], X1[FM];
+#pragma unroll
+    for (int f = 0; f < FM; ++f)
+      if (f < F) {
+        X0[f] = p[f * fplane];
+        if (sizeof(R) == 4 && nslots > 1) X1[f] = p[slot + f * fplane];
+      }
+    int pr0 = 0;                                        // index of pair (a, a)
+#pragma unroll
+    for (int a = 0; a < FM; ++a) {
+      if (a >= F) break;
+      const int am = a % (2 * gs);
+      if (am == grp || am == 2 * gs - 1 - grp) {
+#pragma unroll
+        for (int b0 = a; b0 < FM; b0 += kPairBatch) {
+          double2 acc[kPairBatch];
+#pragma unroll
+          for (int u = 0; u < kPairBatch; ++u) {
+            const int b = b0 + u;
+            if (b >= FM || b >= F) break;
+            const double* q = reinterpret_cast<const double*>(ws + d.pair_off[pr0 + b - a]);
+            if (b == a) acc[u].x = q[pt];
+            else acc[u] = load_sum2(q + 2 * pt);
+          }
+#pragma unroll
+          for (int u = 0; u < kPairBatch; ++u) {
+            const int b = b0 + u;
+            if (b >= FM || b >= F) break;
+            double* q = reinterpret_cast<double*>(ws + d.pair_off[pr0 + b - a]);
+            // the product in the transform's precision, the sums in FP64, sample by sample
+#pragma unroll
+            for (int k = 0; k < (sizeof(R) == 4 ? 2 : 1); ++k) {
+              if (k >= nslots) break;
+              const C<R> Xa = k ? X1[a] : X0[a], Xb = k ? X1[b] : X0[b];
+              if (b == a) {
+                acc[u].x += widen(Xa.x * Xa.x + Xa.y * Xa.y);
+              } else {
+                acc[u].x += widen(Xa.x * Xb.x + Xa.y * Xb.y);     // X_a X_b^*
+                acc[u].y += widen(Xa.y * Xb.x - Xa.x * Xb.y);
+              }
+            }
+            if (b == a) q[pt] = acc[u].x;
+            else store_sum2(q + 2 * pt, acc[u]);
+          }
+        }
+      }
+      pr0 += F - a;
+    }
   }
 }
 
@@ -306,7 +466,7 @@ void launch_fft_cols_a16(int mask, const ReplicaDesc* descs, const int64_t* vb_b
                          char* ws, int grid, cudaStream_t st, int slot);
 void launch_fft_cols_acc16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
                            char* ws, int ncol, const ColsSplit& sp, int sms, int max_fields, cudaStream_t st,
-                           const TimeCorr& tc, int nslots);
+                           const TimeCorr& tc, int nslots, bool split);
 cudaError_t set_fft16_smem_limits();
 void launch_fft_rows16(const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks, char* ws,
                        int grid, int nx, cudaStream_t st, int slot);
@@ -345,6 +505,8 @@ cudaError_t set_fft_smem_limits() {
   if ((e = cudaFuncSetAttribute(k_fft_cols_a<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb))) return e;
   if ((e = cudaFuncSetAttribute(k_fft_cols_a<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb))) return e;
   if ((e = cudaFuncSetAttribute(k_fft_cols_acc<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb))) return e;
+  if ((e = cudaFuncSetAttribute(k_fft_cols_t<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb))) return e;
+  if ((e = cudaFuncSetAttribute(k_fft_cols_t<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxb))) return e;
   if ((e = set_rows16_smem_limits())) return e;
   return set_fft16_smem_limits();
 }
@@ -384,11 +546,48 @@ void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* v
                       (int)std::min<int64_t>((int64_t)grid, 4 * (int64_t)sms), st, slot);
 }
 
+void launch_fft_cols_t16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                         char* ws, int grid, cudaStream_t st, int slot);
+
+// Column transforms in place of the one-pass replicas (paths: the lengths among them, as in
+// launch_fft_cols; max_len: the longest of the shared-memory kernel's); returns the launches.
+int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                      char* ws, cudaStream_t st, int paths, int slot, int max_len, int sms) {
+  const int grid = (int)std::min<int64_t>(n_vblocks, 16 * (int64_t)sms);
+  int launches = 0;
+  if (precision == FLB_FP64 || (paths & kColsGeneric)) {
+    const int smem = kColsT * (max_len + 1) * (precision == FLB_FP64 ? 16 : 8);
+    if (precision == FLB_FP64)
+      k_fft_cols_t<double><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, kColsT, slot);
+    else
+      k_fft_cols_t<float><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, kColsT, slot);
+    ++launches;
+  }
+  if (precision != FLB_FP64) {
+    launch_fft_cols_t16(paths & (kColsGeneric - 1), descs, vb_begin, n_reps, n_vblocks, ws, grid, st, slot);
+    launches += __builtin_popcount(paths & (kColsGeneric - 1));
+  }
+  return launches;
+}
+
+void launch_pair_sums(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                      char* ws, int ncol, int max_fields, int nslots, cudaStream_t st, const TimeCorr& tc, int sms) {
+  // groups of field rows where the points alone do not fill the GPU (half the fields at most)
+  int gs = 1;
+  while (2 * gs < max_fields && n_vblocks * gs < 4 * (int64_t)sms) ++gs;
+  const int grid = (int)std::min<int64_t>(n_vblocks * gs, 32 * (int64_t)sms);
+#define FLB_L(R, FM) k_pair_sums<R, FM><<<grid, kColsBlock, 0, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, gs, nslots, tc)
+#define FLB_LR(R) { if (max_fields <= 3) FLB_L(R, 3); else if (max_fields <= 6) FLB_L(R, 6); else FLB_L(R, kMaxFields); }
+  if (precision == FLB_FP64) FLB_LR(double) else FLB_LR(float)
+#undef FLB_LR
+#undef FLB_L
+}
+
 // max_fields, max_len: the most fields and the longest column transform of a replica (the
 // shared-memory kernel's launch holds them)
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
-                     int nslots, int max_fields, int max_len, int max_pairs, int sms) {
+                     int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split) {
   const ColsSplit sp = cols_split(precision, n_vblocks, ncol, max_pairs, sms);
   if (precision == FLB_FP64 || (paths & kColsGeneric)) {    // one slot (the host folds samples only without it)
     const int smem = fft_cols_smem(precision, max_fields, max_len, sp.w);
@@ -396,13 +595,13 @@ void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_
     const int grid = (int)std::min<int64_t>(nb, 8 * (int64_t)sms);
     const int block = std::min(cols_threads(nb, sms, sp.w * max_len, smem), cols_block_max(precision == FLB_FP64 ? 8 : 4));
     if (precision == FLB_FP64)
-      k_fft_cols_acc<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc);
+      k_fft_cols_acc<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc, split);
     else
-      k_fft_cols_acc<float><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc);
+      k_fft_cols_acc<float><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, tc, split);
   }
   if (precision != FLB_FP64)
     launch_fft_cols_acc16(paths & (kColsGeneric - 1), descs, vb_begin, n_reps, n_vblocks, ws, ncol, sp, sms,
-                          max_fields, st, tc, nslots);
+                          max_fields, st, tc, nslots, split);
 }
 
 void launch_time_corr(const ReplicaDesc* descs, int n_reps, int max_fields, const TimeCorr& tc, cudaStream_t st) {

@@ -18,7 +18,11 @@ void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_
                      int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms);
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
-                     int nslots, int max_fields, int max_len, int max_pairs, int sms);
+                     int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split);
+int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                      char* ws, cudaStream_t st, int paths, int slot, int max_len, int sms);
+void launch_pair_sums(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                      char* ws, int ncol, int max_fields, int nslots, cudaStream_t st, const TimeCorr& tc, int sms);
 void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                        int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
                        int paths, int slot, int sms);
@@ -117,9 +121,15 @@ int spectra_launch(int precision, SpectraPlan& P, char* scratch, const void* fie
     launch_fft_cols_a(precision, ddesc, vb + 1, 1, P.n_vb_cols_a, scratch, P.ncol, ga, kColsBlock, P.cols_smem, st,
                       cols16_b(1 << d.log2n1) ? cols16_b(1 << d.log2n1) : kColsGeneric, 0, sms);
   }
-  launch_fft_cols(precision, ddesc, vb + 2, 1, P.n_vb_cols, scratch, P.ncol, st, TimeCorr{},
-                  cols16_b(d.ny >> d.log2n1) ? cols16_b(d.ny >> d.log2n1) : kColsGeneric, 1, (int)d.n_fields,
-                  std::max(1 << d.log2n1, d.ny >> d.log2n1), d.n_pairs, sms);
+  const int paths = precision != FLB_FP64 && cols16_b(d.ny >> d.log2n1) ? cols16_b(d.ny >> d.log2n1) : kColsGeneric;
+  if (!d.log2n1 && (int64_t)d.ny * d.half_nx >= kSplitPoints) {
+    launch_fft_cols_t(precision, ddesc, vb + 2, 1, cols_t_blocks(d), scratch, st, paths, 0, d.ny, sms);
+    launch_pair_sums(precision, ddesc, vb + 2, 1, pair_blocks(d, P.ncol), scratch, P.ncol, (int)d.n_fields, 1, st,
+                     TimeCorr{}, sms);
+  } else {
+    launch_fft_cols(precision, ddesc, vb + 2, 1, P.n_vb_cols, scratch, P.ncol, st, TimeCorr{}, paths, 1,
+                    (int)d.n_fields, std::max(1 << d.log2n1, d.ny >> d.log2n1), d.n_pairs, sms, false);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return set_error(FLB_ECUDA, "spectra launch: %s", cudaGetErrorString(e));
   return FLB_OK;

@@ -285,7 +285,8 @@ k_fft_cols_a16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
 template <int B, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? cols_block_max(4) : kColsBlock, SPLIT ? 1 : FLB_ACC16_MIN_BLOCKS)
 k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
-                 int64_t n_vblocks, char* __restrict__ ws, int ncol, ColsSplit sp, TimeCorr tc, int nslots) {
+                 int64_t n_vblocks, char* __restrict__ ws, int ncol, ColsSplit sp, TimeCorr tc, int nslots,
+                 bool split) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* s = reinterpret_cast<float2*>(smem_raw);
   const int w = SPLIT ? sp.w : ncol, ps = SPLIT ? sp.ps : 1;
@@ -297,7 +298,7 @@ k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restric
     const int rp = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[rp];
     const int n2 = d.ny >> d.log2n1;
-    if (cols16_b(n2) != B) continue;
+    if (cols16_b(n2) != B || (split && !d.log2n1)) continue;
     const int tiles = (d.half_nx + ncol - 1) >> lc;
     const int64_t local = vb - vb_begin[rp];
     const int k1 = (int)(local / tiles);
@@ -309,6 +310,69 @@ k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restric
     cols_acc16_tile<B, SPLIT>(d, ws, s, rp, k1, kx0, min(w, d.half_nx - kx0), w, ncol, tiles, sub >> lsub, ps, tc,
                               nslots);
   }
+}
+
+// One-pass columns of length L in place (the split accumulation, spectra.cu): one unit per (replica,
+// field, tile of kColsT columns), stage 1 from the spectrum, stage 2 back to it; blocks of kT16Units
+// units keep a warp or more per unit length.
+template <int B>
+__global__ void __launch_bounds__(256)
+k_fft_cols_t16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
+               int64_t n_vblocks, char* __restrict__ ws, int slot) {
+  constexpr int L = 16 * B, SS = L + 1, QN = 16 / B, lc = log2_ct<kColsT>(), items = kColsT * B;
+  constexpr int U = 256 / items < 1 ? 1 : 256 / items;          // units of a block (items <= 256)
+  __shared__ float2 s[U * kColsT * SS];
+  __shared__ float2 wl[L];
+  const int u = threadIdx.x / items, i = threadIdx.x % items;
+  const int c = i & (kColsT - 1), r = i >> lc;
+  int cur = -1;
+  for (int64_t v = blockIdx.x; v * U < n_vblocks; v += gridDim.x) {
+    const int64_t vb = v * U + u;
+    const int rp = find_rep(vb_begin, n_reps, vb < n_vblocks ? vb : n_vblocks - 1);
+    const ReplicaDesc& d = descs[rp];
+    const int tiles = (d.half_nx + kColsT - 1) >> lc;
+    const int local = (int)(vb - vb_begin[rp]), f = local / tiles, kx0 = (local - f * tiles) << lc;
+    const bool act = vb < n_vblocks && !d.log2n1 && cols16_b(d.ny) == B && f < (int)d.n_fields;
+    // W_L depends on L alone
+    if (__syncthreads_or(act && cur < 0)) {
+      const int64_t v0 = v * U;
+      for (int k = 0; k < U && cur < 0; ++k) {              // the first unit of this length in the block
+        if (v0 + k >= n_vblocks) break;
+        const ReplicaDesc& dk = descs[find_rep(vb_begin, n_reps, v0 + k)];
+        if (dk.log2n1 || cols16_b(dk.ny) != B) continue;
+        fill_wl(wl, L, reinterpret_cast<const float2*>(ws + dk.off_tw_y), dk.ny);
+        cur = 0;
+      }
+      __syncthreads();
+    }
+    float2* col = reinterpret_cast<float2*>(ws + d.off_spec + slot * d.spec_slot) + (int64_t)f * d.ny * d.wpitch + kx0 + c;
+    const bool in = act && kx0 + c < d.half_nx;
+    float2* e = s + (u * kColsT + c) * SS;
+    if (act) stage1<B>(col + (int64_t)r * d.wpitch, (int64_t)B * d.wpitch, in && FLB_INB(r + B * 15 < d.ny, 211), e + r, wl, r);
+    __syncthreads();
+    if (act) {
+#pragma unroll
+      for (int qi = 0; qi < QN; ++qi) {
+        const int q = r * QN + qi;
+        float2 w8[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) w8[k] = e[q * B + k];
+        dft_reg<float, B>(w8);
+#pragma unroll
+        for (int p = 0; p < B; ++p)
+          if (in) col[(int64_t)(q + 16 * p) * d.wpitch] = w8[p];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+void launch_fft_cols_t16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
+                         char* ws, int grid, cudaStream_t st, int slot) {
+#define FLB_L(B) \
+  if (mask & B) k_fft_cols_t16<B><<<grid, kColsT * B < 256 ? 256 : kColsT * B, 0, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
+  FLB_L(1) FLB_L(2) FLB_L(4) FLB_L(8) FLB_L(16)
+#undef FLB_L
 }
 
 cudaError_t set_fft16_smem_limits() {
@@ -348,7 +412,7 @@ void launch_fft_cols_a16(int mask, const ReplicaDesc* descs, const int64_t* vb_b
 // with the shared memory of its column length (max_fields: the most fields of a replica)
 void launch_fft_cols_acc16(int mask, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
                            char* ws, int ncol, const ColsSplit& sp, int sms, int max_fields, cudaStream_t st,
-                           const TimeCorr& tc, int nslots) {
+                           const TimeCorr& tc, int nslots, bool split) {
   const int64_t nb = n_vblocks * (ncol / sp.w) * sp.ps;
   const int grid = (int)std::min<int64_t>(nb, 8 * (int64_t)sms);
 #define FLB_L(B)                                                                                            \
@@ -357,10 +421,10 @@ void launch_fft_cols_acc16(int mask, const ReplicaDesc* descs, const int64_t* vb
     const int block = cols_threads(nb, sms, sp.w * 16 * B, smem);                                           \
     if (sp.w == ncol && sp.ps == 1 && block == kColsBlock && sp.w * 16 * B >= kColsBlock)                   \
       k_fft_cols_acc16<B, false><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol,   \
-                                                            sp, tc, nslots);                                \
+                                                            sp, tc, nslots, split);                         \
     else                                                                                                    \
       k_fft_cols_acc16<B, true><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, ncol,    \
-                                                           sp, tc, nslots);                                 \
+                                                           sp, tc, nslots, split);                          \
   }
   FLB_L(1) FLB_L(2) FLB_L(4) FLB_L(8) FLB_L(16)
 #undef FLB_L
