@@ -317,6 +317,7 @@ constexpr int kColsA16 = 16;
 // 256); the shared-memory kernels keep the row-major layout.
 constexpr int kSpecTile = 16;
 static_assert(kColsA16 == kSpecTile, "a pass-2a tile is one spectrum tile");
+static_assert(kSpecTile % kColsT == 0, "a transform tile lies within a spectrum tile");
 // element (f, y, kx) of a spectrum slot, the distance between rows y, y + 1, and the
 // complex elements of a slot
 __host__ __device__ __forceinline__ int64_t spec_index(const ReplicaDesc& d, int f, int y, int kx) {

@@ -331,7 +331,8 @@ k_pair_sums(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ v
     const int F = (int)d.n_fields, hn = d.half_nx, ny = d.ny;
     const int64_t pt = (vb - vb_begin[r]) * kColsBlock + threadIdx.x;
     const C<R>* spec = reinterpret_cast<const C<R>*>(ws + d.off_spec);
-    const int64_t fplane = (int64_t)ny * d.wpitch, slot = d.spec_slot / (int64_t)sizeof(C<R>);
+    // (either spectrum layout, spec_index)
+    const int64_t fplane = spec_index(d, 1, 0, 0), slot = d.spec_slot / (int64_t)sizeof(C<R>);
     if (vb == vb_begin[r] && grp == 0) {
       if (tc.base) {
         const int rs = (int)(tc.count[r] % (uint64_t)tc.n_lags);
@@ -339,7 +340,7 @@ k_pair_sums(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ v
         for (int i = threadIdx.x; i < tc.n_k * F; i += blockDim.x) {
           const int j = i % tc.n_k, f = i / tc.n_k;
           if (!FLB_INB(tc.kx[j] < hn && tc.ky[j] < ny, 164)) continue;
-          const C<R> X = spec[f * fplane + (int64_t)tc.ky[j] * d.wpitch + tc.kx[j]];
+          const C<R> X = spec[spec_index(d, f, tc.ky[j], tc.kx[j])];
           ring[((int64_t)rs * F + f) * tc.n_k + j] = make_double2((double)X.x, (double)X.y);
         }
       }
@@ -366,7 +367,7 @@ k_pair_sums(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ v
       in = ky < ny;
     }
     if (!in || !FLB_INB(ky < ny && kx < d.wpitch && pt < sum_limit(d, ncol, (hn + ncol - 1) / ncol), 165)) continue;
-    const C<R>* p = spec + (int64_t)ky * d.wpitch + kx;
+    const C<R>* p = spec + spec_index(d, 0, ky, kx);
     C<R> X0[FM], X1[FM];
 #pragma unroll
     for (int f = 0; f < FM; ++f)

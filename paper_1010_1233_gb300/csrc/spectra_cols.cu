@@ -345,10 +345,12 @@ k_fft_cols_t16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
       }
       __syncthreads();
     }
-    float2* col = reinterpret_cast<float2*>(ws + d.off_spec + slot * d.spec_slot) + (int64_t)f * d.ny * d.wpitch + kx0 + c;
+    // (either spectrum layout: a tile of kColsT columns lies within one of kSpecTile)
+    const int rs = spec_row_stride(d);
+    float2* col = reinterpret_cast<float2*>(ws + d.off_spec + slot * d.spec_slot) + spec_index(d, f, 0, kx0) + c;
     const bool in = act && kx0 + c < d.half_nx;
     float2* e = s + (u * kColsT + c) * SS;
-    if (act) stage1<B>(col + (int64_t)r * d.wpitch, (int64_t)B * d.wpitch, in && FLB_INB(r + B * 15 < d.ny, 211), e + r, wl, r);
+    if (act) stage1<B>(col + (int64_t)r * rs, (int64_t)B * rs, in && FLB_INB(r + B * 15 < d.ny, 211), e + r, wl, r);
     __syncthreads();
     if (act) {
 #pragma unroll
@@ -360,7 +362,7 @@ k_fft_cols_t16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
         dft_reg<float, B>(w8);
 #pragma unroll
         for (int p = 0; p < B; ++p)
-          if (in) col[(int64_t)(q + 16 * p) * d.wpitch] = w8[p];
+          if (in) col[(int64_t)(q + 16 * p) * rs] = w8[p];
       }
     }
     __syncthreads();

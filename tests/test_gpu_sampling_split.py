@@ -1,6 +1,7 @@
 """Sampling passes at the edges of their block split (GPU): groups of row pairs that do not fill
 a block, one field of one row, column tiles past the last column, tiles cut down to single
-sectors and field pairs dealt to several blocks, against numpy's FFT in FP64.
+sectors and field pairs dealt to several blocks, one-pass columns of the column-tiled spectrum,
+against numpy's FFT in FP64.
 
 Tolerance: a transform of V points has a relative error of ~log2(V) roundings in the root
 mean square over its points; products double it: 4 log2(V) eps of the largest sum."""
@@ -16,7 +17,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("F,ny,nx", [(1, 1, 2), (1, 2, 4), (3, 1, 8), (1, 8, 16), (5, 2, 256), (9, 256, 256),
-                                     (2, 64, 512), (11, 32, 64), (3, 1, 2048), (3, 1024, 64), (1, 4, 1024)])
+                                     (2, 64, 512), (11, 32, 64), (3, 1, 2048), (3, 1024, 64), (1, 4, 1024),
+                                     (3, 64, 4096), (2, 256, 4096), (2, 16, 8192)])
 def test_pair_sums_match_fft(precision, F, ny, nx):
     dt, eps = (torch.float64, 2.0 ** -53) if precision == "fp64" else (torch.float32, 2.0 ** -24)
     x = torch.tensor(W.random_perturbation((F, ny, nx), F + ny + nx), dtype=dt, device="cuda")
