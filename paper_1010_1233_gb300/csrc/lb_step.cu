@@ -84,13 +84,20 @@ k_step_d2q9(const ReplicaDesc* __restrict__ descs, const __grid_constant__ Repli
 // have it in the constant bank.  Blocks may be smaller than the kStepThreads units of a virtual
 // block (blockDim = kStepThreads >> split), so that a small lattice reaches more SMs.
 // Fields are stored pair by pair where sampled (their slots follow from the field mask).
-template <int VEC, bool SAMPLE, int FL>
+//
+// EARLY (lattices of at most one unit per thread on the GPU at once): the launch may start while the
+// step before still runs (programmatic dependent launch).  The thread's normals, which depend on
+// nothing but the step, are drawn first; then it waits for the step before and pulls, with loads
+// past L1.  A step of such a lattice is launch latency and one thread's chain: us per step
+// without and with EARLY, 64^2 2.1 -> 1.4, 256^2 2.6 -> 1.9, 512^2 4.9 -> 3.35 (the largest, 4 blocks on each SM).
+template <int VEC, bool SAMPLE, int FL, bool EARLY>
 __global__ void __launch_bounds__(kStepThreads, VEC == 4 ? 3 : 4)
 k_step_d2q9_pair(const ReplicaDesc* __restrict__ descs, const __grid_constant__ ReplicaDesc one,
                  const int64_t* __restrict__ vb_begin, int n_reps, int64_t n_vblocks, char* __restrict__ ws,
                  int parity, uint32_t step, const uint64_t* __restrict__ step_dev, int split) {
   constexpr bool ONE = Flavor<FL>::kOne;
   __shared__ uint4 head[ONE ? 1 : kStepHeadBytes / 16];
+  if constexpr (EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (step_dev) {                  // graph replay: step = device base + offset
     const uint64_t t = *step_dev + step;
     step = (uint32_t)t;
@@ -117,10 +124,22 @@ k_step_d2q9_pair(const ReplicaDesc* __restrict__ descs, const __grid_constant__ 
     const int64_t plane = (int64_t)d.nx * d.ny;
     const float* __restrict__ src = reinterpret_cast<const float*>(ws + d.off_pop[parity]);
     float* __restrict__ dst = reinterpret_cast<float*>(ws + d.off_pop[parity ^ 1]);
-    float f[9][VEC];
-    pull_d2q9<float, VEC>(src, plane, d.nx, d.ny, u, f);
-    const float rho0 = coef<float>(d, kCoRho0);
     const bool noisy = d.noise_mask != 0;
+    float2 early[EARLY ? VEC / 2 : 1][6] = {};
+    if constexpr (EARLY) {
+      if (noisy) {
+#pragma unroll
+        for (int p = 0; p < VEC / 2; ++p) {
+          uint4 w0a, w1a, w0b, w1b;
+          philox_words_pair(d, (uint32_t)u.y * (uint32_t)d.nx + (uint32_t)(u.x0 + 2 * p), step, w0a, w1a, w0b, w1b);
+          normals_pair(w0a, w1a, w0b, w1b, early[p]);
+        }
+      }
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+    float f[9][VEC];
+    pull_d2q9<float, VEC, EARLY>(src, plane, d.nx, d.ny, u, f);
+    const float rho0 = coef<float>(d, kCoRho0);
     const bool in = u.active && FLB_INB(u.y >= 0 && u.y < d.ny && u.x0 >= 0 && u.x0 + VEC <= d.nx, 103);
     const int64_t off = (int64_t)u.y * d.nx + u.x0;
 #pragma unroll
@@ -141,7 +160,10 @@ k_step_d2q9_pair(const ReplicaDesc* __restrict__ descs, const __grid_constant__ 
         }
       }
       float2 n[6] = {};
-      if (noisy) {
+      if constexpr (EARLY) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) n[c] = early[p][c];
+      } else if (noisy) {
         uint4 w0a, w1a, w0b, w1b;
         philox_words_pair(d, (uint32_t)u.y * (uint32_t)d.nx + (uint32_t)(u.x0 + 2 * p), step, w0a, w1a, w0b, w1b);
         normals_pair(w0a, w1a, w0b, w1b, n);
@@ -334,8 +356,29 @@ static void launch_d2q9_vec(const StepLaunch& L, bool sample, bool mlp, cudaStre
   if constexpr (VEC >= 2) {
     // a lattice too small for a block of kStepThreads per SM: blocks of a quarter of that
     const int split = L.n_vblocks < L.sms ? 2 : 0;
-    const int grid = (int)std::min<int64_t>(L.n_vblocks << split, (int64_t)L.grid << split);
-#define FLB_L(S, F) k_step_d2q9_pair<VEC, S, F><<<grid, kStepThreads >> split, 0, st>>>( \
+    const int64_t units = L.n_vblocks << split;
+    const int grid = (int)std::min<int64_t>(units, (int64_t)L.grid << split);
+    // one unit per thread, all resident at once beside the step before: launched early
+    if (VEC == 2 && grid == units && L.n_vblocks <= 4 * (int64_t)L.sms) {
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at[0].val.programmaticStreamSerializationAllowed = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(grid);
+      cfg.blockDim = dim3(kStepThreads >> split);
+      cfg.stream = st;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+#define FLB_L(S, F) cudaLaunchKernelEx(&cfg, k_step_d2q9_pair<VEC, S, F, true>, L.descs, *L.desc0, L.vb_begin, \
+                                       L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
+#define FLB_LF(F) { if (sample) FLB_L(true, F); else FLB_L(false, F); }
+      const int fl = L.flavor();
+      if constexpr (VEC == 2) { if (fl == 0) FLB_LF(0) else if (fl == 1) FLB_LF(1) else FLB_LF(2) }
+      return;
+#undef FLB_LF
+#undef FLB_L
+    }
+#define FLB_L(S, F) k_step_d2q9_pair<VEC, S, F, false><<<grid, kStepThreads >> split, 0, st>>>( \
       L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
 #define FLB_LF(F) { if (sample) FLB_L(true, F); else FLB_L(false, F); }
     const int fl = L.flavor();

@@ -51,6 +51,15 @@ __device__ __forceinline__ void block_sums(double (&acc)[kNumSums], double* __re
 }
 
 template <typename R, int VEC> struct VecIO;
+// loads past L1, for state that a kernel still running at this kernel's launch may write
+template <int VEC> __device__ __forceinline__ void ld_l2(const float* p, float (&v)[VEC]) {
+  if constexpr (VEC == 1) v[0] = __ldcg(p);
+  else if constexpr (VEC == 2) { const float2 t = __ldcg(reinterpret_cast<const float2*>(p)); v[0] = t.x; v[1] = t.y; }
+  else {
+    const float4 t = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+  }
+}
 template <> struct VecIO<float, 1> {
   static __device__ __forceinline__ void ld(const float* p, float (&v)[1]) { v[0] = __ldg(p); }
   static __device__ __forceinline__ void st(float* p, const float (&v)[1]) { *p = v[0]; }
@@ -117,7 +126,7 @@ struct PullRaw {
 __host__ __device__ constexpr int vel_x(int i) { return i == 1 || i == 5 || i == 8 ? 1 : (i == 3 || i == 6 || i == 7 ? -1 : 0); }
 __host__ __device__ constexpr int vel_y(int i) { return i == 2 || i == 5 || i == 6 ? 1 : (i == 4 || i == 7 || i == 8 ? -1 : 0); }
 
-template <typename R, int VEC>
+template <typename R, int VEC, bool L2 = false>
 __device__ __forceinline__ void pull_issue(const R* __restrict__ src, int64_t plane, int nx, int ny, const UnitPos& u,
                                            PullRaw<R, VEC>& raw) {
   const int x0 = u.x0;
@@ -126,17 +135,20 @@ __device__ __forceinline__ void pull_issue(const R* __restrict__ src, int64_t pl
     int ys = u.y - vel_y(i);
     ys = ys < 0 ? ys + ny : (ys >= ny ? ys - ny : ys);
     const R* row = src + i * plane + (int64_t)ys * nx;
-    if (FLB_INB(ys >= 0 && ys < ny && x0 >= 0 && x0 + VEC <= nx, 101)) VecIO<R, VEC>::ld(row + x0, raw.v[i]);
+    if (FLB_INB(ys >= 0 && ys < ny && x0 >= 0 && x0 + VEC <= nx, 101)) {
+      if constexpr (L2) ld_l2<VEC>(row + x0, raw.v[i]);
+      else VecIO<R, VEC>::ld(row + x0, raw.v[i]);
+    }
 #ifdef FLB_CHECK_BOUNDS
     else for (int s = 0; s < VEC; ++s) raw.v[i][s] = (R)0;
 #endif
     raw.e[i] = (R)0;
     if (vel_x(i) == 1) {                          // needs x0 - 1
       const int xe = x0 == 0 ? nx - 1 : x0 - 1;
-      if (!u.left_in_warp && FLB_INB(xe >= 0 && xe < nx, 102)) raw.e[i] = __ldg(row + xe);
+      if (!u.left_in_warp && FLB_INB(xe >= 0 && xe < nx, 102)) raw.e[i] = L2 ? __ldcg(row + xe) : __ldg(row + xe);
     } else if (vel_x(i) == -1) {                  // needs x0 + VEC
       const int xe = x0 + VEC == nx ? 0 : x0 + VEC;
-      if (!u.right_in_warp && FLB_INB(xe >= 0 && xe < nx, 102)) raw.e[i] = __ldg(row + xe);
+      if (!u.right_in_warp && FLB_INB(xe >= 0 && xe < nx, 102)) raw.e[i] = L2 ? __ldcg(row + xe) : __ldg(row + xe);
     }
   }
 }
@@ -163,11 +175,11 @@ __device__ __forceinline__ void pull_finish(const PullRaw<R, VEC>& raw, const Un
   }
 }
 
-template <typename R, int VEC>
+template <typename R, int VEC, bool L2 = false>
 __device__ __forceinline__ void pull_d2q9(const R* __restrict__ src, int64_t plane, int nx, int ny, const UnitPos& u,
                                           R (&f)[9][VEC]) {
   PullRaw<R, VEC> raw;
-  pull_issue<R, VEC>(src, plane, nx, ny, u, raw);
+  pull_issue<R, VEC, L2>(src, plane, nx, ny, u, raw);
   pull_finish<R, VEC>(raw, u, f);
 }
 
