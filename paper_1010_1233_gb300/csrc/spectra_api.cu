@@ -10,7 +10,6 @@
 
 namespace flb {
 
-void launch_twiddles(int precision, void* tw, int n, cudaStream_t st);
 int fft_rows_smem(int precision, int nx);
 int fft_cols_smem(int precision, int F, int ny, int ncol);
 cudaError_t set_fft_smem_limits();
@@ -79,13 +78,27 @@ int spectra_plan(int precision, int nx, int ny, int F, SpectraPlan& P) {
   return FLB_OK;
 }
 
-// One thread stores the plan's descriptor and block tables into device memory, so no
-// host-to-device copy (and no host staging buffer) is involved.
-__global__ void k_store_plan(ReplicaDesc d, ReplicaDesc* dst, int64_t* vb) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    *dst = d;
-    vb[0] = 0; vb[1] = 0; vb[2] = 0;
+// One launch prepares a call: block 0 stores the plan's descriptor and block tables (so no
+// host-to-device copy and no host staging buffer is involved), the others the twiddle tables
+// exp(-2 pi i m / n), m < n / 2, of nx and ny.
+template <typename R>
+__global__ void __launch_bounds__(256) k_store_plan(const __grid_constant__ ReplicaDesc d, ReplicaDesc* dst, int64_t* vb) {
+  if (blockIdx.x == 0) {
+    const uint4* src = reinterpret_cast<const uint4*>(&d);
+    for (int i = threadIdx.x; i < (int)(sizeof(ReplicaDesc) / 16); i += blockDim.x) reinterpret_cast<uint4*>(dst)[i] = src[i];
+    if (threadIdx.x < 3) vb[threadIdx.x] = 0;
+    return;
   }
+  char* base = reinterpret_cast<char*>(dst);              // offsets are relative to the scratch
+  const int hx = d.nx / 2, hy = d.ny / 2;
+  const int m = ((int)blockIdx.x - 1) * (int)blockDim.x + (int)threadIdx.x;
+  if (m >= hx + hy) return;
+  cplx<R>* tw = reinterpret_cast<cplx<R>*>(base + (m < hx ? d.off_tw_x : d.off_tw_y));
+  const int k = m < hx ? m : m - hx, n = m < hx ? d.nx : d.ny;
+  double sn, cs;
+  sincospi(2.0 * (double)k / (double)n, &sn, &cs);
+  tw[k].x = (R)cs;
+  tw[k].y = (R)(-sn);
 }
 
 int spectra_launch(int precision, SpectraPlan& P, char* scratch, const void* fields, double* pair_sums,
@@ -105,11 +118,11 @@ int spectra_launch(int precision, SpectraPlan& P, char* scratch, const void* fie
   }
   cudaError_t e = set_fft_smem_limits();
   if (e != cudaSuccess) return set_error(FLB_ECUDA, "smem limits: %s", cudaGetErrorString(e));
-  ReplicaDesc* ddesc = reinterpret_cast<ReplicaDesc*>(scratch + P.off_desc);
+  ReplicaDesc* ddesc = reinterpret_cast<ReplicaDesc*>(scratch + P.off_desc);     // (off_desc = 0: the scratch's start)
   int64_t* vb = reinterpret_cast<int64_t*>(scratch + P.off_vb);
-  k_store_plan<<<1, 32, 0, st>>>(d, ddesc, vb);
-  launch_twiddles(precision, scratch + P.off_tw_x, d.nx, st);
-  launch_twiddles(precision, scratch + P.off_tw_y, d.ny, st);
+  const int prep = 1 + (d.nx / 2 + d.ny / 2 + 255) / 256;
+  if (precision == FLB_FP64) k_store_plan<double><<<prep, 256, 0, st>>>(d, ddesc, vb);
+  else k_store_plan<float><<<prep, 256, 0, st>>>(d, ddesc, vb);
   int sms = 1, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
