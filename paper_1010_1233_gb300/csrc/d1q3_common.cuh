@@ -49,15 +49,14 @@ __device__ __forceinline__ double widen64(float x) {
   return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
-// out of line: inlined, its FP64 instructions are issued ahead of the branch that needs them
+// out of line, like divide64
 static __device__ __noinline__ double d1q3_sqrt(double a) { return sqrt(a); }
-static __device__ __noinline__ double d1q3_divide(double a, double b) { return a / b; }
 
 // q / rho, rho = g0 + s.  The estimate needs populations and their FP32 sum of ordinary size (and
 // a sum without cancellation, so that it is good to 22 bits); anything else divides.
 __device__ __forceinline__ double d1q3_quotient(double q, double rho, double g0, double g1, double g2) {
   const float f = narrow64(g0) + (narrow64(g1) + narrow64(g2));
-  if (!(ordinary64(g0) && ordinary64(g1) && ordinary64(g2))) return d1q3_divide(q, rho);
+  if (!(ordinary64(g0) && ordinary64(g1) && ordinary64(g2))) return divide64(q, rho);
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f));
   const double y0 = widen64(y);

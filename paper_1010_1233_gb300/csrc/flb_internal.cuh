@@ -180,6 +180,25 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, 
   n1 = nr * sin_approx(th);
 }
 
+// 1 / a in FP64: the hardware's FP32 reciprocal of a (22 bits) and one third-order step y (1 + e + e^2),
+// e = 1 - a y (e^3 < 2^-63): three FP64 instructions, where a division takes about ten and GB300
+// issues one of a warp every 64 cycles.  Narrowing and widening run on the integer pipes.  Magnitudes
+// outside 2^-100 .. 2^100 and non-finite values divide, out of line (inlined, the division's
+// instructions are issued ahead of the branch).
+static __device__ __noinline__ double divide64(double a, double b) { return a / b; }
+__device__ __forceinline__ double recip(double a) {
+  const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
+  if ((hi & 0x7FFFFFFFu) - ((1023u - 100u) << 20) >= (200u << 20)) return divide64(1.0, a);
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y)
+      : "f"(__uint_as_float((hi & 0x80000000u) | (((hi & 0x7FFFFFFFu) - 0x38000000u) << 3) | (lo >> 29))));
+  const uint32_t b = __float_as_uint(y);
+  const double y0 = __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+  const double e = __fma_rn(-a, y0, 1.0);
+  return __fma_rn(y0, __fma_rn(e, e, e), y0);
+}
+__device__ __forceinline__ float recip(float a) { return 1.f / a; }
+
 template <typename T> struct cplx { T x, y; };
 template <typename T> struct vec2_of;
 template <> struct vec2_of<float> { using type = float2; };
@@ -227,6 +246,11 @@ struct StepLaunch {
   // kernel flavour: 0 = one replica, noise mode 0; 1 = one replica, any mode; 2 = batched
   int flavor() const { return n_reps > 1 ? 2 : (noise_general ? 1 : 0); }
 };
+// Blocks of a quarter of a virtual block where a launch has few of them: with one to eight blocks of
+// kStepThreads per SM some SMs get one more than others.  FP64, whose pipe is the bound, us per step
+// (with recip's shorter reciprocal): D2Q9 256^2 (256 blocks, two on some SMs and one on others) 21.5 ->
+// 19.7, D3Q15 64 x 48 x 40 (480 blocks) 62 -> 57.
+inline int step_split(int64_t n_vblocks, int sms) { return n_vblocks < 8 * (int64_t)sms ? 2 : 0; }
 // flavour -> (descriptor in the constant bank, noise modes 1/2 compiled)
 template <int FL> struct Flavor { static constexpr bool kOne = FL != 2, kGen = FL != 0; };
 

@@ -112,7 +112,7 @@ __device__ __forceinline__ void collide_d3q15(const ReplicaDesc& d, R (&g)[15], 
   const R cx = (d1 + d2) + (d3 - d4), cy = (d1 + d2) - (d3 - d4), cz = (d1 - d2) + (d3 + d4);
   const R jx = (g[1] - g[2]) + cx, jy = (g[3] - g[4]) + cy, jz = (g[5] - g[6]) + cz;
   const R rho = DEV ? coef<R>(d, kCoRho0) + sum : sum;
-  const R irho = (R)1 / rho;
+  const R irho = recip(rho);
   const R ux = jx * irho, uy = jy * irho, uz = jz * irho;
   // non-conserved moments
   const R M4 = (R)1.5 * (ax - ay);
@@ -207,7 +207,7 @@ __device__ __forceinline__ void collide_d3q19(const ReplicaDesc& d, R (&g)[19], 
   const R cx = (dA + dB) + (dC + dD), cy = (dA - dB) + (dE + dF), cz = (dC - dD) + (dE - dF);
   const R jx = ox + cx, jy = oy + cy, jz = oz + cz;
   const R rho = DEV ? coef<R>(d, kCoRho0) + sum : sum;
-  const R irho = (R)1 / rho;
+  const R irho = recip(rho);
   const R ux = jx * irho, uy = jy * irho, uz = jz * irho;
   // non-conserved moments
   const R dxy = ax - ay, sxz = Sxz - Syz, pxy = ax + ay, t5 = (R)2 * Sxy - (Sxz + Syz);
@@ -331,16 +331,20 @@ template <int Q, typename R, bool DEV, int VEC, bool SAMPLE, bool ONE>
 __global__ void __launch_bounds__(kStepThreads, FLB_STEP3_MINB)
 k_step_3d(const ReplicaDesc* __restrict__ descs, const __grid_constant__ ReplicaDesc one,
           const int64_t* __restrict__ vb_begin, int n_reps, int64_t n_vblocks, char* __restrict__ ws, int parity,
-          uint32_t step, const uint64_t* __restrict__ step_dev) {
+          uint32_t step, const uint64_t* __restrict__ step_dev, int split) {
   if (step_dev) {
     const uint64_t t = *step_dev + step;
     step = (uint32_t)t;
     parity = (int)(t & 1);
   }
-  for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
+  if (sizeof(R) == 4) split = 0;               // (FP64 only; the index arithmetic costs the FP32 kernels 1 %)
+  for (int64_t h = blockIdx.x; h < n_vblocks << split; h += gridDim.x) {
+    const int64_t vb = h >> split;
+    const int tid = sizeof(R) == 4 ? (int)threadIdx.x
+                                   : (int)(h & ((1 << split) - 1)) * (int)blockDim.x + (int)threadIdx.x;
     const int r = ONE ? 0 : find_replica(vb_begin, n_reps, vb);
     const ReplicaDesc& d = ONE ? one : descs[r];
-    const UnitPos u = unit_position(d, vb, ONE ? 0 : vb_begin[r], (int)threadIdx.x, kStepThreads, VEC);
+    const UnitPos u = unit_position(d, vb, ONE ? 0 : vb_begin[r], tid, kStepThreads, VEC);
     const int row = u.y;                       // z ny + y
     const int z = row / d.ny, y = row - z * d.ny;
     const int64_t vol = (int64_t)d.nx * d.ny * d.nz;
@@ -655,8 +659,10 @@ void launch_finish_sums(const double* partial, int nblocks, double* sums, DevSta
 template <int Q>
 static void launch_step3_q(int precision, int vec, const StepLaunch& L, bool sample, cudaStream_t st) {
   const bool one = L.n_reps == 1;
-#define FLB_L3(R, DEV, V, S, O) k_step_3d<Q, R, DEV, V, S, O><<<L.grid, kStepThreads, 0, st>>>( \
-      L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev)
+  const int split = precision == FLB_FP64 ? step_split(L.n_vblocks, L.sms) : 0;
+  const int grid = (int)std::min<int64_t>(L.n_vblocks << split, (int64_t)L.grid << split);
+#define FLB_L3(R, DEV, V, S, O) k_step_3d<Q, R, DEV, V, S, O><<<grid, kStepThreads >> split, 0, st>>>( \
+      L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
 #define FLB_LS(R, DEV, V) { \
     if (one) { if (sample) FLB_L3(R, DEV, V, true, true); else FLB_L3(R, DEV, V, false, true); } \
     else { if (sample) FLB_L3(R, DEV, V, true, false); else FLB_L3(R, DEV, V, false, false); } }

@@ -29,17 +29,19 @@ template <typename R, bool DEV, int VEC, bool SAMPLE, int FL>
 __global__ void __launch_bounds__(kStepThreads, FLB_STEP_MINB_PLAIN)
 k_step_d2q9(const ReplicaDesc* __restrict__ descs, const __grid_constant__ ReplicaDesc one,
             const int64_t* __restrict__ vb_begin, int n_reps, int64_t n_vblocks, char* __restrict__ ws, int parity,
-            uint32_t step, const uint64_t* __restrict__ step_dev) {
+            uint32_t step, const uint64_t* __restrict__ step_dev, int split) {
   constexpr bool ONE = Flavor<FL>::kOne;
   if (step_dev) {                  // graph replay: step = device base + offset
     const uint64_t t = *step_dev + step;
     step = (uint32_t)t;
     parity = (int)(t & 1);
   }
-  for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
+  for (int64_t h = blockIdx.x; h < n_vblocks << split; h += gridDim.x) {
+    const int64_t vb = h >> split;
+    const int tid = (int)(h & ((1 << split) - 1)) * (int)blockDim.x + (int)threadIdx.x;
     const int r = ONE ? 0 : find_replica(vb_begin, n_reps, vb);
     const ReplicaDesc& d = ONE ? one : descs[r];
-    const UnitPos u = unit_position(d, vb, ONE ? 0 : vb_begin[r], (int)threadIdx.x, kStepThreads, VEC);
+    const UnitPos u = unit_position(d, vb, ONE ? 0 : vb_begin[r], tid, kStepThreads, VEC);
     const int64_t plane = (int64_t)d.nx * d.ny;
     const R* __restrict__ src = reinterpret_cast<const R*>(ws + d.off_pop[parity]);
     R* __restrict__ dst = reinterpret_cast<R*>(ws + d.off_pop[parity ^ 1]);
@@ -387,8 +389,10 @@ static void launch_d2q9_vec(const StepLaunch& L, bool sample, bool mlp, cudaStre
 #undef FLB_LF
 #undef FLB_L
   } else {
-#define FLB_L(S, F) k_step_d2q9<R, DEV, VEC, S, F><<<L.grid, kStepThreads, 0, st>>>( \
-      L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev)
+  const int split = step_split(L.n_vblocks, L.sms);
+  const int grid = (int)std::min<int64_t>(L.n_vblocks << split, (int64_t)L.grid << split);
+#define FLB_L(S, F) k_step_d2q9<R, DEV, VEC, S, F><<<grid, kStepThreads >> split, 0, st>>>( \
+      L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
 #define FLB_LF(F) { if (sample) FLB_L(true, F); else FLB_L(false, F); }
   const int fl = L.flavor();
   if (fl == 0) FLB_LF(0) else if (fl == 1) FLB_LF(1) else FLB_LF(2)

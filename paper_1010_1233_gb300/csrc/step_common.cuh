@@ -206,7 +206,7 @@ template <> struct Lane<double> {
   static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
   static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
   static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
-  static __device__ __forceinline__ double rcp(double a) { return 1.0 / a; }
+  static __device__ __forceinline__ double rcp(double a) { return recip(a); }
   static __device__ __forceinline__ double sqrt_ratio(double a, double b) { return sqrt(a / b); }
 };
 // Packed operations as inline PTX with the rounding mode spelled out (.rn): an operation
