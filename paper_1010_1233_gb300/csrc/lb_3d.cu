@@ -50,7 +50,7 @@ namespace flb {
 // Pull streaming f_i(x) = f*_i(x - v_i) on the periodic box: the source row of population
 // i is (y - v_iy, z - v_iz); the x shift is taken by warp shuffle from the adjacent lane,
 // with one extra load at warp and row edges (as in the D2Q9 kernels).
-template <int Q, typename R, int VEC>
+template <int Q, typename R, int VEC, bool L2 = false>
 __device__ __forceinline__ void pull_3d(const R* __restrict__ src, int64_t vol, int nx, int ny, int nz, int y, int z,
                                         const UnitPos& u, R (&f)[Q][VEC]) {
   R v[Q][VEC], e[Q];
@@ -61,18 +61,20 @@ __device__ __forceinline__ void pull_3d(const R* __restrict__ src, int64_t vol, 
     ys = ys < 0 ? ys + ny : (ys >= ny ? ys - ny : ys);
     zs = zs < 0 ? zs + nz : (zs >= nz ? zs - nz : zs);
     const R* row = src + i * vol + ((int64_t)zs * ny + ys) * nx;
-    if (FLB_INB(ys >= 0 && ys < ny && zs >= 0 && zs < nz && x0 >= 0 && x0 + VEC <= nx, 171))
-      VecIO<R, VEC>::ld(row + x0, v[i]);
+    if (FLB_INB(ys >= 0 && ys < ny && zs >= 0 && zs < nz && x0 >= 0 && x0 + VEC <= nx, 171)) {
+      if constexpr (L2) ld_l2<VEC>(row + x0, v[i]);
+      else VecIO<R, VEC>::ld(row + x0, v[i]);
+    }
 #ifdef FLB_CHECK_BOUNDS
     else for (int s = 0; s < VEC; ++s) v[i][s] = (R)0;
 #endif
     e[i] = (R)0;
     if (v3x<Q>(i) == 1) {
       const int xe = x0 == 0 ? nx - 1 : x0 - 1;
-      if (!u.left_in_warp && FLB_INB(xe >= 0 && xe < nx, 172)) e[i] = __ldg(row + xe);
+      if (!u.left_in_warp && FLB_INB(xe >= 0 && xe < nx, 172)) e[i] = L2 ? __ldcg(row + xe) : __ldg(row + xe);
     } else if (v3x<Q>(i) == -1) {
       const int xe = x0 + VEC == nx ? 0 : x0 + VEC;
-      if (!u.right_in_warp && FLB_INB(xe >= 0 && xe < nx, 172)) e[i] = __ldg(row + xe);
+      if (!u.right_in_warp && FLB_INB(xe >= 0 && xe < nx, 172)) e[i] = L2 ? __ldcg(row + xe) : __ldg(row + xe);
     }
   }
 #pragma unroll
@@ -327,8 +329,10 @@ __device__ __forceinline__ void normals_3d(const ReplicaDesc& d, uint32_t site, 
 // One thread = VEC consecutive sites of a row (y, z); a persistent grid loops over virtual
 // blocks of kStepThreads units, each within one replica.  ONE: a single replica whose
 // description is the kernel argument (constant bank).
-template <int Q, typename R, bool DEV, int VEC, bool SAMPLE, bool ONE>
-__global__ void __launch_bounds__(kStepThreads, FLB_STEP3_MINB)
+// EARLY (FP64, one unit per thread): launched while the step before runs, normals first
+// (k_step_d2q9): D3Q15 64 x 48 x 40 55 -> 45 us.
+template <int Q, typename R, bool DEV, int VEC, bool SAMPLE, bool ONE, bool EARLY = false>
+__global__ void __launch_bounds__(EARLY ? kEarlyThreads : kStepThreads, EARLY ? kEarlyBlocks3 : FLB_STEP3_MINB)
 k_step_3d(const ReplicaDesc* __restrict__ descs, const __grid_constant__ ReplicaDesc one,
           const int64_t* __restrict__ vb_begin, int n_reps, int64_t n_vblocks, char* __restrict__ ws, int parity,
           uint32_t step, const uint64_t* __restrict__ step_dev, int split) {
@@ -350,9 +354,16 @@ k_step_3d(const ReplicaDesc* __restrict__ descs, const __grid_constant__ Replica
     const int64_t vol = (int64_t)d.nx * d.ny * d.nz;
     const R* __restrict__ src = reinterpret_cast<const R*>(ws + d.off_pop[parity]);
     R* __restrict__ dst = reinterpret_cast<R*>(ws + d.off_pop[parity ^ 1]);
-    R f[Q][VEC];
-    pull_3d<Q, R, VEC>(src, vol, d.nx, d.ny, d.nz, y, z, u, f);
     const bool noisy = d.noise_mask != 0;
+    R early[EARLY ? Q - 4 : 1] = {};
+    if constexpr (EARLY) {
+      static_assert(VEC == 1, "one site per thread");
+      if (noisy) normals_3d<Q, R>(d, (uint32_t)row * (uint32_t)d.nx + (uint32_t)u.x0, step, early);
+      // the step after this one is let in only now, so that two steps at most share the SMs
+      asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+    }
+    R f[Q][VEC];
+    pull_3d<Q, R, VEC, EARLY>(src, vol, d.nx, d.ny, d.nz, y, z, u, f);
     const int64_t off = (int64_t)row * d.nx + u.x0;
     R* fields = SAMPLE ? reinterpret_cast<R*>(ws + d.off_fields) : nullptr;
 #pragma unroll
@@ -363,7 +374,12 @@ k_step_3d(const ReplicaDesc* __restrict__ descs, const __grid_constant__ Replica
       R n[Q - 4];
 #pragma unroll
       for (int c = 0; c < Q - 4; ++c) n[c] = (R)0;
-      if (noisy) normals_3d<Q, R>(d, (uint32_t)row * (uint32_t)d.nx + (uint32_t)(u.x0 + s), step, n);
+      if constexpr (EARLY) {
+#pragma unroll
+        for (int c = 0; c < Q - 4; ++c) n[c] = early[c];
+      } else if (noisy) {
+        normals_3d<Q, R>(d, (uint32_t)row * (uint32_t)d.nx + (uint32_t)(u.x0 + s), step, n);
+      }
       R fl[Q];
       collide_3d<Q, R, DEV, SAMPLE>(d, g, noisy, n, fl);
 #pragma unroll
@@ -661,6 +677,15 @@ static void launch_step3_q(int precision, int vec, const StepLaunch& L, bool sam
   const bool one = L.n_reps == 1;
   const int split = precision == FLB_FP64 ? step_split(L.n_vblocks, L.sms) : 0;
   const int grid = (int)std::min<int64_t>(L.n_vblocks << split, (int64_t)L.grid << split);
+  if (precision == FLB_FP64 && split && grid == L.n_vblocks << split && early_ok(grid, kEarlyBlocks3, L.sms)) {
+    EarlyLaunch el(grid, kStepThreads >> split, st);
+#define FLB_LE(S, O) cudaLaunchKernelEx(&el.cfg, k_step_3d<Q, double, false, 1, S, O, true>, L.descs, *L.desc0, \
+                                        L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
+    if (one) { if (sample) FLB_LE(true, true); else FLB_LE(false, true); }
+    else { if (sample) FLB_LE(true, false); else FLB_LE(false, false); }
+    return;
+#undef FLB_LE
+  }
 #define FLB_L3(R, DEV, V, S, O) k_step_3d<Q, R, DEV, V, S, O><<<grid, kStepThreads >> split, 0, st>>>( \
       L.descs, *L.desc0, L.vb_begin, L.n_reps, L.n_vblocks, L.ws, L.parity, L.step, L.step_dev, split)
 #define FLB_LS(R, DEV, V) { \

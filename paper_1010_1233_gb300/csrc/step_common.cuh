@@ -52,6 +52,10 @@ __device__ __forceinline__ void block_sums(double (&acc)[kNumSums], double* __re
 
 template <typename R, int VEC> struct VecIO;
 // loads past L1, for state that a kernel still running at this kernel's launch may write
+template <int VEC> __device__ __forceinline__ void ld_l2(const double* p, double (&v)[VEC]) {
+  static_assert(VEC == 1, "one FP64 site per thread");
+  v[0] = __ldcg(p);
+}
 template <int VEC> __device__ __forceinline__ void ld_l2(const float* p, float (&v)[VEC]) {
   if constexpr (VEC == 1) v[0] = __ldcg(p);
   else if constexpr (VEC == 2) { const float2 t = __ldcg(reinterpret_cast<const float2*>(p)); v[0] = t.x; v[1] = t.y; }

@@ -1,7 +1,8 @@
 """The FP32 D2Q9 step kernel for two and four sites per thread against the one-site kernel (GPU):
 bit-identical states and sampled fields at the edges of its units and blocks -- rows of two
 sites, one row, rows that end inside a warp, lattices of less than a block and of blocks of a
-quarter, every noise mode, masks without noise, uneven batches whose blocks change replica."""
+quarter, every noise mode, masks without noise, uneven batches whose blocks change replica; and
+the FP64 steps that are launched early against plain launches."""
 import numpy as np
 import pytest
 
@@ -42,3 +43,27 @@ def test_batched_pairs_and_fields(fields):
     for vec in (2, 4):
         for a, b in zip(_states(reps, vec, 3), one):
             assert np.array_equal(a, b), vec
+
+
+@pytest.mark.parametrize("lat,dims", [("D2Q9", (2, 1)), ("D2Q9", (16, 16)), ("D2Q9", (254, 67)), ("D2Q9", (256, 266)),
+                                      ("D2Q9", (320, 256)), ("D3Q15", (6, 5, 4)), ("D3Q15", (48, 32, 25)),
+                                      ("D3Q15", (64, 48, 40)), ("D3Q19", (32, 19, 64))])
+def test_early_launches_equal_plain_ones(lat, dims):
+    # FP64 steps launched beside the step before (one unit per thread) against one block that loops
+    # over everything, launched after it: the same states, sampled or not, in and out of graphs
+    kw = dict(kT=1e-3, seed=sum(dims), init_mode=1, fields=(0, 4))
+    p = (W.replica("D2Q9", *dims, W.taus_d2q9(0.6, 0.8, 1.1), u0=(0.1, -0.05), **kw) if lat == "D2Q9" else
+         W.replica3(*dims, (W.taus_d3q15 if lat == "D3Q15" else W.taus_d3q19)(0.7, 0.9, 1.1), u0=(0.05, -0.02, 0.03),
+                    lattice=lat, **kw))
+    pow2 = lat != "D2Q9" or all(n & (n - 1) == 0 for n in dims)
+    every = 5 if pow2 else 0
+    if not pow2:
+        p["fields"] = ()
+    a, b = Sim(p, precision="fp64"), Sim(p, precision="fp64")
+    b.set_step_config(1, 1)
+    for n in (3, 70, 9):
+        a.run(n, every)
+        b.run(n, every)
+    assert np.array_equal(a.populations(), b.populations())
+    if every:
+        assert np.array_equal(a.fields(), b.fields())
