@@ -494,9 +494,9 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
       steps_smem = std::max(steps_smem, d1q3_steps_smem(d.nx));
     }
     if (steps_smem <= kFusedSmemMax && run.sample_smem <= kFusedSmemMax) {
-      // a chunk's noise and pulled populations in at most kD1ScratchBytes, 1024 steps at most; the
+      // a chunk's noise and pulled populations in at most kD1ScratchBytes (or four steps), 1024 steps at most; the
       // sampling kernel's blocks over the GPU
-      run.chunk = (uint32_t)std::max<int64_t>(16, std::min<int64_t>(1024, kD1ScratchBytes / (32 * sites)));
+      run.chunk = (uint32_t)std::max<int64_t>(4, std::min<int64_t>(1024, kD1ScratchBytes / (32 * sites)));
       run.blocks = std::max(1, kD1SampleBlocks / n);
       for (ReplicaDesc& d : L.desc) {
         d.off_d1_noise = off; off = align256(off + 8 * (int64_t)run.chunk * d.nx);
