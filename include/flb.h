@@ -278,8 +278,9 @@ int flb_autotune(flb_ctx* ctx, int trials, int* vec_out, int* grid_out, int* sta
  * chunk of whole sampling periods (at least 32 steps; 32 steps without
  * sampling), which removes the per-kernel launch cost on small lattices.  D1Q3
  * contexts (without time correlators) instead run up to 4096 steps and their
- * samples per launch of one fused kernel, one block per replica with its state
- * in shared memory.  Results are identical to direct launches up to the
+ * samples per launch of one fused kernel in FP32, one block per replica with its
+ * state in shared memory, and in FP64 chunks of up to 1024 steps as four launches
+ * (noise, steps, transforms and pair sums of the samples, their addition).  Results are identical to direct launches up to the
  * contraction of multiply-adds.  The captured graphs are dropped when the
  * launch configuration or the network switch changes.  enable = 0 issues every
  * kernel of every step directly. */

@@ -417,8 +417,14 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
     L.vec = all4 && sites >= kVec4Sites ? 4 : 2;
   } else if (precision == FLB_FP32_DEV && is3d(lat)) {
     bool all4 = lat == FLB_D3Q15;                // nx is even; D3Q19 at vec 4 spills registers
-    for (int r = 0; r < n; ++r) all4 = all4 && reps[r].nx % 4 == 0;
-    L.vec = all4 ? 4 : 2;
+    int64_t sites = 0;
+    for (int r = 0; r < n; ++r) {
+      all4 = all4 && reps[r].nx % 4 == 0;
+      sites += (int64_t)reps[r].nx * reps[r].ny * reps[r].nz;
+    }
+    // two sites per thread on small boxes, as on D2Q9 (the same states; D3Q15 16 x 12 x 10, us per
+    // step: vec 4 5.8, vec 2 4.2; 64 x 48 x 40 6.2 and 5.8; 96 x 64 x 64 equal)
+    L.vec = all4 && sites >= kVec4Sites / 4 ? 4 : 2;
   }
   L.desc.resize(n);
   int64_t off = 0;
