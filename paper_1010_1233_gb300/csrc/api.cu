@@ -499,7 +499,7 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
       if (d.n_fields) run.sample_smem = std::max(run.sample_smem, d1q3_sample_smem(d.nx, (int)d.n_fields));
       steps_smem = std::max(steps_smem, d1q3_steps_smem(d.nx));
     }
-    if (steps_smem <= kFusedSmemMax && run.sample_smem <= kFusedSmemMax) {
+    if (run.max_nx <= kD1MaxSites && steps_smem <= kFusedSmemMax && run.sample_smem <= kFusedSmemMax) {
       // a chunk's noise and pulled populations in at most kD1ScratchBytes (or four steps), 1024 steps at most; the
       // sampling kernel's blocks over the GPU
       run.chunk = (uint32_t)std::max<int64_t>(4, std::min<int64_t>(1024, kD1ScratchBytes / (32 * sites)));

@@ -221,6 +221,9 @@ struct TimeCorr {
   int part_blocks = 0;              // 3D lattices: blocks of the direct transform (partials per replica)
 };
 
+// Sites of a lattice that the FP64 D1Q3 run kernels take: one block of at most 1024 threads, up to
+// kD1SitesPerThread sites each.
+constexpr int kD1SitesPerThread = 4, kD1MaxSites = 1024 * kD1SitesPerThread;
 // A run of FP64 D1Q3 steps (lb_d1q3_runs.cu): steps per chunk and what its launches are sized by
 // (over the replicas of the context), sampling period (0: none).
 struct D1Run {

@@ -231,12 +231,13 @@ k_d1q3_finish(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint
 cudaError_t set_d1q3_runs_smem() {
   const int m = 200 * 1024;
   cudaError_t e = cudaFuncSetAttribute(k_d1q3_steps<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
-  if (!e) e = cudaFuncSetAttribute(k_d1q3_steps<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
+  if (!e) e = cudaFuncSetAttribute(k_d1q3_steps<kD1SitesPerThread>, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
   if (!e) e = cudaFuncSetAttribute(k_d1q3_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, m);
   return e;
 }
 
-// One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= run.chunk) of all replicas; returns the launches.
+// One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= run.chunk) of all replicas (run.max_nx <=
+// kD1MaxSites); returns the launches.
 int launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0, uint32_t n_steps,
                       int sms, cudaStream_t st) {
   const int64_t most = (int64_t)n_steps * run.max_nx;
@@ -246,7 +247,7 @@ int launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Ru
   if (run.max_nx <= 1024)
     k_d1q3_steps<1><<<n_reps, (run.max_nx + 31) & ~31, smem, st>>>(descs, ws, run, t0, n_steps);
   else
-    k_d1q3_steps<4><<<n_reps, 1024, smem, st>>>(descs, ws, run, t0, n_steps);
+    k_d1q3_steps<kD1SitesPerThread><<<n_reps, 1024, smem, st>>>(descs, ws, run, t0, n_steps);
   uint32_t ns = 0;
   if (run.every) {             // samples at the steps t in [t0, t0 + n_steps) with t % every == 0
     const uint64_t first = (t0 + run.every - 1) / run.every * run.every;

@@ -1,0 +1,34 @@
+"""FP64 D1Q3 runs at the limits of their chunked form (csrc/lb_d1q3_runs.cu), against the per-step
+launches (GPU).  The arithmetic of a site is the same on both paths, so states are equal bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1010_1233_gb300 import Sim, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _replica(nx, fields=(), **kw):
+    args = dict(kT=1e-3, u0=(0.05, 0.0), seed=nx, init_mode=1)
+    return W.replica("D1Q3", nx, 1, W.taus_d1q3(0.7), fields=fields, **{**args, **kw})
+
+
+def _launches(sim, n, every):
+    n0 = sim.kernel_launches()
+    sim.run(n, every)
+    return sim.kernel_launches() - n0
+
+
+@pytest.mark.parametrize("sizes", [(4096,), (4098,), (4200,), (4266,), (4268,), (64, 4098), (64, 4266), (4096, 64)])
+def test_lattices_wider_than_a_block_covers(sizes):
+    # 1024 threads of four sites each take 4096 sites; wider lattices, and batches with one, run
+    # one launch per step
+    reps = [_replica(nx, stream=i) for i, nx in enumerate(sizes)]
+    a, b = Sim(reps, precision="fp64"), Sim(reps, precision="fp64")
+    b.set_graphs(False)
+    for n in (3, 9):
+        launched = _launches(a, n, 0)
+        assert (launched < n) == (max(sizes) <= 4096), launched
+        b.run(n)
+    for r in range(len(reps)):
+        assert np.array_equal(a.populations(r), b.populations(r)), r
