@@ -56,8 +56,8 @@ cudaError_t launch_d1q3_fused(const ReplicaDesc* descs, int n_reps, char* ws, ui
 size_t d1q3_steps_smem(int nx);
 size_t d1q3_sample_smem(int nx, int F);
 cudaError_t set_d1q3_runs_smem();
-int launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0, uint32_t n_steps,
-                      int sms, cudaStream_t st);
+cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0,
+                              uint32_t n_steps, int sms, cudaStream_t st, int* launches);
 // D3Q15 / D3Q19 (lb_3d.cu), q = 15 or 19
 void launch_step3(int q, int precision, int vec, const StepLaunch& L, bool sample, cudaStream_t st);
 void launch_init3(int q, int precision, const ReplicaDesc* descs, int r, char* ws, int mode, const double* feq0,
@@ -1166,7 +1166,11 @@ int flb_run(flb_ctx* c, uint64_t n_steps, uint32_t sample_every) {
     run.every = sampling ? sample_every : 0;
     for (uint64_t i = 0; i < n_steps;) {
       const uint32_t n = (uint32_t)std::min<uint64_t>(n_steps - i, run.chunk);
-      count_kernels(c, launch_d1q3_chunk(descs_dev(c), c->n, c->ws, run, c->step, n, c->sms, c->stream));
+      int launches = 0;
+      const int rc = cuda_check(launch_d1q3_chunk(descs_dev(c), c->n, c->ws, run, c->step, n, c->sms, c->stream,
+                                                  &launches), "D1Q3 launch");
+      count_kernels(c, launches);
+      if (rc) return rc;
       if (run.every) {
         const uint64_t first = (c->step + run.every - 1) / run.every * run.every;
         if (first < c->step + n) c->n_samples += (c->step + n - 1 - first) / run.every + 1;
@@ -1174,7 +1178,7 @@ int flb_run(flb_ctx* c, uint64_t n_steps, uint32_t sample_every) {
       c->step += n;
       i += n;
     }
-    return cuda_check(cudaGetLastError(), "D1Q3 launch");
+    return FLB_OK;
   }
   if (c->fused_smem && c->use_graphs && !c->tc.base) {
     // FP32 D1Q3: runs of up to kFusedChunk steps with their sampling in one launch

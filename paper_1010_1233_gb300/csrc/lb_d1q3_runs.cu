@@ -46,12 +46,12 @@ size_t d1q3_sample_smem(int nx, int F) {
 // Scratch of a replica (ReplicaDesc::off_d1_*): noise [chunk][nx], pulled populations [samples][3][nx],
 // partial sums [run.blocks][items] (double2).
 __global__ void __launch_bounds__(256)
-k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, D1Run run, uint64_t t0, uint32_t n_steps) {
-  const ReplicaDesc& d = descs[blockIdx.y];
+k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint64_t t0, uint32_t n_steps) {
+  const ReplicaDesc& d = descs[blockIdx.x];
   const int nx = d.nx;
   double* out = reinterpret_cast<double*>(ws + d.off_d1_noise);
   const uint32_t n = n_steps * (uint32_t)nx;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
     const uint32_t s = i / (uint32_t)nx;
     out[i] = d1q3_noise(d, (int)(i - s * nx), (uint32_t)(t0 + s));
   }
@@ -118,25 +118,25 @@ k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, D1Run
   for (int i = tid; i < 3 * nx; i += nt) dst[i] = fin[i];
 }
 
-// Block g of replica blockIdx.y takes the sample batches g, g + G, .. (G = gridDim.x) of the chunk's
-// ns samples and leaves its sums in partial row g; the block of the last batch writes its fields.
+// Block g = blockIdx.y of replica blockIdx.x takes the sample batches g, g + G, .. (G = gridDim.y) of the
+// chunk's ns samples and leaves its sums in partial row g; the block of the last batch writes its fields.
 __global__ void __launch_bounds__(kD1SampleThreads)
 k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const ReplicaDesc& d = descs[blockIdx.y];
+  const ReplicaDesc& d = descs[blockIdx.x];
   const int nx = d.nx, logn = d.log2nx, F = (int)d.n_fields, hn1 = nx / 2 + 1, tid = (int)threadIdx.x;
   const int nt = (int)blockDim.x;
   if (!F) return;
-  const int rows = d1_rows(F), SB = d1_batch_of(nx, F, ns, (int)gridDim.x), ss = nx + 33;
+  const int rows = d1_rows(F), SB = d1_batch_of(nx, F, ns, (int)gridDim.y), ss = nx + 33;
   const int ps = logn > 5 ? logn - 5 : 31;
   double2* z = reinterpret_cast<double2*>(smem_raw);
   double2* X = z + SB * rows * ss;
   const double2* tw = reinterpret_cast<const double2*>(ws + d.off_tw_x);
   const double* raw = reinterpret_cast<const double*>(ws + d.off_d1_raw);
   const int items = (int)d1q3_items(d);
-  double2* part = reinterpret_cast<double2*>(ws + d.off_d1_part) + (int64_t)blockIdx.x * items;
+  double2* part = reinterpret_cast<double2*>(ws + d.off_d1_part) + (int64_t)blockIdx.y * items;
   bool first = true;
-  for (uint32_t b0 = blockIdx.x * SB; b0 < ns; b0 += gridDim.x * SB) {
+  for (uint32_t b0 = blockIdx.y * SB; b0 < ns; b0 += gridDim.y * SB) {
     const int nb = (int)min((uint32_t)SB, ns - b0), nq = nb * rows;             // samples, packed rows
     const bool last = b0 + nb == ns;
     // bit-reversed load of the packed rows (and, in the last batch, the fields of the last sample)
@@ -195,13 +195,13 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint
 // to the replica's sums.
 __global__ void __launch_bounds__(256)
 k_d1q3_finish(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns, int blocks) {
-  const ReplicaDesc& d = descs[blockIdx.y];
+  const ReplicaDesc& d = descs[blockIdx.x];
   const int F = (int)d.n_fields, hn1 = d.nx / 2 + 1, lane = (int)threadIdx.x & 31;
   if (!F) return;
   const int SB = d1_batch_of(d.nx, F, ns, blocks), items = (int)d1q3_items(d);
   const int used = (int)min((uint32_t)blocks, (ns + SB - 1) / SB);
   const double2* part = reinterpret_cast<const double2*>(ws + d.off_d1_part);
-  for (int it = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += (int)(gridDim.x * blockDim.x) >> 5) {
+  for (int it = (int)(blockIdx.y * blockDim.x + threadIdx.x) >> 5; it < items; it += (int)(gridDim.y * blockDim.x) >> 5) {
     double2 v = make_double2(0.0, 0.0);
     for (int g = lane; g < used; g += 32) {
       const double2 p = part[(int64_t)g * items + it];
@@ -237,26 +237,37 @@ cudaError_t set_d1q3_runs_smem() {
 }
 
 // One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= run.chunk) of all replicas (run.max_nx <=
-// kD1MaxSites); returns the launches.
-int launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0, uint32_t n_steps,
-                      int sms, cudaStream_t st) {
+// kD1MaxSites); adds the launches to *launches.  Replicas are in the grids' x (up to 2^31 - 1; y ends at
+// 65535).  A launch that is refused ends the chunk: its first kernel writes scratch alone, so the
+// state stays as it was when that one fails.
+cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0,
+                              uint32_t n_steps, int sms, cudaStream_t st, int* launches) {
   const int64_t most = (int64_t)n_steps * run.max_nx;
-  k_d1q3_noise<<<dim3((unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms), n_reps), 256, 0, st>>>(
-      descs, ws, run, t0, n_steps);
+  cudaError_t e;
+  k_d1q3_noise<<<dim3(n_reps, (unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms)), 256, 0, st>>>(
+      descs, ws, t0, n_steps);
+  if ((e = cudaGetLastError())) return e;
+  ++*launches;
   const size_t smem = d1q3_steps_smem(run.max_nx);
   if (run.max_nx <= 1024)
     k_d1q3_steps<1><<<n_reps, (run.max_nx + 31) & ~31, smem, st>>>(descs, ws, run, t0, n_steps);
   else
     k_d1q3_steps<kD1SitesPerThread><<<n_reps, 1024, smem, st>>>(descs, ws, run, t0, n_steps);
+  if ((e = cudaGetLastError())) return e;
+  ++*launches;
   uint32_t ns = 0;
   if (run.every) {             // samples at the steps t in [t0, t0 + n_steps) with t % every == 0
     const uint64_t first = (t0 + run.every - 1) / run.every * run.every;
     if (first < t0 + n_steps) ns = (uint32_t)((t0 + n_steps - 1 - first) / run.every + 1);
   }
-  if (!ns || !run.sample_smem) return 2;
-  k_d1q3_sample<<<dim3(run.blocks, n_reps), kD1SampleThreads, run.sample_smem, st>>>(descs, ws, ns);
-  k_d1q3_finish<<<dim3((unsigned)((run.max_items + 7) / 8), n_reps), 256, 0, st>>>(descs, ws, ns, run.blocks);
-  return 4;
+  if (!ns || !run.sample_smem) return cudaSuccess;
+  k_d1q3_sample<<<dim3(n_reps, run.blocks), kD1SampleThreads, run.sample_smem, st>>>(descs, ws, ns);
+  if ((e = cudaGetLastError())) return e;
+  ++*launches;
+  k_d1q3_finish<<<dim3(n_reps, (unsigned)((run.max_items + 7) / 8)), 256, 0, st>>>(descs, ws, ns, run.blocks);
+  if ((e = cudaGetLastError())) return e;
+  ++*launches;
+  return cudaSuccess;
 }
 
 }  // namespace flb

@@ -32,3 +32,21 @@ def test_lattices_wider_than_a_block_covers(sizes):
         b.run(n)
     for r in range(len(reps)):
         assert np.array_equal(a.populations(r), b.populations(r)), r
+
+
+def test_more_replicas_than_a_grid_dimension():
+    # 65,535 blocks is the limit of a grid in y and z, 2^31 - 1 in x
+    n, pick = 65_540, (0, 65_534, 65_535, 65_536, 65_539)
+    reps = [_replica(16, fields=(0,), seed=5, stream=i, init_mode=0, u0=(0.01 * (i % 7), 0.0)) for i in range(n)]
+    sim = Sim(reps, precision="fp64")
+    assert _launches(sim, 9, 3) > 0
+    sim.sync()
+    for r in pick:
+        one = Sim(reps[r], precision="fp64")
+        one.set_graphs(False)
+        one.run(9, 3)
+        assert np.array_equal(sim.populations(r), one.populations()), r
+        c, k = sim.correlator(r, 0, 0, with_count=True)
+        c1, k1 = one.correlator(0, 0, 0, with_count=True)
+        # three samples, added in another order: 2 roundings of 2^-53, and those of the transforms
+        assert k == k1 == 3 and np.abs(c - c1).max() <= 1e-13 * max(1.0, np.abs(c1).max()), r
