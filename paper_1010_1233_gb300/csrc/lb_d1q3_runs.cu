@@ -23,13 +23,21 @@
 namespace flb {
 
 constexpr int kD1SampleThreads = 256;
-constexpr int kD1SamplePoints = 2048;        // points of packed rows in one block's batch
+constexpr int kD1SamplePoints = 2048;        // points of packed rows in one block's batch, at most
+constexpr size_t kD1SampleSmem = 80 * 1024;  // shared memory of a batch of more than one sample
 
 __host__ __device__ inline int d1_rows(int F) { return (F + 1) / 2; }           // packed rows per sample
-// samples of a batch of k_d1q3_sample: at most what its shared memory is sized for, and no more
-// than an even share of the ns samples (a batch's transforms are FP64-bound, 0.5 us a sample at L = 64)
+// shared memory of one sample: its packed rows with their pad slots and the half spectra of its fields
+__host__ __device__ inline size_t d1_sample_bytes(int nx, int F) {
+  return ((size_t)d1_rows(F) * (nx + 33) + (size_t)F * (nx / 2 + 1)) * sizeof(double2);
+}
+// samples of a batch of k_d1q3_sample: as many as kD1SamplePoints and kD1SampleSmem hold (below 32 sites
+// the pad slots take most of a row), and no more than an even share of the ns samples (a batch's
+// transforms are FP64-bound, 0.5 us a sample at L = 64)
 __host__ __device__ inline int d1_batch(int nx, int F) {
-  const int b = kD1SamplePoints / (nx * d1_rows(F > 0 ? F : 1));
+  if (F < 1) return 1;
+  const int pts = kD1SamplePoints / (nx * d1_rows(F)), fit = (int)(kD1SampleSmem / d1_sample_bytes(nx, F));
+  const int b = pts < fit ? pts : fit;
   return b < 1 ? 1 : b;
 }
 __device__ __forceinline__ int d1_batch_of(int nx, int F, uint32_t ns, int blocks) {
@@ -38,10 +46,7 @@ __device__ __forceinline__ int d1_batch_of(int nx, int F, uint32_t ns, int block
 }
 
 size_t d1q3_steps_smem(int nx) { return 6 * (size_t)nx * sizeof(double); }
-size_t d1q3_sample_smem(int nx, int F) {
-  const size_t b = d1_batch(nx, F);
-  return (b * d1_rows(F) * (nx + 33) + b * F * (nx / 2 + 1)) * sizeof(double2);
-}
+size_t d1q3_sample_smem(int nx, int F) { return d1_batch(nx, F) * d1_sample_bytes(nx, F); }
 
 // Scratch of a replica (ReplicaDesc::off_d1_*): noise [chunk][nx], pulled populations [samples][3][nx],
 // partial sums [run.blocks][items] (double2).

@@ -34,6 +34,26 @@ def test_lattices_wider_than_a_block_covers(sizes):
         assert np.array_equal(a.populations(r), b.populations(r)), r
 
 
+@pytest.mark.parametrize("nx,fields", [(2, (0,)), (2, (0, 9)), (2, (0, 1, 2, 9)), (4, (1,)), (4, (0, 1)), (4, (0, 1, 2, 9)),
+                                       (8, (2,)), (8, (0, 1)), (8, (0, 1, 2, 9)), (16, (0, 1, 2)), (2048, (0, 1, 2, 9))])
+def test_sampled_lattices_of_every_size_run_in_chunks(nx, fields):
+    # alone, and as the smallest of a batch, whose launches are sized by the largest of its replicas
+    for reps in ([_replica(nx, fields)], [_replica(64, (0, 1, 2), stream=1), _replica(nx, fields), _replica(32, stream=2)]):
+        a, b = Sim(reps, precision="fp64"), Sim(reps, precision="fp64")
+        b.set_graphs(False)
+        assert _launches(a, 45, 2) <= 4 * 12                    # a few launches a chunk; per step 45 + 2 x 23
+        b.run(45, 2)
+        for r, p in enumerate(reps):
+            assert np.array_equal(a.populations(r), b.populations(r)), r
+            for i, x in enumerate(p["fields"]):
+                for y in p["fields"][i:]:
+                    ca, na = a.correlator(r, x, y, with_count=True)
+                    cb, nb = b.correlator(r, x, y, with_count=True)
+                    # 23 samples in another order: 23 roundings of 2^-53 of the sum's size, and those of
+                    # the transforms
+                    assert na == nb == 23 and np.abs(ca - cb).max() <= 1e-13 * max(1.0, np.abs(cb).max()), (r, x, y)
+
+
 def test_more_replicas_than_a_grid_dimension():
     # 65,535 blocks is the limit of a grid in y and z, 2^31 - 1 in x
     n, pick = 65_540, (0, 65_534, 65_535, 65_536, 65_539)
