@@ -57,7 +57,9 @@ size_t d1q3_steps_smem(int nx);
 size_t d1q3_sample_smem(int nx, int F);
 cudaError_t set_d1q3_runs_smem();
 cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0,
-                              uint32_t n_steps, int sms, cudaStream_t st, int* launches);
+                              uint32_t n_steps, int sms, cudaStream_t st, uint32_t* pending, int* launches);
+cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint32_t pending,
+                             cudaStream_t st, int* launches);
 // D3Q15 / D3Q19 (lb_3d.cu), q = 15 or 19
 void launch_step3(int q, int precision, int vec, const StepLaunch& L, bool sample, cudaStream_t st);
 void launch_init3(int q, int precision, const ReplicaDesc* descs, int r, char* ws, int mode, const double* feq0,
@@ -132,7 +134,7 @@ static constexpr int kStepBlock = 256;
 static constexpr int64_t kVec4Sites = 1 << 20;
 static constexpr size_t kFusedSmemMax = 200 * 1024;           // D1Q3 runs: shared memory of a block
 static constexpr int64_t kD1ScratchBytes = 64 << 20;
-static constexpr int kD1SampleBlocks = 152;
+static constexpr uint32_t kD1LastSamples = 128;
 
 struct Layout {
   std::vector<ReplicaDesc> desc;
@@ -491,24 +493,24 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   if (lat == FLB_D1Q3 && precision == FLB_FP64) {
     D1Run& run = L.d1;
     size_t steps_smem = 0;
-    int64_t sites = 0;
+    int64_t step_bytes = 0;                      // scratch of a sampled step of all replicas
     for (const ReplicaDesc& d : L.desc) {
-      sites += d.nx;
+      step_bytes += 8 * (int64_t)d.nx;
       run.max_nx = std::max(run.max_nx, (int)d.nx);
-      run.max_items = std::max(run.max_items, (int)d1q3_items(d));
-      if (d.n_fields) run.sample_smem = std::max(run.sample_smem, d1q3_sample_smem(d.nx, (int)d.n_fields));
       steps_smem = std::max(steps_smem, d1q3_steps_smem(d.nx));
+      if (!d.n_fields) continue;
+      step_bytes += 24 * (int64_t)d.nx + 8 * d1q3_products(d.nx, (int)d.n_fields);
+      run.max_products = std::max(run.max_products, d1q3_products(d.nx, (int)d.n_fields));
+      run.sample_smem = std::max(run.sample_smem, d1q3_sample_smem(d.nx, (int)d.n_fields));
     }
     if (run.max_nx <= kD1MaxSites && steps_smem <= kFusedSmemMax && run.sample_smem <= kFusedSmemMax) {
-      // a chunk's noise and pulled populations in at most kD1ScratchBytes (or four steps), 1024 steps at most; the
-      // sampling kernel's blocks over the GPU
-      run.chunk = (uint32_t)std::max<int64_t>(4, std::min<int64_t>(1024, kD1ScratchBytes / (32 * sites)));
-      run.blocks = std::max(1, kD1SampleBlocks / n);
+      // a chunk's noise, pulled populations and products in at most kD1ScratchBytes (or four steps), 1024 steps at most
+      run.chunk = (uint32_t)std::max<int64_t>(4, std::min<int64_t>(1024, kD1ScratchBytes / step_bytes));
       for (ReplicaDesc& d : L.desc) {
         d.off_d1_noise = off; off = align256(off + 8 * (int64_t)run.chunk * d.nx);
         if (!d.n_fields) continue;
         d.off_d1_raw = off; off = align256(off + 24 * (int64_t)run.chunk * d.nx);
-        d.off_d1_part = off; off = align256(off + 16 * (int64_t)run.blocks * d1q3_items(d));
+        d.off_d1_prod = off; off = align256(off + 8 * (int64_t)run.chunk * d1q3_products(d.nx, (int)d.n_fields));
       }
     }
   }
@@ -1164,13 +1166,17 @@ int flb_run(flb_ctx* c, uint64_t n_steps, uint32_t sample_every) {
     NvtxRange chunk_range("flb D1Q3 chunks");
     D1Run run = L.d1;
     run.every = sampling ? sample_every : 0;
-    for (uint64_t i = 0; i < n_steps;) {
-      const uint32_t n = (uint32_t)std::min<uint64_t>(n_steps - i, run.chunk);
-      int launches = 0;
-      const int rc = cuda_check(launch_d1q3_chunk(descs_dev(c), c->n, c->ws, run, c->step, n, c->sms, c->stream,
-                                                  &launches), "D1Q3 launch");
-      count_kernels(c, launches);
-      if (rc) return rc;
+    int rc = FLB_OK, launches = 0;
+    uint32_t pending = 0;                        // samples of the last chunk whose products are not yet in the sums
+    for (uint64_t i = 0; i < n_steps && !rc;) {
+      const uint64_t left = n_steps - i;
+      uint32_t n = (uint32_t)std::min<uint64_t>(left, run.chunk);
+      // the additions of the last chunk have no steps beside them (58 ns a sample): leave it few samples,
+      // where that saves more than its other launches take (16 us)
+      if (run.every && n == left && left / run.every > 4 * kD1LastSamples) n -= kD1LastSamples * run.every;
+      rc = cuda_check(launch_d1q3_chunk(descs_dev(c), c->n, c->ws, run, c->step, n, c->sms, c->stream, &pending,
+                                        &launches), "D1Q3 launch");
+      if (rc) break;
       if (run.every) {
         const uint64_t first = (c->step + run.every - 1) / run.every * run.every;
         if (first < c->step + n) c->n_samples += (c->step + n - 1 - first) / run.every + 1;
@@ -1178,7 +1184,9 @@ int flb_run(flb_ctx* c, uint64_t n_steps, uint32_t sample_every) {
       c->step += n;
       i += n;
     }
-    return FLB_OK;
+    if (!rc) rc = cuda_check(launch_d1q3_sums(descs_dev(c), c->n, c->ws, run, pending, c->stream, &launches), "D1Q3 launch");
+    count_kernels(c, launches);
+    return rc;
   }
   if (c->fused_smem && c->use_graphs && !c->tc.base) {
     // FP32 D1Q3: runs of up to kFusedChunk steps with their sampling in one launch

@@ -85,7 +85,7 @@ struct alignas(16) ReplicaDesc {
                                     // the column pass produces the points: [k1][kx / c][k2][kx % c]
                                     // (ky = k1 + N1 k2; kx padded to a multiple of c)
   double dco[kNumCoef];             // fco in FP64
-  int64_t off_d1_noise, off_d1_raw, off_d1_part;   // FP64 D1Q3 runs: scratch (lb_d1q3_runs.cu)
+  int64_t off_d1_noise, off_d1_raw, off_d1_prod;   // FP64 D1Q3 runs: scratch (lb_d1q3_runs.cu)
 };
 constexpr int kStepHeadBytes = offsetof(ReplicaDesc, log2nx);
 static_assert(offsetof(ReplicaDesc, rkey) % 16 == 4 && offsetof(ReplicaDesc, fco) % 16 == 4, "see the head's comment");
@@ -228,12 +228,16 @@ constexpr int kD1SitesPerThread = 4, kD1MaxSites = 1024 * kD1SitesPerThread;
 // (over the replicas of the context), sampling period (0: none).
 struct D1Run {
   uint32_t chunk = 0, every = 0;
-  int max_nx = 0, blocks = 0, max_items = 0;   // blocks of the sampling kernel per replica
+  int max_nx = 0;
+  int64_t max_products = 0;
   size_t sample_smem = 0;
 };
-// partial sums of a block: every pair's half spectrum and the k = 0 value of every field
-__host__ __device__ __forceinline__ int64_t d1q3_items(const ReplicaDesc& d) {
-  return (int64_t)d.n_pairs * (d.nx / 2 + 1) + d.n_fields;
+// products of a sample, in the order of the sums (lb_d1q3_runs.cu): F fields with themselves (one
+// double a wave vector), F (F - 1) / 2 pairs of two (two doubles) and the k = 0 values; the first of
+// pair pr = (a, b), which comes after a pairs of a field with itself, or a + 1 when b > a
+__host__ __device__ __forceinline__ int64_t d1q3_products(int nx, int F) { return (int64_t)F * F * (nx / 2 + 1) + F; }
+__host__ __device__ __forceinline__ int64_t d1q3_pair_first(int nx, int pr, int a, int b) {
+  return (int64_t)(2 * pr - a - (b > a ? 1 : 0)) * (nx / 2 + 1);
 }
 
 // Arguments of one step launch (lb_step.cu).

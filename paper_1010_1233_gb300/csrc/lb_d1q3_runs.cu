@@ -11,8 +11,11 @@
 //                  a step; the noise is loaded two steps ahead; at a sample the pulled
 //                  populations go to memory
 //   k_d1q3_sample  row transforms of all samples (radix-2 passes of fft_common.cuh, two fields
-//                  packed per complex row) and per-block sums of the pair products
-//   k_d1q3_finish  adds the blocks' sums to the replica's, in block order
+//                  packed per complex row) and their pair products
+//   k_d1q3_sums    adds the products to the replica's sums, sample by sample
+// Every sum takes the samples' products one at a time in the order of the steps, as the per-step
+// launches add them, so it does not depend on how runs are cut into calls and chunks or on the other
+// replicas of the context.
 // k_d1q3_steps is bound by its warps' FP64 instructions, one in 64 cycles (15 x 64 = 960 of the 1240
 // cycles of a step up to 128 sites, four warps on four schedulers): L = 64, 0.60 us a step, 0.64 with
 // every step sampled.
@@ -49,7 +52,8 @@ size_t d1q3_steps_smem(int nx) { return 6 * (size_t)nx * sizeof(double); }
 size_t d1q3_sample_smem(int nx, int F) { return d1_batch(nx, F) * d1_sample_bytes(nx, F); }
 
 // Scratch of a replica (ReplicaDesc::off_d1_*): noise [chunk][nx], pulled populations [samples][3][nx],
-// partial sums [run.blocks][items] (double2).
+// products [samples][d1q3_products] in the order of the replica's sums: the pairs (one double a wave
+// vector for a field with itself, two for two fields), then the k = 0 value of every field.
 __global__ void __launch_bounds__(256)
 k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint64_t t0, uint32_t n_steps) {
   const ReplicaDesc& d = descs[blockIdx.x];
@@ -62,12 +66,60 @@ k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint6
   }
 }
 
+// The ns samples' products added to a replica's sums, a thread per product, by block `part` of `parts`.
+// A thread's chain of ns dependent additions (58 ns each) bounds it, so its loads run a step ahead.
+__device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __restrict__ ws, uint32_t ns, int part,
+                                                  int parts) {
+  const int F = (int)d.n_fields, nx = d.nx;
+  if (!F) return;
+  const int64_t np = d1q3_products(nx, F);
+  for (int64_t i = (int64_t)part * blockDim.x + threadIdx.x; i < np; i += (int64_t)parts * blockDim.x) {
+    double* sum;
+    if (i >= np - F) {
+      sum = reinterpret_cast<double*>(ws + d.off_mean0) + (i - (np - F));
+    } else {
+      int pr = d.n_pairs - 1;
+      while (pr > 0 && i < d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr])) --pr;
+      sum = reinterpret_cast<double*>(ws + d.pair_off[pr]) + (i - d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr]));
+    }
+    const double* p = reinterpret_cast<const double*>(ws + d.off_d1_prod) + i;
+    double acc = *sum, v[8], w[8];
+    uint32_t s = 0;
+    if (ns >= 8) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = p[u * np];
+      for (; s + 16 <= ns; s += 8) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) w[u] = p[(s + 8 + u) * np];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, v[u]);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = w[u];
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, v[u]);
+      s += 8;
+    }
+    for (; s < ns; ++s) acc = __dadd_rn(acc, p[s * np]);
+    *sum = acc;
+  }
+}
+
 // SPT sites per thread (x = tid + k blockDim): steps t0 .. t0 + n_steps - 1 of replica blockIdx.x,
-// state from the buffer of parity t0 & 1 to that of (t0 + n_steps) & 1.
+// state from the buffer of parity t0 & 1 to that of (t0 + n_steps) & 1.  The blocks from n_reps on add
+// the products of the chunk before (its sum_ns samples), sum_parts of them a replica: 60 us of a chain
+// for 1024 samples, beside the 620 us of 1024 steps (2000 steps at L = 64, every step sampled: 1.41 ms with
+// the additions after each chunk, 1.36 here, 1.33 with a short last chunk).
 template <int SPT>
 __global__ void __launch_bounds__(1024)
-k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, D1Run run, uint64_t t0, uint32_t n_steps) {
+k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t every, uint64_t t0, uint32_t n_steps,
+             int n_reps, uint32_t sum_ns, int sum_parts) {
   extern __shared__ __align__(16) double pop[];              // [2][3][nx]
+  if ((int)blockIdx.x >= n_reps) {
+    const int b = (int)blockIdx.x - n_reps;
+    d1q3_add_products(descs[b / sum_parts], ws, sum_ns, b % sum_parts, sum_parts);
+    return;
+  }
   const ReplicaDesc& d = descs[blockIdx.x];
   const int nx = d.nx, tid = (int)threadIdx.x, nt = (int)blockDim.x;
   const double* src = reinterpret_cast<const double*>(ws + d.off_pop[t0 & 1]);
@@ -87,13 +139,13 @@ k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, D1Run
     n1[k] = in && n_steps > 1 ? noise[nx + xs[k]] : 0.0;
   }
   // steps until the next sample (never without sampled fields)
-  uint32_t wait = run.every && d.n_fields ? (uint32_t)((run.every - t0 % run.every) % run.every) : 0xFFFFFFFFu;
+  uint32_t wait = every && d.n_fields ? (uint32_t)((every - t0 % every) % every) : 0xFFFFFFFFu;
   __syncthreads();
   for (uint32_t s = 0; s < n_steps; ++s) {
     const double* in = pop + (s & 1) * 3 * nx;
     double* out = pop + ((s & 1) ^ 1) * 3 * nx;
     const bool sample = wait == 0;
-    wait = sample ? run.every - 1 : wait - 1;
+    wait = sample ? every - 1 : wait - 1;
     const double* nn = noise + (int64_t)(s + 2) * nx;
 #pragma unroll
     for (int k = 0; k < SPT; ++k) {
@@ -124,7 +176,7 @@ k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, D1Run
 }
 
 // Block g = blockIdx.y of replica blockIdx.x takes the sample batches g, g + G, .. (G = gridDim.y) of the
-// chunk's ns samples and leaves its sums in partial row g; the block of the last batch writes its fields.
+// chunk's ns samples and leaves their products; the block of the last batch writes its fields.
 __global__ void __launch_bounds__(kD1SampleThreads)
 k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -138,9 +190,8 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint
   double2* X = z + SB * rows * ss;
   const double2* tw = reinterpret_cast<const double2*>(ws + d.off_tw_x);
   const double* raw = reinterpret_cast<const double*>(ws + d.off_d1_raw);
-  const int items = (int)d1q3_items(d);
-  double2* part = reinterpret_cast<double2*>(ws + d.off_d1_part) + (int64_t)blockIdx.y * items;
-  bool first = true;
+  double* prod = reinterpret_cast<double*>(ws + d.off_d1_prod);
+  const int64_t np = d1q3_products(nx, F);
   for (uint32_t b0 = blockIdx.y * SB; b0 < ns; b0 += gridDim.y * SB) {
     const int nb = (int)min((uint32_t)SB, ns - b0), nq = nb * rows;             // samples, packed rows
     const bool last = b0 + nb == ns;
@@ -172,65 +223,35 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint
       if (fa + 1 < F) o[hn1] = make_double2(0.5 * (Zk.y + Zm.y), 0.5 * (Zm.x - Zk.x));
     }
     __syncthreads();
-    for (int it = tid; it < items; it += nt) {
-      double2 acc = first ? make_double2(0.0, 0.0) : part[it];
-      const int pr = it / hn1, k = it - pr * hn1;
-      if (pr < d.n_pairs) {
-        const double2* xa = X + (int64_t)d.pair_a[pr] * hn1 + k;
-        const double2* xb = X + (int64_t)d.pair_b[pr] * hn1 + k;
-        const bool cross = d.pair_a[pr] != d.pair_b[pr];
-        if (!FLB_INB(d.pair_a[pr] < F && d.pair_b[pr] < F, 182)) continue;
-        for (int b = 0; b < nb; ++b) {
-          const double2 A = xa[(int64_t)b * F * hn1], Bv = xb[(int64_t)b * F * hn1];
-          acc.x += A.x * Bv.x + A.y * Bv.y;                                      // X_a X_b^*
-          if (cross) acc.y += A.y * Bv.x - A.x * Bv.y;
+    // one item per (pair, sample, k), then the k = 0 values
+    const int body = d.n_pairs * nb * hn1;
+    for (int it = tid; it < body + nb * F; it += nt) {
+      if (it < body) {
+        const int row = it / hn1, k = it - row * hn1, pr = row / nb, b = row - pr * nb;
+        const int fa = d.pair_a[pr], fb = d.pair_b[pr];
+        if (!FLB_INB(fa < F && fb < F, 182)) continue;
+        const double2 A = X[((int64_t)b * F + fa) * hn1 + k], B = X[((int64_t)b * F + fb) * hn1 + k];
+        double* o = prod + (b0 + b) * np + d1q3_pair_first(nx, pr, fa, fb);
+        if (fa == fb) {
+          o[k] = A.x * A.x + A.y * A.y;
+        } else {                                                                 // X_a X_b^*
+          o[2 * k] = A.x * B.x + A.y * B.y;
+          o[2 * k + 1] = A.y * B.x - A.x * B.y;
         }
-      } else {                                                                   // X_f(0) of field it - n_pairs hn1
-        const int f = it - d.n_pairs * hn1;
-        for (int b = 0; b < nb; ++b) acc.x += X[((int64_t)b * F + f) * hn1].x;
+      } else {
+        const int b = (it - body) / F, f = it - body - b * F;
+        prod[(b0 + b + 1) * np - F + f] = X[((int64_t)b * F + f) * hn1].x;
       }
-      part[it] = acc;
     }
-    first = false;
     __syncthreads();
   }
 }
 
-// The partial sums of blocks 0 .. used - 1 (used: the blocks that had a batch), a warp per item, added
-// to the replica's sums.
-__global__ void __launch_bounds__(256)
-k_d1q3_finish(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns, int blocks) {
-  const ReplicaDesc& d = descs[blockIdx.x];
-  const int F = (int)d.n_fields, hn1 = d.nx / 2 + 1, lane = (int)threadIdx.x & 31;
-  if (!F) return;
-  const int SB = d1_batch_of(d.nx, F, ns, blocks), items = (int)d1q3_items(d);
-  const int used = (int)min((uint32_t)blocks, (ns + SB - 1) / SB);
-  const double2* part = reinterpret_cast<const double2*>(ws + d.off_d1_part);
-  for (int it = (int)(blockIdx.y * blockDim.x + threadIdx.x) >> 5; it < items; it += (int)(gridDim.y * blockDim.x) >> 5) {
-    double2 v = make_double2(0.0, 0.0);
-    for (int g = lane; g < used; g += 32) {
-      const double2 p = part[(int64_t)g * items + it];
-      v.x += p.x;
-      v.y += p.y;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-      v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-    }
-    if (lane) continue;
-    const int pr = it / hn1, k = it - pr * hn1;
-    if (pr < d.n_pairs) {
-      if (d.pair_a[pr] == d.pair_b[pr]) {
-        reinterpret_cast<double*>(ws + d.pair_off[pr])[k] += v.x;
-      } else {
-        double2* a = reinterpret_cast<double2*>(ws + d.pair_off[pr]) + k;
-        const double2 s = *a;
-        *a = make_double2(s.x + v.x, s.y + v.y);
-      }
-    } else {
-      reinterpret_cast<double*>(ws + d.off_mean0)[it - d.n_pairs * hn1] += v.x;
-    }
-  }
+// The products of the last chunk of a run.
+constexpr int kD1SumThreads = 64;
+__global__ void __launch_bounds__(kD1SumThreads)
+k_d1q3_sums(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns) {
+  d1q3_add_products(descs[blockIdx.x], ws, ns, (int)blockIdx.y, (int)gridDim.y);
 }
 
 cudaError_t set_d1q3_runs_smem() {
@@ -241,12 +262,25 @@ cudaError_t set_d1q3_runs_smem() {
   return e;
 }
 
+// additions by themselves (a run's last chunk; every chunk of a large batch)
+cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint32_t ns,
+                             cudaStream_t st, int* launches) {
+  if (!ns) return cudaSuccess;
+  k_d1q3_sums<<<dim3(n_reps, (unsigned)((run.max_products + kD1SumThreads - 1) / kD1SumThreads)), kD1SumThreads, 0, st>>>(
+      descs, ws, ns);
+  const cudaError_t e = cudaGetLastError();
+  if (!e) ++*launches;
+  return e;
+}
+
 // One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= run.chunk) of all replicas (run.max_nx <=
-// kD1MaxSites); adds the launches to *launches.  Replicas are in the grids' x (up to 2^31 - 1; y ends at
-// 65535).  A launch that is refused ends the chunk: its first kernel writes scratch alone, so the
-// state stays as it was when that one fails.
+// kD1MaxSites), and the additions of the chunk before (*pending samples).  While the steps leave SMs
+// idle the chunk leaves its own additions in *pending, for the next one or launch_d1q3_sums; on large
+// batches they follow at once.  Adds the launches to *launches.  Replicas are in the grids' x (up to
+// 2^31 - 1; y ends at 65535).  A launch that is refused ends the chunk: its first kernel writes scratch
+// alone, so the state stays as it was when that one fails.
 cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0,
-                              uint32_t n_steps, int sms, cudaStream_t st, int* launches) {
+                              uint32_t n_steps, int sms, cudaStream_t st, uint32_t* pending, int* launches) {
   const int64_t most = (int64_t)n_steps * run.max_nx;
   cudaError_t e;
   k_d1q3_noise<<<dim3(n_reps, (unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms)), 256, 0, st>>>(
@@ -254,24 +288,30 @@ cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, co
   if ((e = cudaGetLastError())) return e;
   ++*launches;
   const size_t smem = d1q3_steps_smem(run.max_nx);
+  const int block = run.max_nx <= 1024 ? (run.max_nx + 31) & ~31 : 1024;
+  const int64_t parts = (run.max_products + block - 1) / block;
+  const bool beside = n_reps * (1 + parts) <= sms;
+  const int grid = n_reps + (*pending ? (int)(n_reps * parts) : 0);      // (left pending only where `beside` holds)
   if (run.max_nx <= 1024)
-    k_d1q3_steps<1><<<n_reps, (run.max_nx + 31) & ~31, smem, st>>>(descs, ws, run, t0, n_steps);
+    k_d1q3_steps<1><<<grid, block, smem, st>>>(descs, ws, run.every, t0, n_steps, n_reps, *pending, (int)parts);
   else
-    k_d1q3_steps<kD1SitesPerThread><<<n_reps, 1024, smem, st>>>(descs, ws, run, t0, n_steps);
+    k_d1q3_steps<kD1SitesPerThread><<<grid, block, smem, st>>>(descs, ws, run.every, t0, n_steps, n_reps, *pending,
+                                                               (int)parts);
   if ((e = cudaGetLastError())) return e;
   ++*launches;
+  *pending = 0;
   uint32_t ns = 0;
   if (run.every) {             // samples at the steps t in [t0, t0 + n_steps) with t % every == 0
     const uint64_t first = (t0 + run.every - 1) / run.every * run.every;
     if (first < t0 + n_steps) ns = (uint32_t)((t0 + n_steps - 1 - first) / run.every + 1);
   }
   if (!ns || !run.sample_smem) return cudaSuccess;
-  k_d1q3_sample<<<dim3(n_reps, run.blocks), kD1SampleThreads, run.sample_smem, st>>>(descs, ws, ns);
+  const int blocks = std::max(1, sms / n_reps);                   // of the sampling kernel, per replica
+  k_d1q3_sample<<<dim3(n_reps, blocks), kD1SampleThreads, run.sample_smem, st>>>(descs, ws, ns);
   if ((e = cudaGetLastError())) return e;
   ++*launches;
-  k_d1q3_finish<<<dim3(n_reps, (unsigned)((run.max_items + 7) / 8)), 256, 0, st>>>(descs, ws, ns, run.blocks);
-  if ((e = cudaGetLastError())) return e;
-  ++*launches;
+  if (!beside) return launch_d1q3_sums(descs, n_reps, ws, run, ns, st, launches);
+  *pending = ns;
   return cudaSuccess;
 }
 

@@ -54,6 +54,40 @@ def test_sampled_lattices_of_every_size_run_in_chunks(nx, fields):
                     assert na == nb == 23 and np.abs(ca - cb).max() <= 1e-13 * max(1.0, np.abs(cb).max()), (r, x, y)
 
 
+def _sums(sim, reps, r=0):
+    f = reps[r]["fields"]
+    return [sim.correlator(r, x, y) for i, x in enumerate(f) for y in f[i:]]
+
+
+@pytest.mark.parametrize("nx,fields", [(4, (0, 1)), (64, (0, 1, 2)), (64, (0, 1, 2, 9)), (1024, (1, 9))])
+@pytest.mark.parametrize("every", [1, 7])
+def test_sums_do_not_depend_on_calls_chunks_or_batch(nx, fields, every):
+    # a sum takes one product per sample in the order of the steps, whatever the launches: equal bit
+    # for bit for one call over several chunks (of at most 1024 steps), calls that end inside chunks and
+    # sampling periods, one step a call, per-step launches, and in a batch
+    p = _replica(nx, fields)
+    others = [_replica(128, (0, 2), stream=2), _replica(30, stream=3)]
+    n = 2100
+    a = Sim([p], precision="fp64")
+    assert 2 * 4 < _launches(a, n, every) < n                      # the chunked path, three chunks or more
+    ref, pop = _sums(a, [p]), a.populations()
+
+    def check(reps, runs, r=0, graphs=True):
+        s = Sim(reps, precision="fp64")
+        s.set_graphs(graphs)
+        for k in runs:
+            s.run(k, every)
+        assert np.array_equal(s.populations(r), pop)
+        for x, y in zip(_sums(s, reps, r), ref):
+            assert np.array_equal(x, y)
+        s.close()
+
+    check([p], (n // 2, n - n // 2))
+    check([p], (1,) * 40 + (n - 40,))
+    check([p], (n,), graphs=False)
+    check(others + [p], (5, 1030, n - 1035), r=2)
+
+
 def test_more_replicas_than_a_grid_dimension():
     # 65,535 blocks is the limit of a grid in y and z, 2^31 - 1 in x
     n, pick = 65_540, (0, 65_534, 65_535, 65_536, 65_539)
