@@ -7,6 +7,8 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <tuple>
+#include <utility>
 #include <vector>
 
 #include <complex>
@@ -56,9 +58,11 @@ cudaError_t launch_d1q3_fused(const ReplicaDesc* descs, int n_reps, char* ws, ui
 size_t d1q3_steps_smem(int nx);
 size_t d1q3_sample_smem(int nx, int F);
 cudaError_t set_d1q3_runs_smem();
-cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0,
-                              uint32_t n_steps, int sms, cudaStream_t st, uint32_t* pending, int* launches);
-cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint32_t pending,
+bool d1q3_sums_beside(const D1Group& g, int sms);
+cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t every,
+                              uint64_t t0, uint32_t n_steps, bool beside, int sms, cudaStream_t st,
+                              uint32_t* pending, int* launches);
+cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t ns,
                              cudaStream_t st, int* launches);
 // D3Q15 / D3Q19 (lb_3d.cu), q = 15 or 19
 void launch_step3(int q, int precision, int vec, const StepLaunch& L, bool sample, cudaStream_t st);
@@ -133,8 +137,15 @@ static constexpr int kMaxPointItems = 2048;    // 3D direct transforms: fields x
 static constexpr int kStepBlock = 256;
 static constexpr int64_t kVec4Sites = 1 << 20;
 static constexpr size_t kFusedSmemMax = 200 * 1024;           // D1Q3 runs: shared memory of a block
-static constexpr int64_t kD1ScratchBytes = 64 << 20;
-static constexpr uint32_t kD1LastSamples = 128;
+// FP64 D1Q3 runs: steps of a chunk at most; samples left to a run's last chunk; replicas and sites that
+// close a group (two blocks of 1024 threads on each of 152 SMs; 16 warps keep an SM's FP64 pipe busy); scratch
+// of a chunk: half of L2, so that what a chunk's kernels hand on stays there, or up to four times that
+// for 16 sampled steps of the largest group (2000 replicas of 1024 sites, four fields, every step sampled:
+// 747 us a step in these groups, 8 steps a chunk; 1426 in groups of 80 replicas; 732 as one group
+// with 1.2 GB).
+static constexpr uint32_t kD1Chunk = 1024, kD1LastSamples = 128;
+static constexpr int kD1GroupReplicas = 304;
+static constexpr int64_t kD1GroupSites = 80 * 1024, kD1ScratchBytes = 64 << 20;
 
 struct Layout {
   std::vector<ReplicaDesc> desc;
@@ -152,7 +163,8 @@ struct Layout {
   int fold = 1;               // 2: two spectrum slots, two samples per accumulation pass
   int max_fields = 0;         // the most sampled fields of a replica with pair sums
   int max_len = 1;            // the longest column transform
-  D1Run d1;                   // FP64 D1Q3: chunked runs (chunk = 0: not used)
+  std::vector<D1Group> d1_groups;        // FP64 D1Q3: chunked runs by groups of replicas (empty: not used)
+  int64_t off_d1 = 0, d1_bytes = 0;      // their scratch
   int staged = 0;             // 1: the step kernel of lb_step_bulk.cu (tiles of 256 vec sites)
   bool any_fields = false;
 };
@@ -401,6 +413,20 @@ static void plan_step(int lattice, int vec, int staged, Layout& L) {
   }
 }
 
+// Scratch areas of chunks of `steps` FP64 D1Q3 steps sampled every `every` (0: not), for any group of the
+// context, and their bytes.
+static std::pair<D1Scratch, int64_t> d1_scratch(const Layout& L, uint32_t steps, uint32_t every) {
+  D1Scratch sc{};
+  int64_t sites = 0, products = 0;
+  for (const D1Group& g : L.d1_groups) { sites = std::max(sites, g.sites); products = std::max(products, g.products); }
+  sc.steps = steps;
+  sc.samples = every && products ? (steps + every - 1) / every : 0;
+  sc.noise = L.off_d1;
+  sc.raw = align256(sc.noise + 8 * sites * steps);
+  sc.products = align256(sc.raw + 24 * sites * sc.samples);
+  return {sc, align256(sc.products + 8 * products * sc.samples) - L.off_d1};
+}
+
 static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   int rc = validate(precision, reps, n);
   if (rc) return rc;
@@ -491,27 +517,37 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
     }
   }
   if (lat == FLB_D1Q3 && precision == FLB_FP64) {
-    D1Run& run = L.d1;
-    size_t steps_smem = 0;
-    int64_t step_bytes = 0;                      // scratch of a sampled step of all replicas
-    for (const ReplicaDesc& d : L.desc) {
-      step_bytes += 8 * (int64_t)d.nx;
-      run.max_nx = std::max(run.max_nx, (int)d.nx);
-      steps_smem = std::max(steps_smem, d1q3_steps_smem(d.nx));
-      if (!d.n_fields) continue;
-      step_bytes += 24 * (int64_t)d.nx + 8 * d1q3_products(d.nx, (int)d.n_fields);
-      run.max_products = std::max(run.max_products, d1q3_products(d.nx, (int)d.n_fields));
-      run.sample_smem = std::max(run.sample_smem, d1q3_sample_smem(d.nx, (int)d.n_fields));
-    }
-    if (run.max_nx <= kD1MaxSites && steps_smem <= kFusedSmemMax && run.sample_smem <= kFusedSmemMax) {
-      // a chunk's noise, pulled populations and products in at most kD1ScratchBytes (or four steps), 1024 steps at most
-      run.chunk = (uint32_t)std::max<int64_t>(4, std::min<int64_t>(1024, kD1ScratchBytes / step_bytes));
-      for (ReplicaDesc& d : L.desc) {
-        d.off_d1_noise = off; off = align256(off + 8 * (int64_t)run.chunk * d.nx);
-        if (!d.n_fields) continue;
-        d.off_d1_raw = off; off = align256(off + 24 * (int64_t)run.chunk * d.nx);
-        d.off_d1_prod = off; off = align256(off + 8 * (int64_t)run.chunk * d1q3_products(d.nx, (int)d.n_fields));
+    int64_t sites = 0, products = 0;
+    bool fit = true;
+    for (int r = 0; r < n; ++r) {
+      ReplicaDesc& d = L.desc[r];
+      const int F = (int)d.n_fields;
+      d.d1_site0 = sites;
+      d.d1_product0 = products;
+      if (L.d1_groups.empty() ||
+          (L.d1_groups.back().n >= kD1GroupReplicas && L.d1_groups.back().sites >= kD1GroupSites))
+        L.d1_groups.push_back(D1Group{r});
+      D1Group& g = L.d1_groups.back();
+      ++g.n;
+      g.sites += d.nx;
+      g.max_nx = std::max(g.max_nx, (int)d.nx);
+      if (F) {
+        g.products += d1q3_products(d.nx, F);
+        g.max_products = std::max(g.max_products, d1q3_products(d.nx, F));
+        g.sample_smem = std::max(g.sample_smem, d1q3_sample_smem(d.nx, F));
+        products += d1q3_products(d.nx, F);
       }
+      sites += d.nx;
+      fit = fit && g.max_nx <= kD1MaxSites && d1q3_steps_smem(g.max_nx) <= kFusedSmemMax && g.sample_smem <= kFusedSmemMax;
+    }
+    if (fit) {
+      // (one sampled step of the largest group is at most 304 replicas of 4096 sites with two fields or of
+      // 2048 with four, 60 MB)
+      L.d1_bytes = std::min({d1_scratch(L, kD1Chunk, 1).second, 4 * kD1ScratchBytes,
+                             std::max(kD1ScratchBytes, d1_scratch(L, 16, 1).second)});
+      L.off_d1 = off; off = align256(off + L.d1_bytes);
+    } else {
+      L.d1_groups.clear();
     }
   }
   // one-pass columns apart from their pair sums, from kSplitPoints points of the launch
@@ -957,7 +993,7 @@ int flb_create(int precision, const flb_replica* reps, int n_replicas, void* dev
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
   if ((rc = cuda_check(set_fft_smem_limits(), "smem limits"))) { delete c; return rc; }
-  if (c->L.d1.chunk && (rc = cuda_check(set_d1q3_runs_smem(), "smem limits"))) { delete c; return rc; }
+  if (!c->L.d1_groups.empty() && (rc = cuda_check(set_d1q3_runs_smem(), "smem limits"))) { delete c; return rc; }
   if (c->lattice == FLB_D1Q3 && precision != FLB_FP64) {      // the fused kernel holds a replica in one block's shared memory
     size_t smem = 0;
     for (const ReplicaDesc& d : c->L.desc)
@@ -1155,39 +1191,51 @@ static int chunk_graph(flb_ctx* c, uint32_t len, uint32_t every, cudaGraphExec_t
   return FLB_OK;
 }
 
+// FP64 D1Q3: chunks of steps, their noise before and their sampling after the serial part (one sampled step
+// by itself: 27 us, as separate launches 17; two 28 and 29), group after group through one scratch.
+static int run_d1q3_chunks(flb_ctx* c, uint64_t n_steps, uint32_t every) {
+  NvtxRange chunk_range("flb D1Q3 chunks");
+  const Layout& L = c->L;
+  D1Scratch sc;
+  uint32_t chunk = kD1Chunk;
+  for (int64_t bytes; std::tie(sc, bytes) = d1_scratch(L, chunk, every), bytes > L.d1_bytes && chunk > 1;) chunk -= (chunk + 7) / 8;
+  const bool beside = L.d1_groups.size() == 1 && d1q3_sums_beside(L.d1_groups[0], c->sms);
+  int rc = FLB_OK, launches = 0;
+  uint32_t pending = 0;                        // samples of the last chunk whose products are not yet in the sums
+  for (uint64_t i = 0; i < n_steps && !rc;) {
+    const uint64_t left = n_steps - i;
+    uint32_t n = (uint32_t)std::min<uint64_t>(left, chunk);
+    // the additions of the last chunk have no steps beside them (58 ns a sample): leave it few samples,
+    // where that saves more than its other launches take (16 us)
+    if (beside && every && n == left && left / every > 4 * kD1LastSamples) n -= kD1LastSamples * every;
+    for (const D1Group& g : L.d1_groups) {
+      sc.site0 = L.desc[g.first].d1_site0;
+      sc.product0 = L.desc[g.first].d1_product0;
+      rc = cuda_check(launch_d1q3_chunk(descs_dev(c), g, c->ws, sc, every, c->step, n, beside, c->sms, c->stream,
+                                        &pending, &launches), "D1Q3 launch");
+      if (rc) break;
+    }
+    if (rc) break;
+    if (every) {
+      const uint64_t first = (c->step + every - 1) / every * every;
+      if (first < c->step + n) c->n_samples += (c->step + n - 1 - first) / every + 1;
+    }
+    c->step += n;
+    i += n;
+  }
+  if (!rc) rc = cuda_check(launch_d1q3_sums(descs_dev(c), L.d1_groups[0], c->ws, sc, pending, c->stream, &launches),
+                           "D1Q3 launch");
+  count_kernels(c, launches);
+  return rc;
+}
+
 int flb_run(flb_ctx* c, uint64_t n_steps, uint32_t sample_every) {
   NvtxRange range("flb_run");
   if (!c) return set_error(FLB_EINVAL, "ctx is NULL");
   const Layout& L = c->L;
   const bool sampling = sample_every && L.any_fields;
-  if (L.d1.chunk && c->use_graphs && !c->tc.base && n_steps > 1) {
-    // FP64 D1Q3: chunks of steps, their noise before and their sampling after the serial part (one
-    // sampled step by itself: 27 us, as separate launches 17; two 28 and 29)
-    NvtxRange chunk_range("flb D1Q3 chunks");
-    D1Run run = L.d1;
-    run.every = sampling ? sample_every : 0;
-    int rc = FLB_OK, launches = 0;
-    uint32_t pending = 0;                        // samples of the last chunk whose products are not yet in the sums
-    for (uint64_t i = 0; i < n_steps && !rc;) {
-      const uint64_t left = n_steps - i;
-      uint32_t n = (uint32_t)std::min<uint64_t>(left, run.chunk);
-      // the additions of the last chunk have no steps beside them (58 ns a sample): leave it few samples,
-      // where that saves more than its other launches take (16 us)
-      if (run.every && n == left && left / run.every > 4 * kD1LastSamples) n -= kD1LastSamples * run.every;
-      rc = cuda_check(launch_d1q3_chunk(descs_dev(c), c->n, c->ws, run, c->step, n, c->sms, c->stream, &pending,
-                                        &launches), "D1Q3 launch");
-      if (rc) break;
-      if (run.every) {
-        const uint64_t first = (c->step + run.every - 1) / run.every * run.every;
-        if (first < c->step + n) c->n_samples += (c->step + n - 1 - first) / run.every + 1;
-      }
-      c->step += n;
-      i += n;
-    }
-    if (!rc) rc = cuda_check(launch_d1q3_sums(descs_dev(c), c->n, c->ws, run, pending, c->stream, &launches), "D1Q3 launch");
-    count_kernels(c, launches);
-    return rc;
-  }
+  if (!L.d1_groups.empty() && c->use_graphs && !c->tc.base && n_steps > 1)
+    return run_d1q3_chunks(c, n_steps, sampling ? sample_every : 0);
   if (c->fused_smem && c->use_graphs && !c->tc.base) {
     // FP32 D1Q3: runs of up to kFusedChunk steps with their sampling in one launch
     NvtxRange fused_range("flb fused D1Q3 steps");

@@ -85,7 +85,7 @@ struct alignas(16) ReplicaDesc {
                                     // the column pass produces the points: [k1][kx / c][k2][kx % c]
                                     // (ky = k1 + N1 k2; kx padded to a multiple of c)
   double dco[kNumCoef];             // fco in FP64
-  int64_t off_d1_noise, off_d1_raw, off_d1_prod;   // FP64 D1Q3 runs: scratch (lb_d1q3_runs.cu)
+  int64_t d1_site0, d1_product0;    // FP64 D1Q3 runs: sites and products of a sample of the replicas before
 };
 constexpr int kStepHeadBytes = offsetof(ReplicaDesc, log2nx);
 static_assert(offsetof(ReplicaDesc, rkey) % 16 == 4 && offsetof(ReplicaDesc, fco) % 16 == 4, "see the head's comment");
@@ -224,12 +224,19 @@ struct TimeCorr {
 // Sites of a lattice that the FP64 D1Q3 run kernels take: one block of at most 1024 threads, up to
 // kD1SitesPerThread sites each.
 constexpr int kD1SitesPerThread = 4, kD1MaxSites = 1024 * kD1SitesPerThread;
-// A run of FP64 D1Q3 steps (lb_d1q3_runs.cu): steps per chunk and what its launches are sized by
-// (over the replicas of the context), sampling period (0: none).
-struct D1Run {
-  uint32_t chunk = 0, every = 0;
-  int max_nx = 0;
-  int64_t max_products = 0;
+// Scratch of a chunk of FP64 D1Q3 steps of a group of replicas (lb_d1q3_runs.cu): three areas (byte
+// offsets from the workspace base), each replica's part of them by the sites and products of the group's
+// replicas before it.
+struct D1Scratch {
+  int64_t noise, raw, products;      // [steps][nx], [samples][3][nx], [samples][d1q3_products] of a replica
+  int64_t site0, product0;           // of the group's first replica
+  uint32_t steps, samples;           // a chunk's, at most
+};
+// A group of replicas: what its launches are sized by (bytes of shared memory, products of a replica at
+// most) and its sites and products in all.
+struct D1Group {
+  int first = 0, n = 0, max_nx = 0;
+  int64_t max_products = 0, sites = 0, products = 0;
   size_t sample_smem = 0;
 };
 // products of a sample, in the order of the sums (lb_d1q3_runs.cu): F fields with themselves (one

@@ -51,14 +51,24 @@ __device__ __forceinline__ int d1_batch_of(int nx, int F, uint32_t ns, int block
 size_t d1q3_steps_smem(int nx) { return 6 * (size_t)nx * sizeof(double); }
 size_t d1q3_sample_smem(int nx, int F) { return d1_batch(nx, F) * d1_sample_bytes(nx, F); }
 
-// Scratch of a replica (ReplicaDesc::off_d1_*): noise [chunk][nx], pulled populations [samples][3][nx],
-// products [samples][d1q3_products] in the order of the replica's sums: the pairs (one double a wave
-// vector for a field with itself, two for two fields), then the k = 0 value of every field.
+// A replica's scratch: noise, pulled populations, and products in the order of its sums: the pairs (one
+// double a wave vector for a field with itself, two for two fields), then the k = 0 value of every field.
+__device__ __forceinline__ double* d1_noise(const ReplicaDesc& d, char* ws, const D1Scratch& sc) {
+  return reinterpret_cast<double*>(ws + sc.noise) + (d.d1_site0 - sc.site0) * sc.steps;
+}
+__device__ __forceinline__ double* d1_raw(const ReplicaDesc& d, char* ws, const D1Scratch& sc) {
+  return reinterpret_cast<double*>(ws + sc.raw) + (d.d1_site0 - sc.site0) * 3 * sc.samples;
+}
+__device__ __forceinline__ double* d1_products(const ReplicaDesc& d, char* ws, const D1Scratch& sc) {
+  return reinterpret_cast<double*>(ws + sc.products) + (d.d1_product0 - sc.product0) * sc.samples;
+}
+
 __global__ void __launch_bounds__(256)
-k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint64_t t0, uint32_t n_steps) {
+k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint64_t t0,
+             uint32_t n_steps) {
   const ReplicaDesc& d = descs[blockIdx.x];
   const int nx = d.nx;
-  double* out = reinterpret_cast<double*>(ws + d.off_d1_noise);
+  double* out = d1_noise(d, ws, sc);
   const uint32_t n = n_steps * (uint32_t)nx;
   for (uint32_t i = blockIdx.y * blockDim.x + threadIdx.x; i < n; i += gridDim.y * blockDim.x) {
     const uint32_t s = i / (uint32_t)nx;
@@ -68,8 +78,8 @@ k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint6
 
 // The ns samples' products added to a replica's sums, a thread per product, by block `part` of `parts`.
 // A thread's chain of ns dependent additions (58 ns each) bounds it, so its loads run a step ahead.
-__device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __restrict__ ws, uint32_t ns, int part,
-                                                  int parts) {
+__device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __restrict__ ws, const D1Scratch& sc,
+                                                  uint32_t ns, int part, int parts) {
   const int F = (int)d.n_fields, nx = d.nx;
   if (!F) return;
   const int64_t np = d1q3_products(nx, F);
@@ -82,7 +92,7 @@ __device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __
       while (pr > 0 && i < d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr])) --pr;
       sum = reinterpret_cast<double*>(ws + d.pair_off[pr]) + (i - d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr]));
     }
-    const double* p = reinterpret_cast<const double*>(ws + d.off_d1_prod) + i;
+    const double* p = d1_products(d, ws, sc) + i;
     double acc = *sum, v[8], w[8];
     uint32_t s = 0;
     if (ns >= 8) {
@@ -112,12 +122,12 @@ __device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __
 // the additions after each chunk, 1.36 here, 1.33 with a short last chunk).
 template <int SPT>
 __global__ void __launch_bounds__(1024)
-k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t every, uint64_t t0, uint32_t n_steps,
-             int n_reps, uint32_t sum_ns, int sum_parts) {
+k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t every,
+             uint64_t t0, uint32_t n_steps, int n_reps, uint32_t sum_ns, int sum_parts) {
   extern __shared__ __align__(16) double pop[];              // [2][3][nx]
   if ((int)blockIdx.x >= n_reps) {
     const int b = (int)blockIdx.x - n_reps;
-    d1q3_add_products(descs[b / sum_parts], ws, sum_ns, b % sum_parts, sum_parts);
+    d1q3_add_products(descs[b / sum_parts], ws, sc, sum_ns, b % sum_parts, sum_parts);
     return;
   }
   const ReplicaDesc& d = descs[blockIdx.x];
@@ -125,8 +135,8 @@ k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint3
   const double* src = reinterpret_cast<const double*>(ws + d.off_pop[t0 & 1]);
   for (int i = tid; i < 3 * nx; i += nt) pop[i] = src[i];
   const D1Coef coef(d);
-  const double* noise = reinterpret_cast<const double*>(ws + d.off_d1_noise);
-  double* raw = reinterpret_cast<double*>(ws + d.off_d1_raw);
+  const double* noise = d1_noise(d, ws, sc);
+  double* raw = d1_raw(d, ws, sc);
   int xs[SPT], xl[SPT], xr[SPT];
   double n0[SPT], n1[SPT];                                    // noise of this step and the next
 #pragma unroll
@@ -178,7 +188,7 @@ k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint3
 // Block g = blockIdx.y of replica blockIdx.x takes the sample batches g, g + G, .. (G = gridDim.y) of the
 // chunk's ns samples and leaves their products; the block of the last batch writes its fields.
 __global__ void __launch_bounds__(kD1SampleThreads)
-k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns) {
+k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t ns) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ReplicaDesc& d = descs[blockIdx.x];
   const int nx = d.nx, logn = d.log2nx, F = (int)d.n_fields, hn1 = nx / 2 + 1, tid = (int)threadIdx.x;
@@ -189,8 +199,8 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint
   double2* z = reinterpret_cast<double2*>(smem_raw);
   double2* X = z + SB * rows * ss;
   const double2* tw = reinterpret_cast<const double2*>(ws + d.off_tw_x);
-  const double* raw = reinterpret_cast<const double*>(ws + d.off_d1_raw);
-  double* prod = reinterpret_cast<double*>(ws + d.off_d1_prod);
+  const double* raw = d1_raw(d, ws, sc);
+  double* prod = d1_products(d, ws, sc);
   const int64_t np = d1q3_products(nx, F);
   for (uint32_t b0 = blockIdx.y * SB; b0 < ns; b0 += gridDim.y * SB) {
     const int nb = (int)min((uint32_t)SB, ns - b0), nq = nb * rows;             // samples, packed rows
@@ -250,8 +260,8 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint
 // The products of the last chunk of a run.
 constexpr int kD1SumThreads = 64;
 __global__ void __launch_bounds__(kD1SumThreads)
-k_d1q3_sums(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint32_t ns) {
-  d1q3_add_products(descs[blockIdx.x], ws, ns, (int)blockIdx.y, (int)gridDim.y);
+k_d1q3_sums(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t ns) {
+  d1q3_add_products(descs[blockIdx.x], ws, sc, ns, (int)blockIdx.y, (int)gridDim.y);
 }
 
 cudaError_t set_d1q3_runs_smem() {
@@ -263,54 +273,58 @@ cudaError_t set_d1q3_runs_smem() {
 }
 
 // additions by themselves (a run's last chunk; every chunk of a large batch)
-cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint32_t ns,
+cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t ns,
                              cudaStream_t st, int* launches) {
   if (!ns) return cudaSuccess;
-  k_d1q3_sums<<<dim3(n_reps, (unsigned)((run.max_products + kD1SumThreads - 1) / kD1SumThreads)), kD1SumThreads, 0, st>>>(
-      descs, ws, ns);
+  k_d1q3_sums<<<dim3(g.n, (unsigned)((g.max_products + kD1SumThreads - 1) / kD1SumThreads)), kD1SumThreads, 0, st>>>(
+      descs + g.first, ws, sc, ns);
   const cudaError_t e = cudaGetLastError();
   if (!e) ++*launches;
   return e;
 }
 
-// One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= run.chunk) of all replicas (run.max_nx <=
-// kD1MaxSites), and the additions of the chunk before (*pending samples).  While the steps leave SMs
-// idle the chunk leaves its own additions in *pending, for the next one or launch_d1q3_sums; on large
-// batches they follow at once.  Adds the launches to *launches.  Replicas are in the grids' x (up to
-// 2^31 - 1; y ends at 65535).  A launch that is refused ends the chunk: its first kernel writes scratch
-// alone, so the state stays as it was when that one fails.
-cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, int n_reps, char* ws, const D1Run& run, uint64_t t0,
-                              uint32_t n_steps, int sms, cudaStream_t st, uint32_t* pending, int* launches) {
-  const int64_t most = (int64_t)n_steps * run.max_nx;
+static int d1_block(const D1Group& g) { return g.max_nx <= 1024 ? (g.max_nx + 31) & ~31 : 1024; }
+static int64_t d1_sum_parts(const D1Group& g) { return (g.max_products + d1_block(g) - 1) / d1_block(g); }
+// do a chunk's additions run beside the next chunk's steps (on SMs that the steps leave idle)?
+bool d1q3_sums_beside(const D1Group& g, int sms) { return g.n * (1 + d1_sum_parts(g)) <= sms; }
+
+// One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= sc.steps) of a group (max_nx <= kD1MaxSites), sampled
+// every `every` (0: not), and the additions of the group's chunk before (*pending samples).  With `beside`
+// (the context's only group, and d1q3_sums_beside) the chunk leaves its own additions in *pending, for
+// the next one or launch_d1q3_sums; else they follow at once.  Adds the launches to *launches.  Replicas are in the grids' x
+// (up to 2^31 - 1; y ends at 65535).  A launch that is refused ends the chunk: its first kernel writes
+// scratch alone, so the state stays as it was when that one fails.
+cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t every,
+                              uint64_t t0, uint32_t n_steps, bool beside, int sms, cudaStream_t st,
+                              uint32_t* pending, int* launches) {
+  descs += g.first;
+  const int64_t most = (int64_t)n_steps * g.max_nx;
   cudaError_t e;
-  k_d1q3_noise<<<dim3(n_reps, (unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms)), 256, 0, st>>>(
-      descs, ws, t0, n_steps);
+  k_d1q3_noise<<<dim3(g.n, (unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms)), 256, 0, st>>>(
+      descs, ws, sc, t0, n_steps);
   if ((e = cudaGetLastError())) return e;
   ++*launches;
-  const size_t smem = d1q3_steps_smem(run.max_nx);
-  const int block = run.max_nx <= 1024 ? (run.max_nx + 31) & ~31 : 1024;
-  const int64_t parts = (run.max_products + block - 1) / block;
-  const bool beside = n_reps * (1 + parts) <= sms;
-  const int grid = n_reps + (*pending ? (int)(n_reps * parts) : 0);      // (left pending only where `beside` holds)
-  if (run.max_nx <= 1024)
-    k_d1q3_steps<1><<<grid, block, smem, st>>>(descs, ws, run.every, t0, n_steps, n_reps, *pending, (int)parts);
+  const size_t smem = d1q3_steps_smem(g.max_nx);
+  const int block = d1_block(g), parts = (int)d1_sum_parts(g);
+  const int grid = g.n + (*pending ? g.n * parts : 0);              // (left pending only where that is at most sms)
+  if (g.max_nx <= 1024)
+    k_d1q3_steps<1><<<grid, block, smem, st>>>(descs, ws, sc, every, t0, n_steps, g.n, *pending, parts);
   else
-    k_d1q3_steps<kD1SitesPerThread><<<grid, block, smem, st>>>(descs, ws, run.every, t0, n_steps, n_reps, *pending,
-                                                               (int)parts);
+    k_d1q3_steps<kD1SitesPerThread><<<grid, block, smem, st>>>(descs, ws, sc, every, t0, n_steps, g.n, *pending, parts);
   if ((e = cudaGetLastError())) return e;
   ++*launches;
   *pending = 0;
   uint32_t ns = 0;
-  if (run.every) {             // samples at the steps t in [t0, t0 + n_steps) with t % every == 0
-    const uint64_t first = (t0 + run.every - 1) / run.every * run.every;
-    if (first < t0 + n_steps) ns = (uint32_t)((t0 + n_steps - 1 - first) / run.every + 1);
+  if (every && g.sample_smem) {             // samples at the steps t in [t0, t0 + n_steps) with t % every == 0
+    const uint64_t first = (t0 + every - 1) / every * every;
+    if (first < t0 + n_steps) ns = (uint32_t)((t0 + n_steps - 1 - first) / every + 1);
   }
-  if (!ns || !run.sample_smem) return cudaSuccess;
-  const int blocks = std::max(1, sms / n_reps);                   // of the sampling kernel, per replica
-  k_d1q3_sample<<<dim3(n_reps, blocks), kD1SampleThreads, run.sample_smem, st>>>(descs, ws, ns);
+  if (!ns) return cudaSuccess;
+  const int blocks = std::max(1, sms / g.n);                   // of the sampling kernel, per replica
+  k_d1q3_sample<<<dim3(g.n, blocks), kD1SampleThreads, g.sample_smem, st>>>(descs, ws, sc, ns);
   if ((e = cudaGetLastError())) return e;
   ++*launches;
-  if (!beside) return launch_d1q3_sums(descs, n_reps, ws, run, ns, st, launches);
+  if (!beside) return launch_d1q3_sums(descs - g.first, g, ws, sc, ns, st, launches);
   *pending = ns;
   return cudaSuccess;
 }

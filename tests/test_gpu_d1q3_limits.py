@@ -88,6 +88,27 @@ def test_sums_do_not_depend_on_calls_chunks_or_batch(nx, fields, every):
     check(others + [p], (5, 1030, n - 1035), r=2)
 
 
+@pytest.mark.parametrize("sizes,every", [((1024,) * 310, 1), ((2048, 64, 4096, 30, 1024) * 70, 3), ((256,) * 700, 50),
+                                         ((512,) * 400, 0), ((4096, 4096, 4096, 4096) * 76 + (8,) * 9, 1)])
+def test_large_batches_run_in_groups_through_one_scratch(sizes, every):
+    # batches of several groups of replicas (of 304 and 81,920 sites or more), the last group small, whose
+    # chunks are shorter than the run (at most 256 MB of scratch); against single replicas, bit for bit
+    reps = [_replica(nx, () if nx == 30 else (0, 2)[: 1 + i % 2], seed=7, stream=i, init_mode=0, kT=1e-4)
+            for i, nx in enumerate(sizes)]
+    n = 150
+    sim = Sim(reps, precision="fp64")
+    assert _launches(sim, n, every) > 2 * 2
+    assert sim.workspace_bytes < 270e6 + 8000 * len(reps) + sum(sizes) * 8 * (6 + 2 + 8)   # state, fields, spectra, sums
+    for r in sorted({0, 1, 3, len(reps) // 2, len(reps) // 2 + 1, len(reps) - 2, len(reps) - 1}):
+        one = Sim(reps[r], precision="fp64")
+        one.run(n, every)
+        assert np.array_equal(sim.populations(r), one.populations()), r
+        if every and reps[r]["fields"]:
+            for x, y in zip(_sums(sim, reps, r), _sums(one, [reps[r]])):
+                assert np.array_equal(x, y), r
+        one.close()
+
+
 def test_more_replicas_than_a_grid_dimension():
     # 65,535 blocks is the limit of a grid in y and z, 2^31 - 1 in x
     n, pick = 65_540, (0, 65_534, 65_535, 65_536, 65_539)
