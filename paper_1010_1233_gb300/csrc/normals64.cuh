@@ -12,13 +12,18 @@
 //        (Tang, ACM TOMS 16, 1990): c ~ 1/m to 9 bits by the top 7 fraction bits of m, z = m c - 1
 //        exactly, |z| < 2^-7.7, -ln ua = (33 - e) ln 2 + ln c - ln(1 + z), the last by its Taylor
 //        series to z^7 (z^8 / 8 < 2^-64); result in Q59, or in Q63 for ua >= 1/2, where it can be
-//        small.
+//        small.  The last entry is c = 1/2 exactly, so that for ua >= 1 - 2^-8 the first two terms
+//        cancel and z = -(1 - ua) is all of the argument: it keeps its leading zeros apart (an even
+//        number of them), and the result has 61 significant bits however small it is.
 //   sqrt: a 23-bit reciprocal root y of the mantissa v, h = v y, e = 1 - h y, sqrt v = h / sqrt(1 - e)
 //        by its binomial series to e^2 (5/16 e^3 < 2^-61).
 //   sin, cos: 256 table angles (i + 1/2) 2 pi / 256 by the top 8 bits of ub, the remainder
 //        |delta| <= pi / 256 by Taylor series (errors below 2^-66) and the addition theorems.
-// The root-mean-square error of 3 10^6 random pairs is 4.7e-17, that of the final rounding (with
-// FP64 log and sqrt and correctly rounded sine and cosine 8.1e-17).
+// The result is the product of two fixed-point numbers and a power of two, so its error goes with r: at
+// most 1.2e-16 r for every scale of 1 - ua down to 2^-33 (2.9e-16 r with FP64 log and sqrt and correctly
+// rounded sine and cosine); where the sine or cosine is small it stays below 2^-60 r, but not below the
+// last bit of the product.  The root-mean-square error of 3 10^6 random pairs is 4.7e-17, that of the
+// final rounding (8.1e-17).
 #pragma once
 #include <cstdint>
 #ifdef __CUDACC__
@@ -34,7 +39,7 @@ namespace flb {
 
 struct alignas(16) Fx2 { uint64_t a, b; };
 
-// by the top 7 fraction bits of m: c = round(2^9 / (1 + (i + 1/2) / 128)) and -ln(c / 512) in Q63
+// by the top 7 fraction bits of m: c = round(2^9 / (1 + (i + 1/2) / 128)), the last 2^8, and -ln(c / 512) in Q63
 FLB_TAB Fx2 kFxLog[128] = {
   {510, 0x0080402acac459acull}, {506, 0x0182448a388a2aa2ull}, {502, 0x02865524b3019814ull},
   {498, 0x038c7a5d82955e32ull}, {495, 0x045278f90016a33bull}, {491, 0x055c571300f3bbb9ull},
@@ -78,7 +83,7 @@ FLB_TAB Fx2 kFxLog[128] = {
   {267, 0x5356750ff6ae87b3ull}, {266, 0x53d16a0d693864ecull}, {265, 0x544cd5999ff15ce5ull},
   {264, 0x54c8b89a19e15cccull}, {263, 0x554513f6f2f589d6ull}, {262, 0x55c1e89aee319981ull},
   {261, 0x563f377380130e38ull}, {260, 0x56bd0170d9277e99ull}, {259, 0x573b4785f0d71568ull},
-  {258, 0x57ba0aa89064808eull}, {257, 0x58394bd15e238dd5ull},
+  {258, 0x57ba0aa89064808eull}, {256, 0x58b90bfbe8e7bcd6ull},
 };
 
 // cos and sin of 2 pi (i + 1/2) / 256 in Q62 (two's complement)
@@ -247,12 +252,13 @@ FLB_HD uint64_t fx_mul64x32(uint64_t a, uint32_t b) {
   return (a >> 32) * b + (((a & 0xFFFFFFFFull) * b) >> 32);
 }
 
-// sqrt(-2 ln((w + 1/2) 2^-32)) in Q60
-FLB_HD int64_t fx_radius(uint32_t w) {
+// sqrt(-2 ln((w + 1/2) 2^-32)) = s 2^-(60 + k): returns s < 2^63
+FLB_HD int64_t fx_radius(uint32_t w, int& k) {
   const uint64_t x = 2 * (uint64_t)w + 1;
   const int e = 63 - fx_clz(x);                                   // 0 .. 32
   const uint64_t m = x << (32 - e);                               // Q32, [1, 2)
-  const Fx2 t = fx_load(&kFxLog[(m >> 25) & 127]);
+  const int i = (int)(m >> 25) & 127;
+  const Fx2 t = fx_load(&kFxLog[i]);
   const int64_t z = (int64_t)(m * (uint32_t)t.a) - (1ll << 41);   // Q41, exact, |z| < 2^33.3
   const int32_t zs = (int32_t)(z >> 3);                           // Q38
   // 1/4 - z (1/5 - z (1/6 - z / 7)) in Q32
@@ -262,11 +268,13 @@ FLB_HD int64_t fx_radius(uint32_t w) {
   const int64_t t3 = 0x1555555555555555ll - (((int64_t)zs * (int32_t)t4) >> 8);   // 1/3 - z t4, Q62
   const uint64_t t2 = (1ull << 63) - ((uint64_t)fx_mulhi_s((int64_t)((uint64_t)z << 22), t3) << 3);   // 1/2 - z t3, Q64
   const uint64_t az = (uint64_t)(z < 0 ? -z : z) << 23;           // |z|, Q64
-  const uint64_t q = fx_mulhi(fx_mulhi(az, az), t2);              // z^2 t2, Q64
-  const uint64_t l1 = ((uint64_t)z << 22) - (q >> 1);             // ln(1 + z), Q63 (two's complement)
+  // near: ln 2 - ln c = 0, and all from here is scaled by 2^sn
+  const bool top = e == 32;
+  const int sn = top && i == 127 ? fx_clz(az) & ~1 : 0;
+  const uint64_t q = fx_mulhi(az << sn, fx_mulhi(az, t2));        // z^2 t2, Q64
+  const uint64_t l1 = ((uint64_t)z << (22 + sn)) - (q >> 1);      // ln(1 + z), Q63 (two's complement)
   // ln 2 - ln m in Q63, the whole of -ln ua for ua >= 1/2; otherwise plus (32 - e) ln 2 in Q59
   const uint64_t f = 0x58b90bfbe8e7bcd6ull - t.b - l1;
-  const bool top = e == 32;
   const uint64_t a = top ? f : (f >> 4) + (uint64_t)(32 - e) * 0x058b90bfbe8e7bcdull;
   // sqrt(2 a 2^-59), a = v 2^-sh: 2^(3 - sh/2) sqrt(v 2^-64), two halvings fewer for Q63
   const int sh = fx_clz(a) & ~1;
@@ -286,7 +294,8 @@ FLB_HD int64_t fx_radius(uint32_t w) {
   const int32_t e32 = (int32_t)(er >> 16);                        // Q48
   const int64_t c = (er >> 1) + (int64_t)((((uint64_t)((int64_t)e32 * e32) >> 32) * 3) >> 3);   // e / 2 + 3/8 e^2
   const int64_t s = (int64_t)(h >> 1) + fx_mulhi_s((int64_t)(h >> 1), c);         // Q63
-  return s >> ((sh >> 1) + (top ? 2 : 0));
+  k = ((sh + sn) >> 1) + (top ? 2 : 0);
+  return s;
 }
 
 // cos and sin of 2 pi (w + 1/2) 2^-32 in Q62
@@ -313,12 +322,12 @@ FLB_HD void fx_sincos(uint32_t w, int64_t& c, int64_t& s) {
   s = S - (fx_mulhi_s(S, cm) >> 12) + (fx_mulhi_s(C, sn) >> 5);
 }
 
-// a Q58 value rounded to a double (assembled from its bits: a conversion would use the FP64 pipe)
-FLB_HD double fx_to_double(int64_t a) {
+// a 2^-p rounded to a double (assembled from its bits: a conversion would use the FP64 pipe)
+FLB_HD double fx_to_double(int64_t a, int p) {
   const uint64_t m = (uint64_t)(a < 0 ? -a : a);
   const int lz = fx_clz(m);
   const uint64_t t = m << (lz & 63);
-  uint64_t b = ((uint64_t)(1023 + 63 - 58 - 1 - lz) << 52) + (t >> 11) + ((t >> 10) & 1);
+  uint64_t b = ((uint64_t)(1023 + 63 - 1 - p - lz) << 52) + (t >> 11) + ((t >> 10) & 1);
   if (m == 0) b = 0;
   b |= (uint64_t)a & (1ull << 63);
 #ifdef __CUDA_ARCH__
@@ -332,11 +341,12 @@ FLB_HD double fx_to_double(int64_t a) {
 
 // Box-Muller on a word pair, FP64 results
 FLB_HD void fx_box_muller(uint32_t wa, uint32_t wb, double& n0, double& n1) {
-  const int64_t r = fx_radius(wa);                                // Q60, < 6.8
+  int k;
+  const int64_t r = fx_radius(wa, k);                             // r 2^-(60 + k) < 6.8
   int64_t c, s;
   fx_sincos(wb, c, s);
-  n0 = fx_to_double(fx_mulhi_s(r, c));                            // Q60 + Q62 - 64
-  n1 = fx_to_double(fx_mulhi_s(r, s));
+  n0 = fx_to_double(fx_mulhi_s(r, c), 58 + k);                    // 60 + k + 62 - 64
+  n1 = fx_to_double(fx_mulhi_s(r, s), 58 + k);
 }
 
 }  // namespace flb
