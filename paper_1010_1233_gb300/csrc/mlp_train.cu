@@ -12,7 +12,7 @@
 #include <algorithm>
 #include <cstring>
 
-#include "flb_internal.cuh"
+#include "fft_common.cuh"
 
 namespace flb {
 
@@ -163,12 +163,13 @@ k_mlp_fwd_stats(const float* __restrict__ Wg, const float* __restrict__ X, int B
 }
 
 // Pass 2 (one block, a warp per run): m_rc, the per-run loss and, from the Gram terms,
-// dL/dm_rc 2 / B (the factor of s_c in dL/ds_c of a sample) as a sum of two FP32; thread 0 then adds the per-run losses in order.  Lane c + 8 j (c < 6, j < 4) sums
-// channel c's partials j, j + 4, ..; all the loads of a run are in flight together.
+// dL/dm_rc 2 / B (the factor of s_c in dL/ds_c of a sample); thread 0 then adds the per-run losses in
+// order.  Lane c + 8 j (c < 6, j < 4) sums channel c's partials j, j + 4, ..; all the loads of a run are in
+// flight together.
 constexpr int kLossBlock = 512;
 __global__ void __launch_bounds__(kLossBlock)
 k_mlp_loss(const double* __restrict__ partial, int R, int B, int blocks_per_run, const double* __restrict__ gram,
-           double norm, double* __restrict__ m_out, float2* __restrict__ dm, double* __restrict__ loss_r,
+           double norm, double* __restrict__ m_out, double* __restrict__ dm, double* __restrict__ loss_r,
            double* __restrict__ loss) {
   const int lane = threadIdx.x & 31, c = lane & 7, j = lane >> 3;
   for (int r = threadIdx.x >> 5; r < R; r += blockDim.x >> 5) {
@@ -191,9 +192,7 @@ k_mlp_loss(const double* __restrict__ partial, int R, int B, int blocks_per_run,
     const double term = 2.0 * g * (m - 1.0) + (m - 1.0) * hd;
     if (lane < kO) {
       m_out[r * kO + c] = m;
-      const double d = norm * (2.0 * g + 2.0 * hd) * 2.0 / B;
-      const float hi = (float)d;
-      dm[r * kO + c] = make_float2(hi, isfinite(hi) ? (float)(d - (double)hi) : 0.f);
+      dm[r * kO + c] = norm * (2.0 * g + 2.0 * hd) * 2.0 / B;
     }
     double L = gm[0];
 #pragma unroll
@@ -259,7 +258,7 @@ __host__ __device__ inline int grad_blocks(int64_t n) {
 }
 
 __global__ void __launch_bounds__(kGradThreads, 2)
-k_mlp_grad(const float* __restrict__ Wg, const float* __restrict__ X, int R, int B, const float2* __restrict__ dm,
+k_mlp_grad(const float* __restrict__ Wg, const float* __restrict__ X, int R, int B, const double* __restrict__ dm,
            double* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* rows = reinterpret_cast<float*>(smem_raw + sizeof(TrainNet));
@@ -309,8 +308,8 @@ k_mlp_grad(const float* __restrict__ Wg, const float* __restrict__ X, int R, int
       o[kRowOne * kGradStride] = 1.f;
 #pragma unroll
       for (int k = 0; k < kO; ++k) {
-        const float2 d = dm[run * kO + k];
-        dout[k] = fmaf(d.x, sc[k], d.y * sc[k]);       // (d.x + d.y) s, rounded once to FP32
+        // in FP64: dL/dm alone may leave FP32's range (s = 1 + o is never subnormal, widen is exact)
+        dout[k] = (float)(dm[run * kO + k] * widen(sc[k]));
         o[(kRowDo + k) * kGradStride] = dout[k];
       }
       o[(kRowDo + 6) * kGradStride] = 0.f;
@@ -484,15 +483,16 @@ int flb_mlp_train_step(float* w_dev, float* adam_m_dev, float* adam_v_dev, int t
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   char* s = static_cast<char*>(scratch_dev);
   double* partial = reinterpret_cast<double*>(s + T.off_partial);
-  float2* dm = reinterpret_cast<float2*>(s + T.off_dm);
+  double* dm = reinterpret_cast<double*>(s + T.off_dm);
   double* part = reinterpret_cast<double*>(s + T.off_part);
   float* grad = grad_dev ? grad_dev : reinterpret_cast<float*>(s + T.off_grad);
   const double norm = 1.0 / ((double)R * P * K);
   cudaError_t e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
   if (e != cudaSuccess) return set_error(FLB_ECUDA, "flb_mlp_train_step: %s", cudaGetErrorString(e));
   k_mlp_fwd_stats<<<R * T.blocks_per_run, kTrainBlock, 0, st>>>(w_dev, x_dev, B, T.blocks_per_run, partial);
-  k_mlp_loss<<<1, std::min(kLossBlock, 32 * R), 0, st>>>(partial, R, B, T.blocks_per_run, gram_dev, norm, m_dev, dm,
-                                                         reinterpret_cast<double*>(s + T.off_lossr), loss_dev);
+  k_mlp_loss<<<1, R < kLossBlock / 32 ? 32 * R : kLossBlock, 0, st>>>(partial, R, B, T.blocks_per_run, gram_dev, norm,
+                                                                      m_dev, dm, reinterpret_cast<double*>(s + T.off_lossr),
+                                                                      loss_dev);
   const int blocks = grad_blocks((int64_t)R * B);
   k_mlp_grad<<<blocks, kGradThreads, kGradSmem, st>>>(w_dev, x_dev, R, B, dm, part);
   const float c1 = lr > 0.f ? 1.f - powf(beta1, (float)t) : 1.f, c2 = lr > 0.f ? 1.f - powf(beta2, (float)t) : 1.f;

@@ -1,0 +1,41 @@
+"""Range and precision of the gradient of the training step (csrc/mlp_train.cu, GPU).
+
+With W3 = 0 the outputs are s_c = 1 + b3_c for every input, and with a Gram matrix H = 0 the loss is
+linear in <s_c^2>: dL/ds_c of a sample is d_rc s_c with d_rc = 4 g_rc / (R 6 K B), so that the gradients of
+W3 and b3 are sums of known factors."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_1010_1233_gb300 import learned, workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _gradient(X, g, w, K):
+    """(gradient, d) for the slopes g (R, 6) of the loss."""
+    R, B = X.shape[:2]
+    gram = np.zeros((R, 43))
+    gram[:, 1:7] = g
+    _, _, grad = learned.Trainer(X, torch.tensor(gram, device="cuda"), K, w).loss_and_grad()
+    return grad, (1.0 / (float(R) * 6 * K)) * (2.0 * g) * 2.0 / B
+
+
+@pytest.mark.parametrize("d,s", [(1e-42, 2.0 ** 20), (3e-45, 2.0 ** 40), (1e-30, 1.0), (1e40, 2.0 ** -20)])
+def test_loss_slopes_outside_fp32(d, s):
+    # d_rc has FP64's range and precision; only the product d s is rounded to FP32.  Tolerance: hidden
+    # layers of ~70 FP32 operations, 70 x 2^-24 = 4e-6 of the largest value, and sums of one sign.
+    R, B, K = 2, 50, 7
+    X = np.stack([W.mlp_inputs(B, r) for r in range(R)]).astype(np.float32)
+    w = W.mlp_weights(3, out_scale=0.0)
+    w["W3"][:] = 0
+    w["b3"][:] = s - 1
+    g = np.outer([1.0, 0.7], [1, -1, 0.5, 2, -0.25, 1]) * d * R * 6 * K * B / 4
+    grad, d = _gradient(X, g, w, K)
+    w64 = {k: v.astype(np.float64) for k, v in w.items()}
+    h1 = np.maximum(X.astype(np.float64) @ w64["W1"].T + w64["b1"], 0)
+    h2 = np.maximum(h1 @ w64["W2"].T + w64["b2"], 0)
+    for name, want in (("b3", B * s * d.sum(0)), ("W3", s * np.einsum("rc,rbh->ch", d, h2))):
+        assert np.abs(grad[name] - want).max() <= 1e-5 * np.abs(want).max(), name
