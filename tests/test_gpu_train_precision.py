@@ -39,3 +39,38 @@ def test_loss_slopes_outside_fp32(d, s):
     h2 = np.maximum(h1 @ w64["W2"].T + w64["b2"], 0)
     for name, want in (("b3", B * s * d.sum(0)), ("W3", s * np.einsum("rc,rbh->ch", d, h2))):
         assert np.abs(grad[name] - want).max() <= 1e-5 * np.abs(want).max(), name
+
+
+@pytest.mark.parametrize("pairs,B", [(1000, 8), (3, 900), (200, 177)])
+def test_cancelling_sums(pairs, B):
+    # Runs in pairs of opposite slopes and almost the same inputs, so that each gradient of W3 is 10^-6 to
+    # 10^-9 of the sum of its terms' magnitudes.  Hidden unit h passes input h % 3 through (positive
+    # inputs, one-hot weights), so a term is the product of two known FP32 numbers and math.fsum of the
+    # FP64 products is the exact sum.
+    # Tolerance: half an ulp for the rounding to FP32, and of the sum of magnitudes gamma_n^2 for Dot2 on n
+    # terms (Ogita, Rump & Oishi, Prop. 5.5; gamma_n = n 2^-24 / (1 - n 2^-24)) and 2^-53 per FP64 addition
+    # of the blocks' two partials.  n: half of a block's samples, in groups of four.
+    R, N = 2 * pairs, 2 * pairs * B
+    rng = np.random.default_rng(pairs + B)
+    X = np.exp2(rng.uniform(-12, 6, (pairs, 2, B, 3))).astype(np.float32)
+    X[:, 1] = X[:, 0, ::-1]
+    few = rng.integers(0, B, pairs)
+    X[np.arange(pairs), 1, few] = np.nextafter(X[np.arange(pairs), 1, few], np.float32(np.inf))
+    X = X.reshape(R, B, 3)
+    w = {k: np.zeros_like(v) for k, v in W.mlp_weights(1).items()}
+    for h in range(32):
+        w["W1"][h, h % 3] = 1
+        w["W2"][h, h] = 1
+    g = np.tile(rng.uniform(0.5, 2, (pairs, 6)), 2).reshape(R, 6) * np.tile([[1.0], [-1.0]], (pairs, 1))
+    grad, d = _gradient(X, g, w, 11)
+    d = d.astype(np.float32).astype(np.float64)                      # dL/ds at s = 1
+    blocks = min(304, -(-N // 64))
+    n = 4 * (-(-(-(-N // blocks)) // 8)) + 4
+    gamma = n * 2.0 ** -24 / (1 - n * 2.0 ** -24)
+    for c in range(6):
+        for h in range(3):
+            t = (d[:, None, c] * X[:, :, h].astype(np.float64)).ravel()
+            want, size = math.fsum(t), np.abs(t).sum()
+            assert abs(want) < 1e-6 * size
+            tol = 2.0 ** -24 * abs(want) + (gamma * gamma + (2 * blocks + 16) * 2.0 ** -53) * size
+            assert (np.abs(grad["W3"][c, h::3] - want) <= tol).all(), (c, h, grad["W3"][c, h::3], want, tol)
