@@ -279,9 +279,13 @@ int flb_autotune(flb_ctx* ctx, int trials, int* vec_out, int* grid_out, int* sta
  * sampling), which removes the per-kernel launch cost on small lattices.  D1Q3
  * contexts (without time correlators) instead run up to 4096 steps and their
  * samples per launch of one fused kernel in FP32, one block per replica with its
- * state in shared memory, and in FP64 chunks of up to 1024 steps as four launches
- * (noise, steps, transforms and pair sums of the samples, their addition).  Results are identical to direct launches up to the
- * contraction of multiply-adds.  The captured graphs are dropped when the
+ * state in shared memory, and in FP64 (runs of two steps or more on lattices of up
+ * to 4096 sites) chunks of up to 1024 steps of a group of replicas as three or four
+ * launches: noise; steps; transforms and products of the samples; their addition,
+ * beside the next chunk's steps on small contexts.  Results are identical to direct
+ * launches up to the contraction of multiply-adds; the FP64 D1Q3 sums take the
+ * samples in the order of the steps and do not depend on how a run is cut into
+ * calls or on the other replicas.  The captured graphs are dropped when the
  * launch configuration or the network switch changes.  enable = 0 issues every
  * kernel of every step directly. */
 int flb_set_graphs(flb_ctx* ctx, int enable);

@@ -50,8 +50,8 @@ void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* v
                        int64_t n_vblocks, char* ws, int ncol, int grid, int block, int smem, cudaStream_t st,
                        int paths, int slot, int sms);
 void launch_wait_probe(DevStatus* status, long long limit, cudaStream_t st);   // lb_step_tc.cu
-// D1Q3 runs of steps with their sampling in one launch (lb_d1q3_fused.cu)
-size_t d1q3_fused_smem(int precision, int nx, int F);
+// FP32 D1Q3 runs of steps with their sampling in one launch (lb_d1q3_fused.cu)
+size_t d1q3_fused_smem(int nx, int F);
 cudaError_t launch_d1q3_fused(const ReplicaDesc* descs, int n_reps, char* ws, uint64_t t0,
                               uint32_t n_steps, uint32_t every, size_t smem, cudaStream_t st);
 // FP64 D1Q3 runs (lb_d1q3_runs.cu)
@@ -997,7 +997,7 @@ int flb_create(int precision, const flb_replica* reps, int n_replicas, void* dev
   if (c->lattice == FLB_D1Q3 && precision != FLB_FP64) {      // the fused kernel holds a replica in one block's shared memory
     size_t smem = 0;
     for (const ReplicaDesc& d : c->L.desc)
-      smem = std::max(smem, d1q3_fused_smem(precision, d.nx, (int)d.n_fields));
+      smem = std::max(smem, d1q3_fused_smem(d.nx, (int)d.n_fields));
     c->fused_smem = smem <= kFusedSmemMax ? smem : 0;
   }
   cudaStream_t st = c->stream;

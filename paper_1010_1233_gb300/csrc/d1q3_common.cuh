@@ -1,5 +1,5 @@
-// The D1Q3 step of one site, shared by the per-step kernel (lb_step.cu) and the fused
-// multi-step kernel (lb_d1q3_fused.cu).
+// The D1Q3 step of one site, shared by the per-step kernel (lb_step.cu), the fused FP32
+// multi-step kernel (lb_d1q3_fused.cu) and the FP64 run kernels (lb_d1q3_runs.cu).
 //
 // D1Q3: v = (0, +1, -1), w = (2/3, 1/6, 1/6), moments 1, sqrt3 v, (3 v^2 - 1)/sqrt2 (the
 // projection of the D2Q9 basis).  Pull streaming (Eq. 1) from src, relaxation of the one

@@ -265,9 +265,6 @@ struct StepLaunch {
 // (with recip's shorter reciprocal): D2Q9 256^2 (256 blocks, two on some SMs and one on others) 21.5 ->
 // 19.7, D3Q15 64 x 48 x 40 (480 blocks) 62 -> 57.
 inline int step_split(int64_t n_vblocks, int sms) { return n_vblocks < 8 * (int64_t)sms ? 2 : 0; }
-// flavour -> (descriptor in the constant bank, noise modes 1/2 compiled)
-// Programmatic dependent launch: the launch may start while the kernel before it runs (kernels that
-// wait for it with griddepcontrol.wait before they touch what it writes)
 // FP64 step kernels are launched early when two steps' blocks fit the GPU at once (per_sm blocks on
 // each SM), or when one step's do not: in between, the SMs that finish a step first take most of the
 // next one's blocks, and its FP64 work is uneven (256^2 with 12 blocks per SM: 24.5 us for 19.9).
@@ -275,6 +272,8 @@ inline bool early_ok(int64_t grid, int per_sm, int sms) {
   return 2 * grid <= (int64_t)per_sm * sms || grid > (int64_t)per_sm * sms;
 }
 constexpr int kEarlyThreads = kStepThreads / 4, kEarlyBlocks2 = 14, kEarlyBlocks3 = 8;
+// Programmatic dependent launch: the launch may start while the kernel before it runs (kernels that
+// wait for it with griddepcontrol.wait before they touch what it writes)
 struct EarlyLaunch {
   cudaLaunchAttribute at[1];
   cudaLaunchConfig_t cfg = {};
@@ -289,6 +288,7 @@ struct EarlyLaunch {
   }
   EarlyLaunch(const EarlyLaunch&) = delete;
 };
+// flavour -> (descriptor in the constant bank, noise modes 1/2 compiled)
 template <int FL> struct Flavor { static constexpr bool kOne = FL != 2, kGen = FL != 0; };
 
 // Shared-memory budget of the column transforms and their split rule: one pass of

@@ -22,8 +22,8 @@ __host__ __device__ constexpr size_t a16(size_t x) { return (x + 15) & ~size_t(1
 
 // Shared memory of one block: populations [2][3][nx], fields [F][nx], the packed row
 // [nx + 32] (complex), the row transforms [F][nx/2 + 1] (complex).
-size_t d1q3_fused_smem(int precision, int nx, int F) {
-  const size_t rs = precision == FLB_FP64 ? 8 : 4, cs = 2 * rs;
+size_t d1q3_fused_smem(int nx, int F) {
+  const size_t rs = sizeof(float), cs = 2 * rs;
   return a16(6 * (size_t)nx * rs) + a16((size_t)F * nx * rs) + a16(((size_t)nx + 32) * cs) +
          a16((size_t)F * (nx / 2 + 1) * cs);
 }
@@ -31,10 +31,10 @@ size_t d1q3_fused_smem(int precision, int nx, int F) {
 // Steps t0 .. t0 + n_steps - 1 of every replica (block r = replica r), sampling at the
 // steps with t % every == 0 (every = 0: none).  Reads the state from the population
 // buffer of parity t0 & 1 and leaves it in the buffer of parity (t0 + n_steps) & 1.
-template <typename R, bool DEV>
 __global__ void __launch_bounds__(kD1q3FusedThreads)
 k_d1q3_fused(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint64_t t0, uint32_t n_steps,
              uint32_t every) {
+  using R = float;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ReplicaDesc& d = descs[blockIdx.x];
   const int nx = d.nx, F = (int)d.n_fields, tid = (int)threadIdx.x, nt = (int)blockDim.x;
@@ -60,9 +60,9 @@ k_d1q3_fused(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint6
     const R* src = pop + (s & 1) * 3 * nx;
     R* dst = pop + ((s & 1) ^ 1) * 3 * nx;
     if (sample) {
-      for (int x = tid; x < nx; x += nt) d1q3_site<R, DEV, true>(d, src, dst, fld, nx, x, (uint32_t)t);
+      for (int x = tid; x < nx; x += nt) d1q3_site<R, true, true>(d, src, dst, fld, nx, x, (uint32_t)t);
     } else {
-      for (int x = tid; x < nx; x += nt) d1q3_site<R, DEV, false>(d, src, dst, nullptr, nx, x, (uint32_t)t);
+      for (int x = tid; x < nx; x += nt) d1q3_site<R, true, false>(d, src, dst, nullptr, nx, x, (uint32_t)t);
     }
     __syncthreads();
     if (!sample) continue;
@@ -93,7 +93,7 @@ k_d1q3_fused(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint6
             if (FLB_INB(i0 + q < nx, 181)) z[i0 + q + ((i0 + q) >> ps)] = v[q];
         }
         __syncthreads();
-        dit_fft<R, sizeof(R) == 4 ? 4 : 3>(z, logn, 1, 0, tw, 1, ps, 3);
+        dit_fft<R, 4>(z, logn, 1, 0, tw, 1, ps, 3);
       } else {
         for (int x = tid; x < nx; x += nt) {
           C<R> v;
@@ -160,10 +160,9 @@ k_d1q3_fused(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, uint6
 
 cudaError_t launch_d1q3_fused(const ReplicaDesc* descs, int n_reps, char* ws, uint64_t t0,
                               uint32_t n_steps, uint32_t every, size_t smem, cudaStream_t st) {
-  const cudaError_t e = cudaFuncSetAttribute(k_d1q3_fused<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+  const cudaError_t e = cudaFuncSetAttribute(k_d1q3_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e) return e;
-  k_d1q3_fused<float, true><<<n_reps, kD1q3FusedThreads, smem, st>>>(descs, ws, t0, n_steps, every);
+  k_d1q3_fused<<<n_reps, kD1q3FusedThreads, smem, st>>>(descs, ws, t0, n_steps, every);
   return cudaGetLastError();
 }
 

@@ -1,18 +1,17 @@
 // Runs of D1Q3 steps in FP64 with their correlator sampling.
 //
 // The lattices are small (L = 64 in the D1Q3 workload) and each step needs the one before, so a
-// run is a chain; what can be taken off the chain decides its time.  One block that did the
-// noise, the step, the row transforms and the pair sums of every step in turn took 10 - 12 us a
-// step at L = 64 with every step sampled, nearly all of it latency between barriers.  Here only
-// the step itself is serial, and the rest runs on the whole GPU before and after it, a chunk of
-// steps at a time:
+// run is a chain; what can be taken off the chain decides its time (all of it in one block: 10 - 12 us
+// a step at L = 64 with every step sampled, nearly all latency between barriers).  Only the step itself is
+// serial here, and the rest runs on the whole GPU before and after it, a chunk of steps at a time:
 //   k_d1q3_noise   the noise of every (step, site) of the chunk
 //   k_d1q3_steps   one block per replica: pull and collide, 15 FP64 instructions a site, one barrier
 //                  a step; the noise is loaded two steps ahead; at a sample the pulled
 //                  populations go to memory
 //   k_d1q3_sample  row transforms of all samples (radix-2 passes of fft_common.cuh, two fields
 //                  packed per complex row) and their pair products
-//   k_d1q3_sums    adds the products to the replica's sums, sample by sample
+//   k_d1q3_sums    adds the products to the replica's sums, sample by sample (on small batches blocks of
+//                  the next k_d1q3_steps do it)
 // Every sum takes the samples' products one at a time in the order of the steps, as the per-step
 // launches add them, so it does not depend on how runs are cut into calls and chunks or on the other
 // replicas of the context.

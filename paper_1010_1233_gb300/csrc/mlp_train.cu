@@ -249,7 +249,8 @@ constexpr int kGradGroup = 96, kGradGroups = 2, kGradThreads = kGradGroup * kGra
 constexpr int kGradTile = 176, kGradStride = 180;
 constexpr int kRowDz1 = 0, kRowDz2 = kRowDz1 + kH, kRowDo = kRowDz2 + kH, kRowX = kRowDo + 8, kRowOne = kRowX + 3;
 constexpr int kRowH1 = kRowOne + 1, kRowH2 = kRowH1 + kH, kGradRows = kRowH2 + kH;
-constexpr int kGradMaxBlocks = 304;          // two blocks on each of 152 SMs
+constexpr int kGradMaxBlocks = 304;          // two blocks on each of GB300's 152 SMs; a constant, so that the
+                                             // scratch size and the order of the sums do not follow the device
 constexpr size_t kGradSmem = sizeof(TrainNet) + sizeof(float) * kGradRows * kGradStride;
 static_assert(2 * (kGradSmem + 1024) <= 228 * 1024, "two blocks per SM");
 static_assert(kGradTile <= kGradThreads && kGradTile % 8 == 0 && kGradTile <= kGradStride, "one sample per thread");

@@ -269,21 +269,21 @@ k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
 // the 64-replica sweep 286 -> 231, 3 x 1024 x 2048 96 -> 73; whole runs: 256^2 with 9 fields FP32, 2000
 // steps with 200 samples, 11.5 -> 10.5 ms.
 
-// One block per (replica, field, tile of w columns): the columns transformed over y in place.
+// One block per (replica, field, tile of kColsT columns): the columns transformed over y in place.
 template <typename R>
 __global__ void __launch_bounds__(kColsBlock, sizeof(R) == 4 ? 4 : 2)
 k_fft_cols_t(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
-             int64_t n_vblocks, char* __restrict__ ws, int w, int slot) {
+             int64_t n_vblocks, char* __restrict__ ws, int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C<R>* s = reinterpret_cast<C<R>*>(smem_raw);
-  const int lw = 31 - __clz(w);
+  constexpr int w = kColsT, lw = 2;
+  static_assert(1 << lw == w, "log2 of the tile width");
   for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
     const int r = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[r];
     if (d.log2n1 || (sizeof(R) == 4 && cols16_b(d.ny))) continue;      // another kernel's replica
     const int tiles = (d.half_nx + w - 1) >> lw;
     const int local = (int)(vb - vb_begin[r]), f = local / tiles;
-    if (f >= (int)d.n_fields) continue;                 // (the prefix counts the narrowest tiles)
     const int kx0 = (local - f * tiles) << lw, ncl = min(w, d.half_nx - kx0);
     const int logn = d.log2ny, n = d.ny, total = n << lw;
     C<R>* col = reinterpret_cast<C<R>*>(ws + d.off_spec + slot * d.spec_slot) + (int64_t)f * n * d.wpitch + kx0;
@@ -559,9 +559,9 @@ int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb
   if (precision == FLB_FP64 || (paths & kColsGeneric)) {
     const int smem = kColsT * (max_len + 1) * (precision == FLB_FP64 ? 16 : 8);
     if (precision == FLB_FP64)
-      k_fft_cols_t<double><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, kColsT, slot);
+      k_fft_cols_t<double><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
     else
-      k_fft_cols_t<float><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, kColsT, slot);
+      k_fft_cols_t<float><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
     ++launches;
   }
   if (precision != FLB_FP64) {

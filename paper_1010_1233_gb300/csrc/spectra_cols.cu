@@ -313,8 +313,8 @@ k_fft_cols_acc16(const ReplicaDesc* __restrict__ descs, const int64_t* __restric
 }
 
 // One-pass columns of length L in place (the split accumulation, spectra.cu): one unit per (replica,
-// field, tile of kColsT columns), stage 1 from the spectrum, stage 2 back to it; blocks of kT16Units
-// units keep a warp or more per unit length.
+// field, tile of kColsT columns), stage 1 from the spectrum, stage 2 back to it; a block of
+// 256 threads takes as many units as it has threads for (kColsT B each).
 template <int B>
 __global__ void __launch_bounds__(256)
 k_fft_cols_t16(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
