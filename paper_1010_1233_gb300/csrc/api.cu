@@ -60,8 +60,8 @@ size_t d1q3_sample_smem(int nx, int F);
 cudaError_t set_d1q3_runs_smem();
 bool d1q3_sums_beside(const D1Group& g, int sms);
 cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t every,
-                              uint64_t t0, uint32_t n_steps, bool beside, int sms, cudaStream_t st,
-                              uint32_t* pending, int* launches);
+                              uint64_t t0, uint32_t n_steps, uint32_t noise_steps, bool beside, int sms,
+                              cudaStream_t st, uint32_t* pending, int* launches);
 cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t ns,
                              cudaStream_t st, int* launches);
 // D3Q15 / D3Q19 (lb_3d.cu), q = 15 or 19
@@ -137,13 +137,13 @@ static constexpr int kMaxPointItems = 2048;    // 3D direct transforms: fields x
 static constexpr int kStepBlock = 256;
 static constexpr int64_t kVec4Sites = 1 << 20;
 static constexpr size_t kFusedSmemMax = 200 * 1024;           // D1Q3 runs: shared memory of a block
-// FP64 D1Q3 runs: steps of a chunk at most; samples left to a run's last chunk; replicas and sites that
+// FP64 D1Q3 runs: steps of a chunk at most; samples from which a run's last chunk is cut; replicas and sites that
 // close a group (two blocks of 1024 threads on each of 152 SMs; 16 warps keep an SM's FP64 pipe busy); scratch
 // of a chunk: half of L2, so that what a chunk's kernels hand on stays there, or up to four times that
 // for 16 sampled steps of the largest group (2000 replicas of 1024 sites, four fields, every step sampled:
 // 747 us a step in these groups, 8 steps a chunk; 1426 in groups of 80 replicas; 732 as one group
 // with 1.2 GB).
-static constexpr uint32_t kD1Chunk = 1024, kD1LastSamples = 128;
+static constexpr uint32_t kD1Chunk = 1024, kD1SplitSamples = 450;
 static constexpr int kD1GroupReplicas = 304;
 static constexpr int64_t kD1GroupSites = 80 * 1024, kD1ScratchBytes = 64 << 20;
 
@@ -1201,18 +1201,22 @@ static int run_d1q3_chunks(flb_ctx* c, uint64_t n_steps, uint32_t every) {
   for (int64_t bytes; std::tie(sc, bytes) = d1_scratch(L, chunk, every), bytes > L.d1_bytes && chunk > 1;) chunk -= (chunk + 7) / 8;
   const bool beside = L.d1_groups.size() == 1 && d1q3_sums_beside(L.d1_groups[0], c->sms);
   int rc = FLB_OK, launches = 0;
+  uint32_t drawn = 0;                          // steps whose noise the scratch still holds
   uint32_t pending = 0;                        // samples of the last chunk whose products are not yet in the sums
   for (uint64_t i = 0; i < n_steps && !rc;) {
     const uint64_t left = n_steps - i;
     uint32_t n = (uint32_t)std::min<uint64_t>(left, chunk);
-    // the additions of the last chunk have no steps beside them (58 ns a sample): leave it few samples,
-    // where that saves more than its other launches take (16 us)
-    if (beside && every && n == left && left / every > 4 * kD1LastSamples) n -= kD1LastSamples * every;
+    const uint32_t noise_steps = drawn ? 0 : n;
+    // the additions of the last chunk have no steps beside them: leave it an eighth of the samples that are
+    // left (64 .. 128), where that saves more than its other launches take (L = 64, two fields, every
+    // step sampled: 589 steps 425 -> 415 us, 1000 steps 700 -> 673)
+    if (beside && every && n == left && left / every > kD1SplitSamples)
+      n -= (uint32_t)std::min<uint64_t>(128, std::max<uint64_t>(64, left / every / 8)) * every;
     for (const D1Group& g : L.d1_groups) {
       sc.site0 = L.desc[g.first].d1_site0;
       sc.product0 = L.desc[g.first].d1_product0;
-      rc = cuda_check(launch_d1q3_chunk(descs_dev(c), g, c->ws, sc, every, c->step, n, beside, c->sms, c->stream,
-                                        &pending, &launches), "D1Q3 launch");
+      rc = cuda_check(launch_d1q3_chunk(descs_dev(c), g, c->ws, sc, every, c->step, n, noise_steps, beside, c->sms,
+                                        c->stream, &pending, &launches), "D1Q3 launch");
       if (rc) break;
     }
     if (rc) break;
@@ -1222,6 +1226,8 @@ static int run_d1q3_chunks(flb_ctx* c, uint64_t n_steps, uint32_t every) {
     }
     c->step += n;
     i += n;
+    drawn = noise_steps ? noise_steps - n : drawn - n;
+    sc.noise_first = drawn ? n : 0;
   }
   if (!rc) rc = cuda_check(launch_d1q3_sums(descs_dev(c), L.d1_groups[0], c->ws, sc, pending, c->stream, &launches),
                            "D1Q3 launch");

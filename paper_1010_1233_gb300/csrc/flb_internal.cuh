@@ -231,6 +231,7 @@ struct D1Scratch {
   int64_t noise, raw, products;      // [steps][nx], [samples][3][nx], [samples][d1q3_products] of a replica
   int64_t site0, product0;           // of the group's first replica
   uint32_t steps, samples;           // a chunk's, at most
+  uint32_t noise_first;              // the chunk's first step in the noise area
 };
 // A group of replicas: what its launches are sized by (bytes of shared memory, products of a replica at
 // most) and its sites and products in all.

@@ -75,39 +75,32 @@ k_d1q3_noise(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const
   }
 }
 
-// The ns samples' products added to a replica's sums, a thread per product, by block `part` of `parts`.
-// A thread's chain of ns dependent additions (58 ns each) bounds it, so its loads run a step ahead.
+// The sum of product i (lb_d1q3_runs.cu's order).
+__device__ __forceinline__ double* d1_sum(const ReplicaDesc& d, char* __restrict__ ws, int64_t i, int64_t np) {
+  const int nx = d.nx;
+  if (i >= np - d.n_fields) return reinterpret_cast<double*>(ws + d.off_mean0) + (i - (np - d.n_fields));
+  int pr = d.n_pairs - 1;
+  while (pr > 0 && i < d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr])) --pr;
+  return reinterpret_cast<double*>(ws + d.pair_off[pr]) + (i - d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr]));
+}
+
+// The ns samples' products added to a replica's sums, a thread per product, by block `part` of `parts`:
+// beside steps, so a few loads ahead in registers do (58 ns a sample).
 __device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __restrict__ ws, const D1Scratch& sc,
                                                   uint32_t ns, int part, int parts) {
-  const int F = (int)d.n_fields, nx = d.nx;
-  if (!F) return;
-  const int64_t np = d1q3_products(nx, F);
+  if (!d.n_fields) return;
+  const int64_t np = d1q3_products(d.nx, (int)d.n_fields);
   for (int64_t i = (int64_t)part * blockDim.x + threadIdx.x; i < np; i += (int64_t)parts * blockDim.x) {
-    double* sum;
-    if (i >= np - F) {
-      sum = reinterpret_cast<double*>(ws + d.off_mean0) + (i - (np - F));
-    } else {
-      int pr = d.n_pairs - 1;
-      while (pr > 0 && i < d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr])) --pr;
-      sum = reinterpret_cast<double*>(ws + d.pair_off[pr]) + (i - d1q3_pair_first(nx, pr, d.pair_a[pr], d.pair_b[pr]));
-    }
+    double* sum = d1_sum(d, ws, i, np);
     const double* p = d1_products(d, ws, sc) + i;
-    double acc = *sum, v[8], w[8];
+    double acc = *sum;
     uint32_t s = 0;
-    if (ns >= 8) {
+    for (; s + 8 <= ns; s += 8) {
+      double v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = p[u * np];
-      for (; s + 16 <= ns; s += 8) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) w[u] = p[(s + 8 + u) * np];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, v[u]);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = w[u];
-      }
+      for (int u = 0; u < 8; ++u) v[u] = p[(s + u) * np];
 #pragma unroll
       for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, v[u]);
-      s += 8;
     }
     for (; s < ns; ++s) acc = __dadd_rn(acc, p[s * np]);
     *sum = acc;
@@ -117,8 +110,8 @@ __device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __
 // SPT sites per thread (x = tid + k blockDim): steps t0 .. t0 + n_steps - 1 of replica blockIdx.x,
 // state from the buffer of parity t0 & 1 to that of (t0 + n_steps) & 1.  The blocks from n_reps on add
 // the products of the chunk before (its sum_ns samples), sum_parts of them a replica: 60 us of a chain
-// for 1024 samples, beside the 620 us of 1024 steps (2000 steps at L = 64, every step sampled: 1.41 ms with
-// the additions after each chunk, 1.36 here, 1.33 with a short last chunk).
+// for 1024 samples, beside the 620 us of 1024 steps (2000 steps at L = 64, two fields, every step sampled:
+// 1.41 ms with the additions after each chunk, 1.34 here, 1.32 with a short last chunk).
 template <int SPT>
 __global__ void __launch_bounds__(1024)
 k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t every,
@@ -134,7 +127,7 @@ k_d1q3_steps(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const
   const double* src = reinterpret_cast<const double*>(ws + d.off_pop[t0 & 1]);
   for (int i = tid; i < 3 * nx; i += nt) pop[i] = src[i];
   const D1Coef coef(d);
-  const double* noise = d1_noise(d, ws, sc);
+  const double* noise = d1_noise(d, ws, sc) + (int64_t)sc.noise_first * nx;
   double* raw = d1_raw(d, ws, sc);
   int xs[SPT], xl[SPT], xr[SPT];
   double n0[SPT], n1[SPT];                                    // noise of this step and the next
@@ -256,11 +249,50 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, cons
   }
 }
 
-// The products of the last chunk of a run.
-constexpr int kD1SumThreads = 64;
+// The same as a kernel.  The time of a small batch is a thread's chain of dependent additions, 31 ns each
+// at best: their products come by asynchronous copies up to 64 samples ahead into slots of the thread's
+// own.  About 43 ns a sample (loads into registers 8 ahead 58, 32 ahead 50).
+constexpr int kD1SumThreads = 64, kD1SumBatch = 32, kD1SumStages = 3;
 __global__ void __launch_bounds__(kD1SumThreads)
 k_d1q3_sums(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t ns) {
-  d1q3_add_products(descs[blockIdx.x], ws, sc, ns, (int)blockIdx.y, (int)gridDim.y);
+  __shared__ double ring[kD1SumStages][kD1SumBatch][kD1SumThreads];
+  const ReplicaDesc& d = descs[blockIdx.x];
+  const int64_t np = d1q3_products(d.nx, (int)d.n_fields);
+  const int64_t i = (int64_t)blockIdx.y * kD1SumThreads + threadIdx.x;
+  if (!d.n_fields || i >= np) return;
+  const double* p = d1_products(d, ws, sc) + i;
+  const uint32_t batches = (ns + kD1SumBatch - 1) / kD1SumBatch;
+  auto fetch = [&](uint32_t b) {                    // (one group per batch, empty past the end)
+    if (b < batches) {
+#pragma unroll
+      for (int u = 0; u < kD1SumBatch; ++u) {
+        const uint32_t s = b * kD1SumBatch + u;
+        if (s < ns)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::
+                       "r"((uint32_t)__cvta_generic_to_shared(&ring[b % kD1SumStages][u][threadIdx.x])), "l"(p + s * np) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (uint32_t b = 0; b < kD1SumStages - 1; ++b) fetch(b);
+  double* sum = d1_sum(d, ws, i, np);
+  double acc = *sum;
+  for (uint32_t b = 0; b < batches; ++b) {
+    fetch(b + kD1SumStages - 1);                    // into the slots that batch b - 1 has left
+    asm volatile("cp.async.wait_group %0;" :: "n"(kD1SumStages - 1) : "memory");
+    const double (*r)[kD1SumThreads] = ring[b % kD1SumStages];
+    const uint32_t left = ns - b * kD1SumBatch;
+    if (left >= kD1SumBatch) {
+      double v[kD1SumBatch];
+#pragma unroll
+      for (int u = 0; u < kD1SumBatch; ++u) v[u] = r[u][threadIdx.x];
+#pragma unroll
+      for (int u = 0; u < kD1SumBatch; ++u) acc = __dadd_rn(acc, v[u]);
+    } else {
+      for (uint32_t u = 0; u < left; ++u) acc = __dadd_rn(acc, r[u][threadIdx.x]);
+    }
+  }
+  *sum = acc;
 }
 
 cudaError_t set_d1q3_runs_smem() {
@@ -287,22 +319,25 @@ static int64_t d1_sum_parts(const D1Group& g) { return (g.max_products + d1_bloc
 // do a chunk's additions run beside the next chunk's steps (on SMs that the steps leave idle)?
 bool d1q3_sums_beside(const D1Group& g, int sms) { return g.n * (1 + d1_sum_parts(g)) <= sms; }
 
-// One chunk: steps t0 .. t0 + n_steps - 1 (n_steps <= sc.steps) of a group (max_nx <= kD1MaxSites), sampled
+// One chunk: steps t0 .. t0 + n_steps - 1 of a group (max_nx <= kD1MaxSites), with the noise of noise_steps
+// steps drawn before them (at most sc.steps; 0: the noise area has it from sc.noise_first on), sampled
 // every `every` (0: not), and the additions of the group's chunk before (*pending samples).  With `beside`
 // (the context's only group, and d1q3_sums_beside) the chunk leaves its own additions in *pending, for
 // the next one or launch_d1q3_sums; else they follow at once.  Adds the launches to *launches.  Replicas are in the grids' x
 // (up to 2^31 - 1; y ends at 65535).  A launch that is refused ends the chunk: its first kernel writes
 // scratch alone, so the state stays as it was when that one fails.
 cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t every,
-                              uint64_t t0, uint32_t n_steps, bool beside, int sms, cudaStream_t st,
-                              uint32_t* pending, int* launches) {
+                              uint64_t t0, uint32_t n_steps, uint32_t noise_steps, bool beside, int sms,
+                              cudaStream_t st, uint32_t* pending, int* launches) {
   descs += g.first;
-  const int64_t most = (int64_t)n_steps * g.max_nx;
   cudaError_t e;
-  k_d1q3_noise<<<dim3(g.n, (unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms)), 256, 0, st>>>(
-      descs, ws, sc, t0, n_steps);
-  if ((e = cudaGetLastError())) return e;
-  ++*launches;
+  if (noise_steps) {
+    const int64_t most = (int64_t)noise_steps * g.max_nx;
+    k_d1q3_noise<<<dim3(g.n, (unsigned)std::min<int64_t>((most + 255) / 256, 8 * (int64_t)sms)), 256, 0, st>>>(
+        descs, ws, sc, t0, noise_steps);
+    if ((e = cudaGetLastError())) return e;
+    ++*launches;
+  }
   const size_t smem = d1q3_steps_smem(g.max_nx);
   const int block = d1_block(g), parts = (int)d1_sum_parts(g);
   const int grid = g.n + (*pending ? g.n * parts : 0);              // (left pending only where that is at most sms)
