@@ -63,7 +63,7 @@ cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, const D1Group& g, char* 
                               uint64_t t0, uint32_t n_steps, uint32_t noise_steps, bool beside, int sms,
                               cudaStream_t st, uint32_t* pending, int* launches);
 cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t ns,
-                             cudaStream_t st, int* launches);
+                             bool beside, cudaStream_t st, int* launches);
 // D3Q15 / D3Q19 (lb_3d.cu), q = 15 or 19
 void launch_step3(int q, int precision, int vec, const StepLaunch& L, bool sample, cudaStream_t st);
 void launch_init3(int q, int precision, const ReplicaDesc* descs, int r, char* ws, int mode, const double* feq0,
@@ -141,7 +141,7 @@ static constexpr size_t kFusedSmemMax = 200 * 1024;           // D1Q3 runs: shar
 // close a group (two blocks of 1024 threads on each of 152 SMs; 16 warps keep an SM's FP64 pipe busy); scratch
 // of a chunk: half of L2, so that what a chunk's kernels hand on stays there, or up to four times that
 // for 16 sampled steps of the largest group (2000 replicas of 1024 sites, four fields, every step sampled:
-// 747 us a step in these groups, 8 steps a chunk; 1426 in groups of 80 replicas; 732 as one group
+// 730 us a step in these groups, 8 steps a chunk; 1426 in groups of 80 replicas; 732 as one group
 // with 1.2 GB).
 static constexpr uint32_t kD1Chunk = 1024, kD1SplitSamples = 450;
 static constexpr int kD1GroupReplicas = 304;
@@ -1229,8 +1229,8 @@ static int run_d1q3_chunks(flb_ctx* c, uint64_t n_steps, uint32_t every) {
     drawn = noise_steps ? noise_steps - n : drawn - n;
     sc.noise_first = drawn ? n : 0;
   }
-  if (!rc) rc = cuda_check(launch_d1q3_sums(descs_dev(c), L.d1_groups[0], c->ws, sc, pending, c->stream, &launches),
-                           "D1Q3 launch");
+  if (!rc) rc = cuda_check(launch_d1q3_sums(descs_dev(c), L.d1_groups[0], c->ws, sc, pending, true, c->stream,
+                                            &launches), "D1Q3 launch");
   count_kernels(c, launches);
   return rc;
 }

@@ -10,8 +10,8 @@
 //                  populations go to memory
 //   k_d1q3_sample  row transforms of all samples (radix-2 passes of fft_common.cuh, two fields
 //                  packed per complex row) and their pair products
-//   k_d1q3_sums    adds the products to the replica's sums, sample by sample (on small batches blocks of
-//                  the next k_d1q3_steps do it)
+//   k_d1q3_sums    adds the products to the replica's sums, sample by sample (k_d1q3_sums_many on large
+//                  batches; on small ones blocks of the next k_d1q3_steps do it while there is one)
 // Every sum takes the samples' products one at a time in the order of the steps, as the per-step
 // launches add them, so it does not depend on how runs are cut into calls and chunks or on the other
 // replicas of the context.
@@ -85,7 +85,7 @@ __device__ __forceinline__ double* d1_sum(const ReplicaDesc& d, char* __restrict
 }
 
 // The ns samples' products added to a replica's sums, a thread per product, by block `part` of `parts`:
-// beside steps, so a few loads ahead in registers do (58 ns a sample).
+// beside steps, or in many blocks, so a few loads ahead in registers do (58 ns a sample).
 __device__ __forceinline__ void d1q3_add_products(const ReplicaDesc& d, char* __restrict__ ws, const D1Scratch& sc,
                                                   uint32_t ns, int part, int parts) {
   if (!d.n_fields) return;
@@ -249,10 +249,17 @@ k_d1q3_sample(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, cons
   }
 }
 
-// The same as a kernel.  The time of a small batch is a thread's chain of dependent additions, 31 ns each
-// at best: their products come by asynchronous copies up to 64 samples ahead into slots of the thread's
-// own.  About 43 ns a sample (loads into registers 8 ahead 58, 32 ahead 50).
+// The same for large batches, whose warps hide each other's loads.
 constexpr int kD1SumThreads = 64, kD1SumBatch = 32, kD1SumStages = 3;
+__global__ void __launch_bounds__(kD1SumThreads)
+k_d1q3_sums_many(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t ns) {
+  d1q3_add_products(descs[blockIdx.x], ws, sc, ns, (int)blockIdx.y, (int)gridDim.y);
+}
+
+// The same for the last chunk of a small batch, where the time is a thread's chain of dependent additions,
+// 31 ns each at best: their products come by asynchronous copies up to 64 samples ahead into slots of the
+// thread's own.  About 43 ns a sample (loads into registers 8 ahead 58, 32 ahead 50); its shared memory
+// leaves an SM 8 warps, so that batches of 2000 x 1024 sites, four fields, would take 861 us a step for 730.
 __global__ void __launch_bounds__(kD1SumThreads)
 k_d1q3_sums(const ReplicaDesc* __restrict__ descs, char* __restrict__ ws, const D1Scratch sc, uint32_t ns) {
   __shared__ double ring[kD1SumStages][kD1SumBatch][kD1SumThreads];
@@ -303,12 +310,13 @@ cudaError_t set_d1q3_runs_smem() {
   return e;
 }
 
-// additions by themselves (a run's last chunk; every chunk of a large batch)
+// additions by themselves: a run's last chunk where d1q3_sums_beside, every chunk of a large batch
 cudaError_t launch_d1q3_sums(const ReplicaDesc* descs, const D1Group& g, char* ws, const D1Scratch& sc, uint32_t ns,
-                             cudaStream_t st, int* launches) {
+                             bool beside, cudaStream_t st, int* launches) {
   if (!ns) return cudaSuccess;
-  k_d1q3_sums<<<dim3(g.n, (unsigned)((g.max_products + kD1SumThreads - 1) / kD1SumThreads)), kD1SumThreads, 0, st>>>(
-      descs + g.first, ws, sc, ns);
+  const dim3 grid(g.n, (unsigned)((g.max_products + kD1SumThreads - 1) / kD1SumThreads));
+  if (beside) k_d1q3_sums<<<grid, kD1SumThreads, 0, st>>>(descs + g.first, ws, sc, ns);
+  else k_d1q3_sums_many<<<grid, kD1SumThreads, 0, st>>>(descs + g.first, ws, sc, ns);
   const cudaError_t e = cudaGetLastError();
   if (!e) ++*launches;
   return e;
@@ -358,7 +366,7 @@ cudaError_t launch_d1q3_chunk(const ReplicaDesc* descs, const D1Group& g, char* 
   k_d1q3_sample<<<dim3(g.n, blocks), kD1SampleThreads, g.sample_smem, st>>>(descs, ws, sc, ns);
   if ((e = cudaGetLastError())) return e;
   ++*launches;
-  if (!beside) return launch_d1q3_sums(descs - g.first, g, ws, sc, ns, st, launches);
+  if (!beside) return launch_d1q3_sums(descs - g.first, g, ws, sc, ns, false, st, launches);
   *pending = ns;
   return cudaSuccess;
 }
