@@ -33,11 +33,12 @@ size_t mlp_weights_bytes();
 void launch_set_step(uint64_t* s, uint64_t v, cudaStream_t st);
 void launch_advance_step(uint64_t* s, uint64_t n, cudaStream_t st);
 void launch_twiddles(int precision, void* tw, int n, cudaStream_t st);
-int fft_rows_smem(int precision, int nx);
+int fft_rows_smem(int precision, int nx, int most);
 int fft_cols_smem(int precision, int F, int ny, int ncol);
 cudaError_t set_fft_smem_limits();
 void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms);
+                     int64_t n_vblocks, char* ws, int grid, int smem, int most, cudaStream_t st, int slot, int paths,
+                     int sms);
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
                      int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split);
@@ -160,6 +161,7 @@ struct Layout {
   bool any_fused = true;      // some sampled replica's columns go through the fused pass
   int t_paths = 0, t_len = 1; // split: lengths among the one-pass replicas, the longest of the shared-memory kernel's
   int rows_paths = 0;                     // row-pass kernels (launch_fft_rows)
+  int rows_most = kRowsPairs;             // row pairs in a block of the shared-memory kernel, at most
   int fold = 1;               // 2: two spectrum slots, two samples per accumulation pass
   int max_fields = 0;         // the most sampled fields of a replica with pair sums
   int max_len = 1;            // the longest column transform
@@ -216,7 +218,7 @@ static int validate(int precision, const flb_replica* reps, int n) {
         return set_error(FLB_EINVAL, "replica %d: sampling needs nx, ny, nz <= 4096", r);
     } else if (p.field_mask) {
       if (!is_pow2(p.nx) || !is_pow2(p.ny)) return set_error(FLB_EINVAL, "replica %d: sampling needs power-of-two nx, ny", r);
-      if (fft_rows_smem(precision, p.nx) > 227 * 1024) return set_error(FLB_EINVAL, "replica %d: nx too large for the row FFT", r);
+      if (fft_rows_smem(precision, p.nx, kRowsPairs) > 227 * 1024) return set_error(FLB_EINVAL, "replica %d: nx too large for the row FFT", r);
       const int F = __builtin_popcount(p.field_mask);
       const int l1 = column_split(precision, F, p.ny);
       const int len = std::max(1 << l1, p.ny >> l1);
@@ -576,9 +578,17 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
   L.vb_t.resize(n); L.vb_pts.resize(n);
   L.vb_step.resize(n); L.vb_rows.resize(n); L.vb_cols.resize(n); L.vb_cols_a.resize(n);
   if (maxF) {
+    auto blocks = [&](int most) {
+      int64_t n_blocks = 0;
+      for (const ReplicaDesc& d : L.desc)
+        if (d.n_pairs && !rows16(precision, d.nx)) n_blocks += rows_blocks(precision, d.nx, (int)d.n_fields, d.ny, most);
+      return n_blocks;
+    };
+    while (L.rows_most > 1 && blocks(L.rows_most) < kRowsMinBlocks) L.rows_most >>= 1;
     // the shared-memory row kernel's launch (replicas the Stockham kernel does not take)
     for (const ReplicaDesc& d : L.desc)
-      if (d.n_pairs && !rows16(precision, d.nx)) L.rows_smem = std::max(L.rows_smem, fft_rows_smem(precision, d.nx));
+      if (d.n_pairs && !rows16(precision, d.nx))
+        L.rows_smem = std::max(L.rows_smem, fft_rows_smem(precision, d.nx, L.rows_most));
     L.cols_smem = fft_cols_smem(precision, maxF, maxlen, L.ncol);
   }
   plan_step(lat, L.vec, 0, L);
@@ -595,7 +605,7 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
     }
     if (d.n_pairs) {
       const int64_t tiles = (d.half_nx + L.ncol - 1) / L.ncol;
-      L.n_vb_rows += rows_blocks(precision, d.nx, (int)d.n_fields, d.ny);
+      L.n_vb_rows += rows_blocks(precision, d.nx, (int)d.n_fields, d.ny, L.rows_most);
       L.n_vb_cols += tiles << d.log2n1;                       // (k1, tile)
       L.n_vb_cols_a += cols_a_blocks(precision, d.log2n1, (int)d.n_fields, d.half_nx, d.ny, L.ncol);
     }
@@ -1103,7 +1113,7 @@ static void issue_step(flb_ctx* c, StepLaunch& S, bool sample, cudaStream_t st) 
     const int rows_grid = (int)std::min<int64_t>(L.n_vb_rows, (int64_t)c->sms * 8);
     const int cols_a_grid = (int)std::min<int64_t>(L.n_vb_cols_a, (int64_t)c->sms * 8);
     launch_fft_rows(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_rows), c->n,
-                    L.n_vb_rows, c->ws, rows_grid, L.rows_smem, st, slot, L.rows_paths, c->sms);
+                    L.n_vb_rows, c->ws, rows_grid, L.rows_smem, L.rows_most, st, slot, L.rows_paths, c->sms);
     if (L.n_vb_cols_a)
       launch_fft_cols_a(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_cols_a), c->n,
                         L.n_vb_cols_a, c->ws, L.ncol, cols_a_grid, kColsBlock, L.cols_smem, st,

@@ -319,13 +319,20 @@ __host__ __device__ __forceinline__ bool rows16_nx(int nx) {
   return nx >= 4096 && nx <= 32768 && (nx & (nx - 1)) == 0;
 }
 inline bool rows16(int precision, int nx) { return precision != FLB_FP64 && rows16_nx(nx); }
-// (the shared-memory pass: pairs of rows, 2048 points and at most 8 pairs per block, sequences
-// with 32 pad slots an odd number of elements apart)
-__host__ __device__ __forceinline__ int rows_per_block(int nx) { return nx >= 2048 ? 1 : (nx <= 256 ? 8 : 2048 / nx); }
+// (the shared-memory pass: pairs of rows per block, 2048 points and kRowsPairs pairs at most, sequences
+// with 32 pad slots an odd number of elements apart.  A launch of few rows takes fewer, `most`, until it
+// has kRowsMinBlocks blocks, but 256 points or more: 12 pairs of 1024 points in FP64 took 33 us two to a
+// block, 19 one to a block)
+constexpr int kRowsPairs = 8;
+constexpr int64_t kRowsMinBlocks = 128;
+__host__ __device__ __forceinline__ int rows_per_block(int nx, int most) {
+  const int p = nx >= 2048 ? 1 : (nx <= 2048 / kRowsPairs ? kRowsPairs : 2048 / nx), few = 256 / nx;
+  return p < most ? p : (few < most ? most : (few < p ? few : p));
+}
 __host__ __device__ __forceinline__ int rows_seq_stride(int nx) { return nx + 33; }
-inline int64_t rows_blocks(int precision, int nx, int n_fields, int ny) {
+inline int64_t rows_blocks(int precision, int nx, int n_fields, int ny, int most) {
   if (rows16(precision, nx)) return (int64_t)n_fields * ny;
-  const int64_t pairs = ((int64_t)n_fields * ny + 1) / 2, p = rows_per_block(nx);
+  const int64_t pairs = ((int64_t)n_fields * ny + 1) / 2, p = rows_per_block(nx, most);
   return (pairs + p - 1) / p;
 }
 // How a launch of the accumulation pass (pass 2b) cuts the layout's tiles of ncol columns:

@@ -18,7 +18,7 @@
 
 namespace flb {
 
-// Pass 1: one block per (replica, group of rows_per_block(nx) packed pairs of row units).
+// Pass 1: one block per (replica, group of rows_per_block(nx, most) packed pairs of row units).
 //
 // Each pass of the transform is a few dozen instructions between two barriers, so what
 // bounds it is how many rows an SM works on at a time.  With one pair per block of nx / 2
@@ -29,7 +29,7 @@ namespace flb {
 template <typename R>
 __global__ void __launch_bounds__(kRowsBlock, sizeof(R) == 4 ? 4 : 2)
 k_fft_rows(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin,
-                           int n_reps, int64_t n_vblocks, char* __restrict__ ws, int slot) {
+                           int n_reps, int64_t n_vblocks, char* __restrict__ ws, int slot, int most) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C<R>* z = reinterpret_cast<C<R>*>(smem_raw);
   const int tid = (int)threadIdx.x, nt = (int)blockDim.x;
@@ -41,7 +41,7 @@ k_fft_rows(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb
     // power of two), so an odd field count leaves at most one half-empty transform
     const int nx = d.nx, logn = d.log2nx, hn = nx >> 1;
     const int64_t units = (int64_t)d.n_fields << d.log2ny, pairs = (units + 1) >> 1;
-    const int P = rows_per_block(nx);
+    const int P = rows_per_block(nx, most);
     const int64_t p0 = (vb - vb_begin[r]) * P;
     const int np = (int)min((int64_t)P, pairs - p0);           // this block's pairs, sequences of z
     const int ss = rows_seq_stride(nx);
@@ -54,10 +54,10 @@ k_fft_rows(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb
       const int64_t vbn = vb + gridDim.x;
       const int rn = find_rep(vb_begin, n_reps, vbn);
       const ReplicaDesc& dn = descs[rn];
-      const int64_t un = 2 * (vbn - vb_begin[rn]) * rows_per_block(dn.nx);
+      const int64_t un = 2 * (vbn - vb_begin[rn]) * rows_per_block(dn.nx, most);
       const int64_t left = ((int64_t)dn.n_fields << dn.log2ny) - un;
       const R* fn = reinterpret_cast<const R*>(ws + dn.off_fields) + un * dn.nx;
-      const int64_t bytes = min((int64_t)2 * rows_per_block(dn.nx), left) * dn.nx * (int64_t)sizeof(R);
+      const int64_t bytes = min((int64_t)2 * rows_per_block(dn.nx, most), left) * dn.nx * (int64_t)sizeof(R);
       if (left > 0 && bytes % 16 == 0 && (reinterpret_cast<uintptr_t>(fn) & 15) == 0)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(fn), "r"((uint32_t)bytes) : "memory");
     }
@@ -484,9 +484,9 @@ void launch_twiddles(int precision, void* tw, int n, cudaStream_t st) {
 
 // shared memory of the row pass for rows of nx: k_fft_rows16 holds nx / 2 complex values
 // (one pad slot per 16), k_fft_rows its group of rows
-int fft_rows_smem(int precision, int nx) {
+int fft_rows_smem(int precision, int nx, int most) {
   if (rows16(precision, nx)) return (nx / 2 + nx / 32) * 8;
-  return rows_per_block(nx) * rows_seq_stride(nx) * (precision == FLB_FP64 ? 16 : 8);
+  return rows_per_block(nx, most) * rows_seq_stride(nx) * (precision == FLB_FP64 ? 16 : 8);
 }
 // the columns of every field of a tile, plus a table of up to 256 roots of unity
 // (the register-resident passes of spectra_cols.cu)
@@ -517,13 +517,14 @@ cudaError_t set_fft_smem_limits() {
 // grid: blocks of the shared-memory kernel; the Stockham kernel takes at most two blocks
 // per SM of the sms SMs (its blocks loop over their rows)
 void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms) {
+                     int64_t n_vblocks, char* ws, int grid, int smem, int most, cudaStream_t st, int slot, int paths,
+                     int sms) {
   const int block = kRowsBlock;
   if (precision == FLB_FP64) {
-    k_fft_rows<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
+    k_fft_rows<double><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot, most);
     return;
   }
-  if (paths & kColsGeneric) k_fft_rows<float><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
+  if (paths & kColsGeneric) k_fft_rows<float><<<grid, block, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot, most);
   const int g16 = (int)std::min<int64_t>((int64_t)grid, 2 * (int64_t)sms);
   for (int b = 0; b < 4; ++b)
     if (paths & (1 << b)) launch_fft_rows16(descs, vb_begin, n_reps, n_vblocks, ws, g16, 4096 << b, st, slot);

@@ -10,11 +10,12 @@
 
 namespace flb {
 
-int fft_rows_smem(int precision, int nx);
+int fft_rows_smem(int precision, int nx, int most);
 int fft_cols_smem(int precision, int F, int ny, int ncol);
 cudaError_t set_fft_smem_limits();
 void launch_fft_rows(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
-                     int64_t n_vblocks, char* ws, int grid, int smem, cudaStream_t st, int slot, int paths, int sms);
+                     int64_t n_vblocks, char* ws, int grid, int smem, int most, cudaStream_t st, int slot, int paths,
+                     int sms);
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
                      int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split);
@@ -34,7 +35,7 @@ int spectra_plan(int precision, int nx, int ny, int F, SpectraPlan& P) {
   if (F < 1 || F > kMaxFields) return set_error(FLB_EINVAL, "n_fields must be in 1..%d", kMaxFields);
   auto pow2 = [](int v) { return v > 0 && (v & (v - 1)) == 0; };
   if (!pow2(nx) || !pow2(ny) || nx < 2) return set_error(FLB_EINVAL, "nx, ny must be powers of two, nx >= 2");
-  if (fft_rows_smem(precision, nx) > 227 * 1024) return set_error(FLB_EINVAL, "nx = %d too long for the row FFT", nx);
+  if (fft_rows_smem(precision, nx, kRowsPairs) > 227 * 1024) return set_error(FLB_EINVAL, "nx = %d too long for the row FFT", nx);
   const int l1 = column_split(precision, F, ny);
   int ly = 0;
   while ((1 << ly) < ny) ++ly;
@@ -58,10 +59,12 @@ int spectra_plan(int precision, int nx, int ny, int F, SpectraPlan& P) {
   d.log2n1 = l1;
   P.ncol = kColsMax;
   while (P.ncol > 1 && fft_cols_smem(precision, F, len, P.ncol) > kColsSmemBudget) P.ncol >>= 1;
-  P.rows_smem = fft_rows_smem(precision, nx);
+  P.rows_most = kRowsPairs;
+  while (P.rows_most > 1 && rows_blocks(precision, nx, F, ny, P.rows_most) < kRowsMinBlocks) P.rows_most >>= 1;
+  P.rows_smem = fft_rows_smem(precision, nx, P.rows_most);
   P.cols_smem = fft_cols_smem(precision, F, len, P.ncol);
   const int64_t tiles = (d.half_nx + P.ncol - 1) / P.ncol;
-  P.n_vb_rows = rows_blocks(precision, nx, F, ny);
+  P.n_vb_rows = rows_blocks(precision, nx, F, ny, P.rows_most);
   P.n_vb_cols = tiles << l1;
   P.n_vb_cols_a = cols_a_blocks(precision, l1, F, d.half_nx, ny, P.ncol);
   int64_t off = 0;
@@ -127,7 +130,7 @@ int spectra_launch(int precision, SpectraPlan& P, char* scratch, const void* fie
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int gr = (int)std::min<int64_t>(P.n_vb_rows, (int64_t)sms * 8);
-  launch_fft_rows(precision, ddesc, vb, 1, P.n_vb_rows, scratch, gr, P.rows_smem, st, 0,
+  launch_fft_rows(precision, ddesc, vb, 1, P.n_vb_rows, scratch, gr, P.rows_smem, P.rows_most, st, 0,
                   rows16(precision, d.nx) ? 1 << (d.log2nx - 12) : kColsGeneric, sms);
   if (P.n_vb_cols_a) {
     const int ga = (int)std::min<int64_t>(P.n_vb_cols_a, (int64_t)sms * 8);

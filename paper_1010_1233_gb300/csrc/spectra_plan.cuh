@@ -8,7 +8,7 @@ namespace flb {
 struct SpectraPlan {
   ReplicaDesc desc;
   int64_t n_vb_rows, n_vb_cols, n_vb_cols_a;
-  int ncol, rows_smem, cols_smem;
+  int ncol, rows_smem, rows_most, cols_smem;
   int64_t off_desc, off_vb, off_tw_x, off_tw_y, off_spec;   // byte offsets in the scratch
   size_t scratch_bytes;
   int64_t n_sum_doubles;                                    // length of the pair-sum output
