@@ -590,7 +590,7 @@ void launch_pair_sums(int precision, const ReplicaDesc* descs, const int64_t* vb
 void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
                      int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split) {
-  const ColsSplit sp = cols_split(precision, n_vblocks, ncol, max_pairs, sms);
+  const ColsSplit sp = cols_split(precision, n_vblocks, ncol, max_fields * max_len, max_pairs, sms);
   if (precision == FLB_FP64 || (paths & kColsGeneric)) {    // one slot (the host folds samples only without it)
     const int smem = fft_cols_smem(precision, max_fields, max_len, sp.w);
     const int64_t nb = n_vblocks * (ncol / sp.w) * sp.ps;
