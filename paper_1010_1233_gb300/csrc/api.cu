@@ -43,7 +43,7 @@ void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
                      int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split);
 int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
-                      char* ws, cudaStream_t st, int paths, int slot, int max_len, int sms);
+                      char* ws, cudaStream_t st, int paths, int slot, int smem, int sms);
 void launch_pair_sums(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
                       char* ws, int ncol, int max_fields, int nslots, cudaStream_t st, const TimeCorr& tc, int sms);
 void launch_time_corr(const ReplicaDesc* descs, int n_reps, int max_fields, const TimeCorr& tc, cudaStream_t st);
@@ -159,7 +159,7 @@ struct Layout {
   int cols_a_paths = 0, cols_paths = 0;   // column-pass kernels the replicas need (cols16_b)
   bool split = false;         // one-pass replicas: transforms and pair sums apart (spectra.cu)
   bool any_fused = true;      // some sampled replica's columns go through the fused pass
-  int t_paths = 0, t_len = 1; // split: lengths among the one-pass replicas, the longest of the shared-memory kernel's
+  int t_paths = 0, t_smem = 0; // split: lengths among the one-pass replicas, the shared-memory kernel's bytes
   int rows_paths = 0;                     // row-pass kernels (launch_fft_rows)
   int rows_most = kRowsPairs;             // row pairs in a block of the shared-memory kernel, at most
   int fold = 1;               // 2: two spectrum slots, two samples per accumulation pass
@@ -570,7 +570,7 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
         L.cols_paths |= b ? b : kColsGeneric;
       } else {
         L.t_paths |= b ? b : kColsGeneric;
-        if (!b) L.t_len = std::max(L.t_len, (int)d.ny);
+        if (!b) L.t_smem = std::max(L.t_smem, cols_t_smem(precision, d));
       }
     }
   }
@@ -600,7 +600,7 @@ static int plan(int precision, const flb_replica* reps, int n, Layout& L) {
     L.vb_t[r] = L.n_vb_t;
     L.vb_pts[r] = L.n_vb_pts;
     if (d.n_pairs && L.split && !d.log2n1) {
-      L.n_vb_t += cols_t_blocks(d);
+      L.n_vb_t += cols_t_blocks(precision, d);
       L.n_vb_pts += pair_blocks(d, L.ncol);
     }
     if (d.n_pairs) {
@@ -1122,7 +1122,7 @@ static void issue_step(flb_ctx* c, StepLaunch& S, bool sample, cudaStream_t st) 
                          (L.n_vb_cols_a ? path_launches(c->precision, L.cols_a_paths) : 0));
     if (L.split)
       count_kernels(c, launch_fft_cols_t(c->precision, S.descs, reinterpret_cast<const int64_t*>(c->ws + L.off_vb_t),
-                                         c->n, L.n_vb_t, c->ws, st, L.t_paths, slot, L.t_len, c->sms));
+                                         c->n, L.n_vb_t, c->ws, st, L.t_paths, slot, L.t_smem, c->sms));
     c->pending = slot + 1;
     if (!fold || c->pending == 2) flush_samples(c, S, st);
   }

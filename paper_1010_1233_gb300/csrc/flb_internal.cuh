@@ -370,7 +370,23 @@ inline ColsSplit cols_split(int precision, int64_t n_tiles, int ncol, int col_po
 // of a launch (64^2, 3 fields, is 2112: one fused launch of 11 us against two of 5).
 constexpr int kColsT = 4;
 constexpr int64_t kSplitPoints = 8192;
-inline int64_t cols_t_blocks(const ReplicaDesc& d) { return (int64_t)d.n_fields * ((d.half_nx + kColsT - 1) / kColsT); }
+// the shared-memory kernel's tiles: kColsT columns, more of short columns (kColsTPoints points a block: with 32
+// points, four columns of 8, 9 x 8 x 8192 in FP64 took 145 us, 1024 points 13)
+constexpr int kColsTPoints = 1024;
+__host__ __device__ __forceinline__ int cols_t_log2(int ny, int half_nx) {
+  int lw = 2;
+  while ((ny << lw) < kColsTPoints && (1 << lw) < half_nx) ++lw;
+  return lw;
+}
+static_assert(kColsT == 4, "the narrowest tile");
+inline int64_t cols_t_blocks(int precision, const ReplicaDesc& d) {
+  const int lw = precision != FLB_FP64 && cols16_b(d.ny) ? 2 : cols_t_log2(d.ny, d.half_nx);
+  return (int64_t)d.n_fields * ((d.half_nx + (1 << lw) - 1) >> lw);
+}
+// shared memory of the shared-memory kernel for columns of ny
+inline int cols_t_smem(int precision, const ReplicaDesc& d) {
+  return (d.ny + 1) * (precision == FLB_FP64 ? 16 : 8) << cols_t_log2(d.ny, d.half_nx);
+}
 inline int64_t pair_blocks(const ReplicaDesc& d, int ncol) {
   const int64_t pts = d.acc_ncol ? (int64_t)d.ny * ((d.half_nx + ncol - 1) / ncol) * ncol : (int64_t)d.ny * d.half_nx;
   return (pts + kColsBlock - 1) / kColsBlock;

@@ -269,20 +269,18 @@ k_fft_cols_acc(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict_
 // the 64-replica sweep 286 -> 231, 3 x 1024 x 2048 96 -> 73; whole runs: 256^2 with 9 fields FP32, 2000
 // steps with 200 samples, 11.5 -> 10.5 ms.
 
-// One block per (replica, field, tile of kColsT columns): the columns transformed over y in place.
+// One block per (replica, field, tile of columns, cols_t_log2): the columns transformed over y in place.
 template <typename R>
 __global__ void __launch_bounds__(kColsBlock, sizeof(R) == 4 ? 4 : 2)
 k_fft_cols_t(const ReplicaDesc* __restrict__ descs, const int64_t* __restrict__ vb_begin, int n_reps,
              int64_t n_vblocks, char* __restrict__ ws, int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C<R>* s = reinterpret_cast<C<R>*>(smem_raw);
-  constexpr int w = kColsT, lw = 2;
-  static_assert(1 << lw == w, "log2 of the tile width");
   for (int64_t vb = blockIdx.x; vb < n_vblocks; vb += gridDim.x) {
     const int r = find_rep(vb_begin, n_reps, vb);
     const ReplicaDesc& d = descs[r];
     if (d.log2n1 || (sizeof(R) == 4 && cols16_b(d.ny))) continue;      // another kernel's replica
-    const int tiles = (d.half_nx + w - 1) >> lw;
+    const int lw = cols_t_log2(d.ny, d.half_nx), w = 1 << lw, tiles = (d.half_nx + w - 1) >> lw;
     const int local = (int)(vb - vb_begin[r]), f = local / tiles;
     const int kx0 = (local - f * tiles) << lw, ncl = min(w, d.half_nx - kx0);
     const int logn = d.log2ny, n = d.ny, total = n << lw;
@@ -552,13 +550,12 @@ void launch_fft_cols_t16(int mask, const ReplicaDesc* descs, const int64_t* vb_b
                          char* ws, int grid, cudaStream_t st, int slot);
 
 // Column transforms in place of the one-pass replicas (paths: the lengths among them, as in
-// launch_fft_cols; max_len: the longest of the shared-memory kernel's); returns the launches.
+// launch_fft_cols; smem: of the shared-memory kernel, cols_t_smem); returns the launches.
 int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
-                      char* ws, cudaStream_t st, int paths, int slot, int max_len, int sms) {
+                      char* ws, cudaStream_t st, int paths, int slot, int smem, int sms) {
   const int grid = (int)std::min<int64_t>(n_vblocks, 16 * (int64_t)sms);
   int launches = 0;
   if (precision == FLB_FP64 || (paths & kColsGeneric)) {
-    const int smem = kColsT * (max_len + 1) * (precision == FLB_FP64 ? 16 : 8);
     if (precision == FLB_FP64)
       k_fft_cols_t<double><<<grid, kColsBlock, smem, st>>>(descs, vb_begin, n_reps, n_vblocks, ws, slot);
     else

@@ -20,7 +20,7 @@ void launch_fft_cols(int precision, const ReplicaDesc* descs, const int64_t* vb_
                      int64_t n_vblocks, char* ws, int ncol, cudaStream_t st, const TimeCorr& tc, int paths,
                      int nslots, int max_fields, int max_len, int max_pairs, int sms, bool split);
 int launch_fft_cols_t(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
-                      char* ws, cudaStream_t st, int paths, int slot, int max_len, int sms);
+                      char* ws, cudaStream_t st, int paths, int slot, int smem, int sms);
 void launch_pair_sums(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps, int64_t n_vblocks,
                       char* ws, int ncol, int max_fields, int nslots, cudaStream_t st, const TimeCorr& tc, int sms);
 void launch_fft_cols_a(int precision, const ReplicaDesc* descs, const int64_t* vb_begin, int n_reps,
@@ -139,7 +139,7 @@ int spectra_launch(int precision, SpectraPlan& P, char* scratch, const void* fie
   }
   const int paths = precision != FLB_FP64 && cols16_b(d.ny >> d.log2n1) ? cols16_b(d.ny >> d.log2n1) : kColsGeneric;
   if (!d.log2n1 && (int64_t)d.ny * d.half_nx >= kSplitPoints) {
-    launch_fft_cols_t(precision, ddesc, vb + 2, 1, cols_t_blocks(d), scratch, st, paths, 0, d.ny, sms);
+    launch_fft_cols_t(precision, ddesc, vb + 2, 1, cols_t_blocks(precision, d), scratch, st, paths, 0, cols_t_smem(precision, d), sms);
     launch_pair_sums(precision, ddesc, vb + 2, 1, pair_blocks(d, P.ncol), scratch, P.ncol, (int)d.n_fields, 1, st,
                      TimeCorr{}, sms);
   } else {
