@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import mlp as omlp
 from paper_1010_1233_gb300 import learned, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -74,3 +75,21 @@ def test_cancelling_sums(pairs, B):
             assert abs(want) < 1e-6 * size
             tol = 2.0 ** -24 * abs(want) + (gamma * gamma + (2 * blocks + 16) * 2.0 ** -53) * size
             assert (np.abs(grad["W3"][c, h::3] - want) <= tol).all(), (c, h, grad["W3"][c, h::3], want, tol)
+
+
+@pytest.mark.parametrize("R,B", [(64, 3), (65, 3), (700, 2), (3000, 1)])
+def test_many_runs(R, B):
+    # the loss pass over several blocks from 65 runs on, against the FP64 oracle.  Tolerance: as for the
+    # gradient over the sample split (100 FP32 operations a sample, averaged over the sum's terms)
+    w = W.mlp_weights(R, out_scale=0.3)
+    X = np.stack([W.mlp_inputs(B, 10 + r) for r in range(R)]).astype(np.float32)
+    Sp, G = W.correlator_tables(R, 4, 5)
+    tr = learned.Trainer(X, learned.gram(Sp, G), 4, w)
+    loss, m, grad = tr.loss_and_grad()
+    w64 = {k: v.astype(np.float64) for k, v in w.items()}
+    L0, g0, _ = omlp.loss_grad(w64, X.astype(np.float64), Sp, G)
+    _, m0 = omlp.loss(w64, X.astype(np.float64), Sp, G)
+    assert abs(loss - L0) < 1e-5 * abs(L0)
+    assert np.abs(m - m0).max() < 1e-5
+    for k in w:
+        assert np.abs(grad[k] - g0[k]).max() < 1e-4 * np.abs(g0[k]).max() + 1e-9, k
